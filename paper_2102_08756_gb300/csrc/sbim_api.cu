@@ -5,8 +5,11 @@
 // on the device in FP64, allocates the history ring buffer and creates the
 // cuFFT plans.  sbim_step enqueues, on the handle's stream:
 //   (0) R2C FFT of u                      (cuFFT)
-//   (1) rotate + ring write + convolution  conv_kernel
-//   (2) chunk reduction + assembly         assemble_kernel
+//   (1) history convolution: the sums of the blocks of 16 steps that begin
+//       (ahead_kernel, float-class history), or rotation, ring write and the whole
+//       convolution (conv_kernel, conv_tma_kernel: double, and where the block
+//       sums do not fit)
+//   (2) the step's own lags and assembly   near_kernel, or assemble_kernel
 //   (3) C2R FFT of the traction spectra    (cuFFT)
 //   (4) traction epilogue                  epilogue_kernel
 // with no host synchronisation.
@@ -68,6 +71,8 @@ const char* fft_name(cufftResult r) {
 constexpr double kPi = 3.141592653589793238462643383279502884;
 constexpr int kProfRing = 512;
 constexpr int kProfEvents = 6;
+constexpr size_t kSpareBytes = 256ull << 20;
+constexpr int kAheadLags = sbim::kAhead;   // lags per chunk of the block sums: a multiple of this
 
 // 16-point Gauss-Legendre nodes and weights on [-1, 1] (Newton on P_16).
 void gauss_legendre16(double* x, double* w) {
@@ -110,6 +115,13 @@ struct sbim_ctx {
   bool halves = false;        // records may hold two |k| (half-record layout)
   int lags_per_cta = 0;       // 0: automatic
   size_t part_bytes = 0;
+  bool use_ahead = false;     // time-blocked convolution (sbim_ahead.cuh)
+  int ahead_lc = kAheadLags, ahead_chunks = 1;
+  float* d_ahead = nullptr;
+  size_t ahead_bytes = 0;
+  long long* d_stamp = nullptr;
+  size_t stamp_bytes = 0;
+  int config_id = 0;          // counts changes of chunking and window (part of the stamps)
   double tab_h = 0;
   long long tab_n = 0;
   size_t real_size = 4;
@@ -386,6 +398,89 @@ int alloc_partials(sbim_ctx& c) {
   return SBIM_OK;
 }
 
+// Lag chunks of the block sums.  One chunk is groups x 16 CTAs of 8 records (one
+// tile in 16 is due at a step), 3 CTAs per SM; a CTA takes ~70 ns per lag in a full
+// wave and ~25 lags' worth to fill its pipeline, and every chunk adds partial sums
+// that are written and read once (2 x 160 B per record and step).  The count that
+// minimises the sum of both keeps the last wave full on small grids and few chunks
+// on large ones (4 at 1024^2 x 4096).
+void choose_ahead(sbim_ctx& c, int sms) {
+  const int lags = std::max(1, c.n_cut - 1);
+  auto round16 = [](int x) { return (x + kAheadLags - 1) / kAheadLags * kAheadLags; };
+  if (c.lags_per_cta > 0) {
+    c.ahead_lc = round16(std::min(c.lags_per_cta, lags));
+  } else {
+    const double ctas = sbim::ahead_ctas(c.n_orb_pad);
+    double best = 0;
+    for (int S = 1; S <= std::min(32, round16(lags) / kAheadLags); ++S) {
+      const int lc = round16((lags + S - 1) / S);
+      const double waves = std::ceil(ctas * ((lags + lc - 1) / lc) / (3.0 * sms));
+      const double ns = waves * (lc + 25) * 70.0 + S * (double)c.n_orb_pad * 320.0 / 6000.0;
+      if (S == 1 || ns < best) {
+        best = ns;
+        c.ahead_lc = lc;
+      }
+    }
+  }
+  c.ahead_chunks = (lags + c.ahead_lc - 1) / c.ahead_lc;
+}
+
+size_t ahead_need(const sbim_ctx& c) {
+  return (size_t)c.ahead_chunks * c.n_orb_pad * sbim::kAhead * 4 * sbim::kFields * sizeof(float);
+}
+
+// Marks every block sum as not formed.
+int forget_ahead(sbim_ctx* c) {
+  if (c->d_stamp) CU(cudaMemsetAsync(c->d_stamp, 0xff, c->stamp_bytes, c->stream));
+  return SBIM_OK;
+}
+
+// Room for the block sums of the current chunking, leaving `spare` bytes of the
+// device free; false if there is none (the caller then convolves step by step).
+bool alloc_ahead(sbim_ctx& c, size_t spare) {
+  const size_t need = ahead_need(c);
+  const size_t sneed = (size_t)c.ahead_chunks * c.n_orb_pad / sbim::kAheadRec * sizeof(long long);
+  if (need <= c.ahead_bytes && sneed <= c.stamp_bytes) return forget_ahead(&c) == SBIM_OK;
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || need + sneed + spare > free_b) return false;
+  void *fresh = nullptr, *stamps = nullptr;
+  if (cudaMalloc(&fresh, need) != cudaSuccess || cudaMalloc(&stamps, sneed) != cudaSuccess) {
+    cudaGetLastError();
+    if (fresh) cudaFree(fresh);
+    return false;
+  }
+  if (c.d_ahead) {
+    cudaStreamSynchronize(c.stream);
+    cudaFree(c.d_ahead);
+    cudaFree(c.d_stamp);
+  }
+  c.d_ahead = (float*)fresh;
+  c.ahead_bytes = need;
+  c.d_stamp = (long long*)stamps;
+  c.stamp_bytes = sneed;
+  return forget_ahead(&c) == SBIM_OK;
+}
+
+// Launch, chunking and sums buffer for the current variant, tile and lags_per_cta.
+int configure_conv(sbim_ctx& c, size_t spare) {
+  ++c.config_id;
+  c.use_ahead = false;
+  int rc = choose_chunks(c);
+  if (rc != SBIM_OK) return rc;
+  if (c.prec != SBIM_FP64 && c.variant >= 1) {
+    int dev = 0, sms = 148;
+    CU(cudaGetDevice(&dev));
+    CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    choose_ahead(c, sms);
+    CU(sbim::launch_ahead(sbim::StepArgs{}, c.prec, 0, c.halves, nullptr));
+    if (alloc_ahead(c, spare)) {
+      c.use_ahead = true;
+      return SBIM_OK;
+    }
+  }
+  return alloc_partials(c);
+}
+
 void release(sbim_ctx* c) {
   if (!c) return;
   if (c->have_fwd) cufftDestroy(c->plan_fwd);
@@ -393,7 +488,7 @@ void release(sbim_ctx* c) {
   void* ptrs[] = {c->d_bin, c->d_dir, c->d_wout, c->d_dT, c->d_ustep, c->d_muq,
                   c->d_tab64, c->d_tab32, c->d_gl, c->d_hist, c->d_part, c->d_uhat,
                   c->d_fhat, c->d_s, c->d_step, c->d_err, c->d_io, c->d_lmax,
-                  c->d_tile_lmax, c->d_nonfinite, c->d_wts};
+                  c->d_tile_lmax, c->d_nonfinite, c->d_wts, c->d_ahead, c->d_stamp};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
@@ -477,9 +572,10 @@ int create_impl(sbim_ctx* c) {
   const size_t cplx = 2 * c->real_size;
   size_t free_b = 0, total_b = 0;
   CU(cudaMemGetInfo(&free_b, &total_b));
+  // (the partial sums of a step-by-step convolution: the least a handle needs)
   const size_t need = c->hist_bytes + part_bytes + 2 * 3 * (size_t)c->nbins * cplx +
                       4 * c->field_elems() * c->real_size + (size_t)c->tab_n * 48;
-  if (need + (256ull << 20) > free_b)
+  if (need + kSpareBytes > free_b)
     return fail(SBIM_ERR_OOM, "need %.2f GB of device memory, %.2f GB free",
                 need / 1e9, free_b / 1e9);
   // The FP64 path keeps its convolution weights (32 B per orbit and lag) when
@@ -499,14 +595,13 @@ int create_impl(sbim_ctx* c) {
   if (!dbl) CU(cudaMalloc(&c->d_tab32, (size_t)c->tab_n * 4 * sizeof(float)));
   CU(cudaMalloc(&c->d_gl, 32 * sizeof(double)));
   CU(cudaMalloc(&c->d_hist, c->hist_bytes));
-  c->d_part = nullptr;
-  if (alloc_partials(*c) != SBIM_OK) return SBIM_ERR_OOM;
   CU(cudaMalloc(&c->d_uhat, 3 * (size_t)c->nbins * cplx));
   CU(cudaMalloc(&c->d_fhat, 3 * (size_t)c->nbins * cplx));
   CU(cudaMalloc(&c->d_s, c->field_elems() * c->real_size));
   CU(cudaMalloc(&c->d_step, sizeof(long long)));
   CU(cudaMalloc(&c->d_err, sizeof(int)));
   if (c->wts_bytes) CU(cudaMalloc(&c->d_wts, c->wts_bytes));
+  if (const int rc = configure_conv(*c, kSpareBytes)) return rc == SBIM_ERR_CUDA ? rc : SBIM_ERR_OOM;
 
   cudaStream_t st = c->stream;
   CU(cudaMemcpyAsync(c->d_bin, h_bin.data(), h_bin.size() * sizeof(int), cudaMemcpyHostToDevice, st));
@@ -567,6 +662,11 @@ sbim::StepArgs step_args(const sbim_ctx* c) {
   a.step = c->d_step;
   a.err = c->d_err;
   a.part = c->d_part;
+  a.ahead = c->d_ahead;
+  a.stamp = c->d_stamp;
+  a.ahead_lc = c->ahead_lc;
+  a.ahead_chunks = c->ahead_chunks;
+  a.config_id = c->config_id & 0xffff;
   a.uhat = c->d_uhat;
   a.fhat = c->d_fhat;
   a.n_orb_pad = c->n_orb_pad;
@@ -626,6 +726,13 @@ int handle_epilogue(sbim_handle c, const void* v, void* tau, cudaStream_t st) {
 void handle_advance(sbim_handle c) {
   ++c->n;
   c->can_repeat = false;   // the batch kept its partial sums in its own buffers
+}
+
+bool handle_uses_ahead(sbim_handle c) { return c->use_ahead; }
+
+int handle_step_by_step(sbim_handle c) {
+  c->use_ahead = false;
+  return alloc_partials(*c);
 }
 
 int handle_shape(sbim_handle c, int* precision, int* kahan, int* variant, void** stream) {
@@ -749,14 +856,20 @@ int run_step(sbim_ctx* c, const void* in, const void* aux, void* out, bool adjoi
     CF(cufftExecR2C(c->plan_fwd, (cufftReal*)in, (cufftComplex*)c->d_uhat));
   if (e) CU(cudaEventRecord(e[1], st));
   const sbim::StepArgs a = step_args(c);
-  if (repeat)
+  if (c->use_ahead) {
+    // a repeated level finds its block sums formed: they end before the block
+    if (!repeat) CU(sbim::launch_ahead(a, c->prec, 1, c->halves, st));
+  } else if (repeat)
     CU(sbim::launch_repeat_lag0(a, c->prec, st));
   else if (c->variant >= 1)
     CU(sbim::launch_conv_tma(a, c->prec, c->kahan, c->variant, st, nullptr, c->tile, c->halves));
   else
     CU(sbim::launch_conv(a, c->prec, c->kahan, st));
   if (e) CU(cudaEventRecord(e[2], st));
-  CU(sbim::launch_assemble(a, c->prec, c->kahan, st));
+  if (c->use_ahead)
+    CU(sbim::launch_ahead(a, c->prec, 2, c->halves, st));
+  else
+    CU(sbim::launch_assemble(a, c->prec, c->kahan, st));
   if (e) CU(cudaEventRecord(e[3], st));
   void* s_dst = adjoint ? out : c->d_s;
   if (c->prec == SBIM_FP64)
@@ -843,10 +956,11 @@ int sbim_step_host(sbim_handle h, const void* u, const void* v, void* tau) {
   } else {
     // Every lag >= 1 of Eq. (SBI)'s convolution reads only the stored history,
     // so it runs while u and v cross to the device and are transformed on the
-    // side stream.  The convolution first sees zero spectra (its ring slot
-    // holds zeros, lag 0 adds nothing); the lag-0 pass then stores the new
+    // side stream.  The block sums never hold the current step; the
+    // step-by-step convolution first sees zero spectra (its ring slot
+    // holds zeros, lag 0 adds nothing), and the lag-0 pass then stores the new
     // spectra and adds w(0) D_n to chunk 0's partial sums, as sbim_step_repeat
-    // does.  Equal to sbim_step up to the order of that one addition.
+    // does: equal to sbim_step up to the order of that one addition.
     if (!c->io_stream) {
       CU(cudaStreamCreateWithFlags(&c->io_stream, cudaStreamNonBlocking));
       CU(cudaEventCreateWithFlags(&c->io_fork, cudaEventDisableTiming));
@@ -861,14 +975,20 @@ int sbim_step_host(sbim_handle h, const void* u, const void* v, void* tau) {
     CU(cudaEventRecord(c->io_join, c->io_stream));
     sbim::StepArgs a = step_args(c);
     a.uhat = zero_hat;
-    if (c->variant >= 1)
+    if (c->use_ahead)
+      CU(sbim::launch_ahead(a, c->prec, 1, c->halves, st));
+    else if (c->variant >= 1)
       CU(sbim::launch_conv_tma(a, c->prec, c->kahan, c->variant, st, nullptr, c->tile, c->halves));
     else
       CU(sbim::launch_conv(a, c->prec, c->kahan, st));
     CU(cudaStreamWaitEvent(st, c->io_join, 0));
     a.uhat = c->d_uhat;
-    CU(sbim::launch_repeat_lag0(a, c->prec, st));
-    CU(sbim::launch_assemble(a, c->prec, c->kahan, st));
+    if (c->use_ahead) {
+      CU(sbim::launch_ahead(a, c->prec, 2, c->halves, st));
+    } else {
+      CU(sbim::launch_repeat_lag0(a, c->prec, st));
+      CU(sbim::launch_assemble(a, c->prec, c->kahan, st));
+    }
     rc = sbim::handle_fft_inverse(c, st);
     if (rc != SBIM_OK) return rc;
     rc = sbim::handle_epilogue(c, dv, dtau, st);
@@ -887,6 +1007,7 @@ int sbim_set_window(sbim_handle h, double window) {
   if (!h) return fail(SBIM_ERR_ARG, "NULL handle");
   if (!(window >= 0)) return fail(SBIM_ERR_ARG, "window must be >= 0");
   h->can_repeat = false;
+  ++h->config_id;
   if (window == 0) {
     h->window = 0;
     return SBIM_OK;
@@ -945,6 +1066,8 @@ int sbim_set_conv_config(sbim_handle h, int variant, int lags_per_cta) {
   if (lags_per_cta < 0) return fail(SBIM_ERR_ARG, "lags_per_cta must be >= 0");
   h->can_repeat = false;
   const int old_v = h->variant, old_l = h->lags_per_cta, old_lc = h->lc, old_nc = h->nchunks;
+  const int old_alc = h->ahead_lc, old_anc = h->ahead_chunks;
+  const bool old_ahead = h->use_ahead;
   h->variant = variant;
   h->lags_per_cta = lags_per_cta;
   if (variant >= 1) {
@@ -955,10 +1078,10 @@ int sbim_set_conv_config(sbim_handle h, int variant, int lags_per_cta) {
       return fail(SBIM_ERR_CUDA, "kernel attributes: %s", cudaGetErrorString(e));
     }
   }
-  int rc = choose_chunks(*h);
-  if (rc == SBIM_OK) rc = alloc_partials(*h);
+  const int rc = configure_conv(*h, kSpareBytes);
   if (rc != SBIM_OK) {
     h->variant = old_v; h->lags_per_cta = old_l; h->lc = old_lc; h->nchunks = old_nc;
+    h->ahead_lc = old_alc; h->ahead_chunks = old_anc; h->use_ahead = old_ahead;
     return rc;
   }
   return SBIM_OK;
@@ -973,6 +1096,8 @@ int sbim_set_conv_tile(sbim_handle h, int orbits_per_cta) {
                 h->n_orb_pad, orbits_per_cta);
   h->can_repeat = false;
   const int old_t = h->tile, old_lc = h->lc, old_nc = h->nchunks;
+  const int old_alc = h->ahead_lc, old_anc = h->ahead_chunks;
+  const bool old_ahead = h->use_ahead;
   h->tile = orbits_per_cta;
   if (h->variant >= 1) {
     const cudaError_t e = sbim::prepare_conv_tma(h->prec, h->kahan, h->variant, h->tile, h->halves);
@@ -981,10 +1106,10 @@ int sbim_set_conv_tile(sbim_handle h, int orbits_per_cta) {
       return fail(SBIM_ERR_CUDA, "kernel attributes: %s", cudaGetErrorString(e));
     }
   }
-  int rc = choose_chunks(*h);
-  if (rc == SBIM_OK) rc = alloc_partials(*h);
+  const int rc = configure_conv(*h, kSpareBytes);
   if (rc != SBIM_OK) {
     h->tile = old_t; h->lc = old_lc; h->nchunks = old_nc;
+    h->ahead_lc = old_alc; h->ahead_chunks = old_anc; h->use_ahead = old_ahead;
     return rc;
   }
   return SBIM_OK;
@@ -999,6 +1124,7 @@ int sbim_set_far_field(sbim_handle h, const double tau_inf[3]) {
 int sbim_reset(sbim_handle h) {
   if (!h) return fail(SBIM_ERR_ARG, "NULL handle");
   CU(cudaMemsetAsync(h->d_step, 0, sizeof(long long), h->stream));
+  if (const int rc = forget_ahead(h)) return rc;
   h->n = 0;
   h->can_repeat = false;
   return SBIM_OK;
@@ -1085,6 +1211,7 @@ int sbim_load(sbim_handle h, const void* buf, size_t bytes) {
   CU(cudaMemcpyAsync(h->d_hist, (const char*)buf + sizeof(hd), h->hist_bytes,
                      cudaMemcpyHostToDevice, h->stream));
   CU(cudaMemcpyAsync(h->d_step, &hd.n, sizeof(long long), cudaMemcpyHostToDevice, h->stream));
+  if (const int rc = forget_ahead(h)) return rc;
   CU(cudaStreamSynchronize(h->stream));
   h->n = hd.n;
   h->can_repeat = false;

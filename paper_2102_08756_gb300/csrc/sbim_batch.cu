@@ -19,6 +19,7 @@ struct sbim_batch_ctx {
   int lags = 0;                  // lags per work item last configured
   bool halves = false;           // some member's records hold two |k|
   bool per_item = false;    // one CTA per work item instead of persistent CTAs
+  bool ahead = false;       // every member's convolution is blocked in time
   bool owns = true;
   cudaStream_t stream = nullptr;
   std::vector<sbim_handle> h;
@@ -115,7 +116,18 @@ int configure(sbim_batch_ctx* b, int shape, int lags) {
   }
   b->halves = false;
   for (int i = 0; i < b->nb; ++i) b->halves = b->halves || sbim::handle_step_args(b->h[i]).halves;
-  BCU(sbim::prepare_conv_tma(b->prec, b->kahan, shape, b->tile, b->halves));
+  // time-blocked where every member has room for its block sums
+  b->ahead = true;
+  for (sbim_handle x : b->h) b->ahead = b->ahead && sbim::handle_uses_ahead(x);
+  if (b->ahead) {
+    BCU(sbim::launch_ahead(sbim::StepArgs{}, b->prec, 0, b->halves, nullptr));
+  } else {
+    BCU(sbim::prepare_conv_tma(b->prec, b->kahan, shape, b->tile, b->halves));
+    for (sbim_handle x : b->h) {
+      const int rc = sbim::handle_step_by_step(x);
+      if (rc != SBIM_OK) return rc;
+    }
+  }
   b->shape = shape;
   b->lags = lags;
   std::vector<sbim::StepArgs> args(b->nb);
@@ -123,7 +135,8 @@ int configure(sbim_batch_ctx* b, int shape, int lags) {
   for (int i = 0; i < b->nb; ++i) {
     args[i] = sbim::handle_step_args(b->h[i]);
     tiles[i + 1] = tiles[i] + args[i].n_orb_pad / sbim::kOrbitTile;   // assembly tiles
-    items[i + 1] = items[i] + args[i].n_orb_pad / b->tile * args[i].nchunks;
+    items[i + 1] = items[i] + (b->ahead ? sbim::ahead_ctas(args[i].n_orb_pad) * args[i].ahead_chunks
+                                        : args[i].n_orb_pad / b->tile * args[i].nchunks);
   }
   b->total_items = items[b->nb];
   b->total_tiles = tiles[b->nb];
@@ -177,12 +190,7 @@ int setup(sbim_batch_ctx* b) {
 
 // Enqueue one step of every member (pointer arrays are host arrays of device pointers).
 int enqueue(sbim_batch_ctx* b, const void* const* u, const void* const* v, void* const* tau) {
-  int rc = fork(b);
-  for (int i = 0; i < b->nb && rc == SBIM_OK; ++i)
-    rc = sbim::handle_fft_forward(b->h[i], u[i], side_of(b, i));
-  if (rc == SBIM_OK) rc = join(b);
-  if (rc != SBIM_OK) return rc;
-  BCU(cudaMemsetAsync(b->d_counter, 0, sizeof(int), b->stream));
+  const sbim::StepArgs a0 = sbim::handle_step_args(b->h[0]);
   sbim::BatchLaunch bl;
   bl.args = b->d_args;
   bl.item_prefix = b->d_item_prefix;
@@ -190,10 +198,21 @@ int enqueue(sbim_batch_ctx* b, const void* const* u, const void* const* v, void*
   bl.nb = b->nb;
   bl.counter = b->d_counter;
   bl.ctas = b->ctas;
-  bl.items = b->per_item ? b->total_items : 0;
-  const sbim::StepArgs a0 = sbim::handle_step_args(b->h[0]);
-  BCU(sbim::launch_conv_tma(a0, b->prec, b->kahan, b->shape, b->stream, &bl, b->tile, b->halves));
-  BCU(sbim::launch_assemble_batch(bl, b->total_tiles, b->prec, b->kahan, b->stream));
+  bl.items = b->per_item || b->ahead ? b->total_items : 0;
+  int rc = fork(b);
+  // the block sums need only the stored histories: they run beside the transforms
+  if (rc == SBIM_OK && b->ahead) BCU(sbim::launch_ahead(a0, b->prec, 1, b->halves, b->stream, &bl));
+  for (int i = 0; i < b->nb && rc == SBIM_OK; ++i)
+    rc = sbim::handle_fft_forward(b->h[i], u[i], side_of(b, i));
+  if (rc == SBIM_OK) rc = join(b);
+  if (rc != SBIM_OK) return rc;
+  if (b->ahead) {
+    BCU(sbim::launch_ahead(a0, b->prec, 2, b->halves, b->stream, &bl, b->total_tiles));
+  } else {
+    BCU(cudaMemsetAsync(b->d_counter, 0, sizeof(int), b->stream));
+    BCU(sbim::launch_conv_tma(a0, b->prec, b->kahan, b->shape, b->stream, &bl, b->tile, b->halves));
+    BCU(sbim::launch_assemble_batch(bl, b->total_tiles, b->prec, b->kahan, b->stream));
+  }
   rc = fork(b);
   for (int i = 0; i < b->nb && rc == SBIM_OK; ++i) {
     rc = sbim::handle_fft_inverse(b->h[i], side_of(b, i));

@@ -29,6 +29,23 @@ cudaError_t launch_wait_selftest(int* err, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+cudaError_t ahead_f32(const StepArgs& a, int stage, bool halves, cudaStream_t st,
+                      const BatchLaunch* batch, int tiles);
+cudaError_t ahead_bf16x2(const StepArgs& a, int stage, bool halves, cudaStream_t st,
+                         const BatchLaunch* batch, int tiles);
+cudaError_t ahead_bf16(const StepArgs& a, int stage, bool halves, cudaStream_t st,
+                       const BatchLaunch* batch, int tiles);
+
+cudaError_t launch_ahead(const StepArgs& a, int precision, int stage, bool halves, cudaStream_t st,
+                         const BatchLaunch* batch, int tiles) {
+  switch (precision) {
+    case SBIM_FP32: return ahead_f32(a, stage, halves, st, batch, tiles);
+    case SBIM_BF16X2: return ahead_bf16x2(a, stage, halves, st, batch, tiles);
+    case SBIM_BF16: return ahead_bf16(a, stage, halves, st, batch, tiles);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 cudaError_t launch_conv_tma_f32(const StepArgs& a, int kahan, int shape, cudaStream_t st,
                                  const BatchLaunch* batch, bool prep, int tile, bool halves);
 cudaError_t launch_conv_tma_bf16x2(const StepArgs& a, int kahan, int shape, cudaStream_t st,

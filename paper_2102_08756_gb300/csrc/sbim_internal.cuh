@@ -30,6 +30,8 @@ constexpr int kMembers = 4;      // members per orbit
 constexpr int kFields = 10;      // real accumulators per member: 5 complex sums
 constexpr int kOrbitTile = 128;  // orbits per CTA of the assembly and of the default convolution
                                  // (the TMA convolution also runs 64 or 256: "modes per CTA")
+constexpr int kAhead = 16;       // steps per block of the time-blocked convolution
+constexpr int kAheadRec = 8;     // records per CTA of its block sums
 
 // Everything the per-step kernels read; device pointers unless noted.
 struct StepArgs {
@@ -50,6 +52,8 @@ struct StepArgs {
   long long* step;                 // device step counter n
   int* err;                        // device error word (bounded waits that gave up)
   void* part;                      // [nchunks][40][n_orb_pad] partial sums
+  float* ahead;                    // time-blocked sums: [ahead_chunks][tile][16 steps][10][128 records x 4]
+  long long* stamp;                // [ahead_chunks][tile][16] the block and configuration they belong to
   const void* uhat;                // [3][nbins] forward spectra
   void* fhat;                      // [3][nbins] output spectra (scaled 1/(n1 n3))
   // sizes (host values)
@@ -59,6 +63,9 @@ struct StepArgs {
   int n_cut;
   int lc;                          // lags per chunk
   int nchunks;
+  int ahead_lc;                    // lags per chunk of the time-blocked sums, a multiple of 16
+  int ahead_chunks;
+  int config_id;                   // 16 bits: chunking and window of these arguments
   int side;
   double eta;
   double inv_n;                    // 1 / (n1 n3)
@@ -76,6 +83,20 @@ struct BatchLaunch {
   int items;                // > 0: one CTA per item (this many), no persistent CTAs
 };
 
+// Groups of kAhead tiles: each step renews the block sums of one tile of a group.
+__host__ __device__ constexpr int ahead_groups(int n_orb_pad) {
+  return (n_orb_pad / kOrbitTile + kAhead - 1) / kAhead;
+}
+// CTAs of one lag chunk of the block sums.
+__host__ __device__ constexpr int ahead_ctas(int n_orb_pad) {
+  return ahead_groups(n_orb_pad) * (kOrbitTile / kAheadRec);
+}
+// Time-blocked convolution of float-class histories (sbim_ahead.cuh): stage 0
+// prepares the kernels, stage 1 forms the block sums that are due, stage 2 adds the
+// step's own lags, stores the current spectra and assembles the output spectra.
+// With `batch`, over its members (items and tiles as its prefix sums count them).
+cudaError_t launch_ahead(const StepArgs& a, int precision, int stage, bool halves, cudaStream_t st,
+                         const BatchLaunch* batch = nullptr, int tiles = 0);
 cudaError_t launch_conv(const StepArgs& a, int precision, int kahan, cudaStream_t s);
 cudaError_t launch_assemble_batch(const BatchLaunch& b, int total_tiles, int precision, int kahan,
                                   cudaStream_t s);
@@ -128,6 +149,8 @@ int handle_fft_forward(sbim_handle h, const void* u, cudaStream_t st);
 int handle_fft_inverse(sbim_handle h, cudaStream_t st);
 int handle_epilogue(sbim_handle h, const void* v, void* tau, cudaStream_t st);
 void handle_advance(sbim_handle h);
+bool handle_uses_ahead(sbim_handle h);
+int handle_step_by_step(sbim_handle h);   // leave the time-blocked convolution
 int handle_shape(sbim_handle h, int* precision, int* kahan, int* variant, void** stream);
 
 // Batch over existing handles (not owned); enqueue one step / advance the counters.

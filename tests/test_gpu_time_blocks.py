@@ -1,0 +1,115 @@
+"""The time-blocked convolution (block sums over 16 steps, staggered over the
+record tiles) against the FP64 handle, which convolves step by step: cutoffs
+around the block length, chunk edges, both record layouts, every float-class
+history; the state changes that make the block sums obsolete; and non-finite
+values, which must enter and leave the tractions at the same steps."""
+import numpy as np
+import pytest
+
+from paper_2102_08756_gb300.synth import separable_history
+from tests._errors import Worst, rel_l2
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+CS, CP, RHO = 3464.0, 6000.0, 2670.0
+# the bounds of the parity tests: float storage and transforms, bf16 storage
+TOL = {"fp32": 1e-5, "bf16x2": 1e-4, "bf16": 1e-2}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+def _pair(n1, n3, n_cut, precision, side=1):
+    from paper_2102_08756_gb300.sbim import SBIM
+    dx = 100.0
+    dt = 0.3 * dx / CP
+    make = lambda p, k: SBIM(n1, n3, n1 * dx, n3 * dx, CS, CP, RHO, dt, n_cut, side, p, k)  # noqa: E731
+    return make(precision, precision != "bf16"), make("fp64", False), dt
+
+
+def _fields(n1, n3, dt, steps, seed):
+    h = separable_history(n1, n3, n1 * 100.0, n3 * 100.0, steps, dt, CS, seed=seed, spectrum="k2")
+    return [(torch.from_numpy(h.u(m).astype(np.float32)).cuda(),
+             torch.from_numpy(h.v(m).astype(np.float32)).cuda()) for m in range(steps)]
+
+
+# whole records; half records; 18 tiles, so a full group of 16 and a ragged one
+@pytest.mark.parametrize("precision", ["fp32", "bf16x2", "bf16"])
+@pytest.mark.parametrize("grid", [(32, 32), (64, 6), (176, 96)])
+@pytest.mark.parametrize("n_cut,lags", [(1, 0), (2, 0), (15, 0), (16, 0), (17, 0), (31, 16), (33, 16),
+                                        (50, 20), (70, 0)])
+def test_block_sums_match_step_by_step(precision, grid, n_cut, lags):
+    n1, n3 = grid
+    g, ref, dt = _pair(n1, n3, n_cut, precision, side=-1)
+    if lags:
+        g.set_conv_config(2, lags)
+    err = Worst()
+    for u, v in _fields(n1, n3, dt, 90, seed=n1 + n_cut):
+        t = g.step(u, v).double().cpu().numpy()
+        r = ref.step(u.double(), v.double()).cpu().numpy()
+        err.update(rel_l2(t, r))
+    g.check()
+    assert err.value < TOL[precision], err
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+def test_changes_of_state_between_blocks(precision):
+    """Reset, a new window, another chunking, several rewinds and a checkpoint of
+    another handle, each in the middle of a block."""
+    n1, n3, n_cut = 48, 32, 40
+    g, ref, dt = _pair(n1, n3, n_cut, precision)
+    donor, donor64, _ = _pair(n1, n3, n_cut, precision)
+    f = _fields(n1, n3, dt, 60, seed=5)
+    fd = _fields(n1, n3, dt, 60, seed=6)
+    for u, v in fd[:29]:
+        donor.step(u, v)
+        donor64.step(u.double(), v.double())
+    err = Worst()
+
+    def steps(a, b):
+        for u, v in f[a:b]:
+            r = ref.step(u.double(), v.double()).cpu().numpy()
+            err.update(rel_l2(g.step(u, v).double().cpu().numpy(), r))
+
+    steps(0, 21)
+    for h in (g, ref):
+        h.set_window(5.0)
+    steps(21, 25)
+    for h in (g, ref):
+        h.set_window(0.0)
+    steps(25, 27)
+    g.set_conv_config(1, 16)
+    steps(27, 40)
+    for h in (g, ref):
+        for _ in range(9):
+            h.rewind()
+    steps(40, 55)
+    for h in (g, ref):
+        h.reset()
+    steps(3, 30)
+    g.load(donor.save())
+    ref.load(donor64.save())
+    steps(29, 50)
+    assert err.value < TOL[precision], err
+
+
+def test_non_finite_values_leave_with_their_last_lag():
+    n1, n3, n_cut = 24, 16, 21
+    g, ref, dt = _pair(n1, n3, n_cut, "fp32")
+    f = _fields(n1, n3, dt, 60, seed=8)
+    seen = 0
+    for m, (u, v) in enumerate(f):
+        if m == 9:
+            u = u.clone()
+            u[1, 3, 5] = float("nan")
+        t = torch.isfinite(g.step(u, v))
+        r = torch.isfinite(ref.step(u.double(), v.double()))
+        assert torch.equal(t, r), m
+        seen += int(not bool(r.all()))
+    assert seen == n_cut
