@@ -17,7 +17,7 @@
 // the same.  A tile's block is a function of n and T only, and every sum has a
 // fixed order, so a step's result does not depend on when its sums were formed: a
 // restored checkpoint, a rewound or repeated step and a replayed graph give the
-// same bits as the run they continue.  Each (chunk, tile, 8 records) carries a stamp
+// same bits as the run they continue.  Each (chunk, tile, 32 records) carries a stamp
 // of the block its sums belong to and of the arguments' chunking and window; sums
 // whose stamp is not the current one are formed again, all on the device, so that a
 // captured graph renews them as a direct step does.  sbim_reset and sbim_load, which
@@ -35,23 +35,33 @@ namespace ahead {
 
 using namespace dev;
 
-// Records per CTA: 8 records x 4 members x 5 complex sums = 160 threads, one
-// complex sum of one member per thread.  A thread keeps 16 outputs (running sum
-// and compensation, 64 registers) and a window of 16 weights, each held twice so
-// that one two-lane multiply-add takes (re, im) (32 registers).
-constexpr int kRec = kAheadRec, kSums = 5, kThreads = kRec * kMembers * kSums;
+// 32 records x 4 members x 5 complex sums per CTA, one complex sum of one member per
+// thread: 20 warps, one CTA per SM.  Warp k holds sum k / 4 of the records 8 (k % 4)
+// .. + 7, so each of the SM's four schedulers has five warps and the same work (CTAs
+// of 5 warps, 8 records, put two of them on the first scheduler each: 1.16 ms for
+// 1024^2 x 4096 against 1.05, folding every 64 lags).  A thread keeps 16 outputs (32 registers) and a window
+// of 16 weights, each held twice so that one two-lane multiply-add takes (re, im) (32
+// registers).
+constexpr int kRec = kAheadRec, kSums = 5, kThreads = kRec * kMembers * kSums, kWarps = kThreads / 32;
 constexpr int kSub = kOrbitTile / kRec;     // CTAs per 128-record tile
-constexpr int kStages = 4;                  // 16-lag stages of history in shared memory
-// one record's 16 weights of one kernel: 16 x 8 bytes, padded against bank conflicts
-constexpr int kWRow = kAhead * 8 + 16;
+// Lags per stage, and the 16-lag blocks that are chained before they are folded into
+// the running sums (every 32 lags: the error against 64 bits stays that of the
+// step-by-step sums, 5.44e-7 for 256^2 x 1024; 64 lags were 5 % faster at 5.46e-7).
+constexpr int kLags = kAheadLags, kFold = 2;
+template <bool HALVES> __host__ __device__ constexpr int stages() { return HALVES ? 4 : 5; }
 
 template <class S> __host__ __device__ constexpr int seg() { return kRec * S::kRecBytes; }
-template <class S> __host__ __device__ constexpr int stage_bytes() { return kAhead * 3 * S::kPlanes * seg<S>(); }
-template <bool HALVES> __host__ __device__ constexpr int wbuf_bytes() { return (HALVES ? 2 : 1) * 4 * kRec * kWRow; }
-template <class S, bool HALVES> __host__ __device__ constexpr int smem_bytes() {
-  return kStages * stage_bytes<S>() + 2 * wbuf_bytes<HALVES>();
+template <class S> __host__ __device__ constexpr int hist_bytes() { return kLags * 3 * S::kPlanes * seg<S>(); }
+// The weights of one lag: 32 records (x 2 halves) x (11, 22, 33, 12).
+template <bool HALVES> __host__ __device__ constexpr int wlag_bytes() { return (HALVES ? 2 : 1) * kRec * 16; }
+// A stage: 8 lags of history and the weights 16 lags further on.
+template <class S, bool HALVES> __host__ __device__ constexpr int stage_bytes() {
+  return hist_bytes<S>() + kLags * wlag_bytes<HALVES>();
 }
-
+constexpr int kSumBytes = kThreads * kAhead * 8;   // the running sums
+template <class S, bool HALVES> __host__ __device__ constexpr int smem_bytes() {
+  return stages<HALVES>() * stage_bytes<S, HALVES>() + kSumBytes;
+}
 __device__ __forceinline__ unsigned long long fma2r(unsigned long long a, unsigned long long b,
                                                     unsigned long long c) {
   unsigned long long d;
@@ -69,10 +79,24 @@ __device__ __forceinline__ unsigned long long sub2r(unsigned long long a, unsign
   return d;
 }
 
-// One member's value: in a staged segment (8 records), in the ring, and as stored.
+// Counts one up and returns the value before: releases what this thread did, and the
+// one that reads the last count sees what the others released.
+__device__ __forceinline__ int shared_inc(int* p) {
+  int r;
+  asm volatile("atom.acq_rel.cta.shared.add.s32 %0, [%1], 1;" : "=r"(r) : "r"(tma::smem_addr(p)) : "memory");
+  return r;
+}
+__device__ __forceinline__ void tile_g2s(unsigned dst, const void* map, int x, int y, unsigned bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3}], [%4];" ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
+}
+
+// One member's value: in a staged row (32 records; the lo plane `lo` bytes on), in
+// the ring, and as stored.
 template <class S> struct MemberIO;
 template <> struct MemberIO<StoreF32> {
-  __device__ static float2 smem(const unsigned char* p, int lane) {
+  __device__ static float2 smem(const unsigned char* p, int, int lane) {
     return *reinterpret_cast<const float2*>(p + lane * 8);
   }
   __device__ static float2 load(const void* h, long long i, long long) {
@@ -84,10 +108,10 @@ template <> struct MemberIO<StoreF32> {
   }
 };
 template <bool LO> struct MemberIO<StoreBF16<LO>> {
-  __device__ static float2 smem(const unsigned char* p, int lane) {
+  __device__ static float2 smem(const unsigned char* p, int lo, int lane) {
     float2 d = unpack_bf16(*reinterpret_cast<const unsigned*>(p + lane * 4));
     if (LO) {
-      const float2 l = unpack_bf16(*reinterpret_cast<const unsigned*>(p + kRec * 16 + lane * 4));
+      const float2 l = unpack_bf16(*reinterpret_cast<const unsigned*>(p + lo + lane * 4));
       d.x += l.x;
       d.y += l.y;
     }
@@ -125,6 +149,10 @@ template <bool LO> struct MemberIO<StoreBF16<LO>> {
 __device__ __forceinline__ long long block_base(long long n, int T) {
   return n - ((n + T) & (kAhead - 1));
 }
+// The stamp of sums formed for a block with these arguments' chunking and window.
+__device__ __forceinline__ long long block_mark(const StepArgs& a, long long base) {
+  return base * 65536 + a.config_id;
+}
 // Largest lag m of the block sums A[s] of tile T: the history before `base`, the
 // cutoff, and the tile's truncation window.
 __device__ __forceinline__ int last_lag(const StepArgs& a, long long base, int T) {
@@ -134,208 +162,278 @@ __device__ __forceinline__ int last_lag(const StepArgs& a, long long base, int T
   return m;
 }
 
-// Block sums of records 8 q .. 8 q + 7 of tile T over one chunk of lags.  Stages
-// of 16 lags arrive by bulk copies (3 components x 8 records each); the 16 weights
-// per record of the block after next are interpolated while a block is summed.
-// Per block of 16 lags and output the terms are chained by multiply-adds and every
-// 32 lags folded into the running sum with one compensated addition.
-// Returns false if a bounded wait gave up.
+// What one CTA sums at a time: records 32 q .. 32 q + 31 of tile T over the lags m0 ..
+// m1 of a chunk, in blocks of 16 lags.
+struct Item {
+  int T, rec0, m0, m1, nblk, chunk, bs;
+  long long base;
+  __device__ void set(const StepArgs& a, int T_, int q, int chunk_, long long n) {
+    T = T_;
+    chunk = chunk_;
+    base = block_base(n, T);
+    rec0 = T * kOrbitTile + q * kRec;
+    m0 = 1 + chunk * a.ahead_lc;
+    m1 = min(m0 + a.ahead_lc - 1, last_lag(a, base, T));
+    nblk = (m1 - m0 + kAhead) / kAhead;
+    bs = base < 0x7fffffff ? (int)base % a.n_cut : (int)(base % a.n_cut);
+  }
+};
+
+// Shared state of a CTA: copies landed per stage, warps that have left it, the stages
+// requested so far, and the item (kept here: a request needs it, the sums do not).
+struct Sync {
+  unsigned long long full[5];
+  int left[5];
+  unsigned requested;
+  Item it;
+};
+
+// Request stage j of an item, the CTA's g-th (one thread): the lags m0 + 8 j .. + 7 and
+// the weights 16 lags on.  The history of 8 lags is 24 rows of the ring (slot x
+// component, 32 records each) and arrives as one tiled copy per plane; only where the
+// 8 slots wrap around the ring, row by row.  (Copying every row by itself took the
+// issuing warp four times as many instructions as its sums: 1.96 against 1.42 ms for
+// 1024^2 x 4096.)
 template <class S, bool HALVES>
-__device__ __forceinline__ bool ahead_item(const StepArgs& a, int T, int q, int chunk, long long base,
-                                           int m_end, unsigned char* smem, unsigned long long* full,
-                                           unsigned& gstage) {
-  constexpr int SEG = seg<S>(), STAGE = stage_bytes<S>(), WBUF = wbuf_bytes<HALVES>();
+__device__ __forceinline__ void request_stage(const StepArgs& a, int j, unsigned g, unsigned char* smem,
+                                           Sync& sync) {
+  const Item& it = sync.it;
+  constexpr int SEG = seg<S>(), PLANE = hist_bytes<S>() / S::kPlanes, WL = wlag_bytes<HALVES>();
+  const int buf = (int)(g % stages<HALVES>());
+  unsigned char* st = smem + buf * stage_bytes<S, HALVES>();
+  const unsigned bar = tma::smem_addr(&sync.full[buf]), dst = tma::smem_addr(st);
+  const int mb = it.m0 + j * kLags;
+  int top = it.bs - mb;                          // slot of the stage's first lag
+  if (top < 0) top += a.n_cut;
+  const bool tiled = top >= kLags - 1;
+  const int lags = max(0, min(kLags, it.m1 - mb + 1));
+  tma::mbar_expect_tx(bar, kLags * WL + (tiled ? hist_bytes<S>() : lags * 3 * S::kPlanes * SEG));
+  tma::bulk_g2s(dst + hist_bytes<S>(),
+                a.wts32 + ((long long)(it.rec0 / kRec) * ahead_weight_lags(a.n_cut) + mb + kAhead) * WL,
+                kLags * WL, bar);
+  if (tiled) {
+#pragma unroll
+    for (int pl = 0; pl < S::kPlanes; ++pl)
+      tile_g2s(dst + pl * PLANE, a.tmap, it.rec0 * (S::kRecBytes / 4),
+               (pl * a.n_cut + top - (kLags - 1)) * 3, bar);
+  } else {
+    const unsigned char* hist = reinterpret_cast<const unsigned char*>(a.hist);
+    for (int i = 0; i < lags * 3 * S::kPlanes; ++i) {
+      const int pl = i % S::kPlanes, l = i / S::kPlanes / 3, c = i / S::kPlanes % 3;
+      int slot = top - l;
+      if (slot < 0) slot += a.n_cut;
+      tma::bulk_g2s(dst + pl * PLANE + ((kLags - 1 - l) * 3 + c) * SEG,
+                    hist + (pl * a.slot_stride + ((long long)slot * 3 + c) * a.n_orb_pad + it.rec0) *
+                               S::kRecBytes,
+                    SEG, bar);
+    }
+  }
+}
+
+// A warp's part of an item: one of the five sums for the 32 members of 8 records.
+// The terms of 32 lags are chained by multiply-adds, then folded into the running
+// sums (in shared memory) with one compensated addition.  The warps meet only at the
+// stages: each waits for its copies, and the last to leave one requests its next
+// filling.  Returns false if a bounded wait gave up.
+template <class S, bool HALVES>
+__device__ __forceinline__ bool sum_item(const StepArgs& a, int q, unsigned char* smem, Sync& sync,
+                                         unsigned g) {
+  const Item& it = sync.it;
+  const int m0 = it.m0, m1 = it.m1, nblk = it.nblk, n_cut = a.n_cut;
+  constexpr int SEG = seg<S>(), STAGE = stage_bytes<S, HALVES>(), PLANE = hist_bytes<S>() / S::kPlanes;
+  constexpr int WL = wlag_bytes<HALVES>(), NS = stages<HALVES>();
   using IO = MemberIO<S>;
   using u64 = unsigned long long;
   const int tid = threadIdx.x, lane = tid & 31;
-  const int f = tid >> 5;                        // the sum: C11, C33, C22, C12a, C12b
+  const int f = tid / kOrbitTile, x = tid % kOrbitTile;      // the sum (C11, C33, C22, C12a, C12b); member
   const int comp = f == 0 || f == 4 ? 0 : (f == 1 ? 2 : 1);
   const int kern = f == 0 ? 0 : (f == 1 ? 2 : (f == 2 ? 1 : 3));
-  const int rec0 = T * kOrbitTile + q * kRec;
-  const long long orb = a.n_orb_pad;
-  const int m0 = 1 + chunk * a.ahead_lc;
-  const int m1 = min(m0 + a.ahead_lc - 1, m_end);           // last lag of this chunk
-  const int nblk = (m1 - m0 + kAhead) / kAhead;
-  const int bs = (int)(base % a.n_cut);
-  unsigned char* wsm = smem + kStages * STAGE;
+  const int woff = (HALVES ? x >> 1 : x >> 2) * 16 + kern * 4;
+  // lags with a weight: the cutoff's zeros are in the weights, a window's are not
+  const int lim = a.lmax ? a.lmax[2 * (it.rec0 + (x >> 2)) + ((x >> 1) & 1)] : 0x7fffffff;
+  // this thread's running sums, two per 16 bytes, strided over the threads
+  ulonglong2* run = reinterpret_cast<ulonglong2*>(smem + NS * STAGE) + tid;
 
-  const unsigned char* hist = reinterpret_cast<const unsigned char*>(a.hist);
-  const long long plane_bytes = a.slot_stride * S::kRecBytes;
-  // stage b: lags m0 + 16 b .. +15 (clipped to m1), one copy per lag, component and
-  // plane, issued by the lanes of warp 0
-  auto issue = [&](int b) {
-    const int buf = (int)((gstage + b) % kStages);
-    const int mb = m0 + b * kAhead;
-    const int copies = min(kAhead, m1 - mb + 1) * 3 * S::kPlanes;
-    const unsigned bar = tma::smem_addr(&full[buf]);
-    if (lane == 0) tma::mbar_expect_tx(bar, (unsigned)(copies * SEG));
-    __syncwarp();
-    for (int i = lane; i < copies; i += 32) {
-      const int pl = i % S::kPlanes, lc = i / S::kPlanes;   // lc = lag * 3 + component
-      int slot = bs - (mb + lc / 3);
-      if (slot < 0) slot += a.n_cut;
-      tma::bulk_g2s(tma::smem_addr(smem + buf * STAGE + i * SEG),
-                    hist + pl * plane_bytes + (((long long)slot * 3 + lc % 3) * orb + rec0) * S::kRecBytes,
-                    SEG, bar);
+  u64 y[kAhead], w[kAhead];
+  {
+    const unsigned char* w0 = a.wts32 + ((long long)(it.rec0 / kRec) * ahead_weight_lags(a.n_cut) + it.m0) * WL + woff;
+#pragma unroll
+    for (int s = 0; s < kAhead; ++s) {
+      y[s] = 0ull;                               // (0.f, 0.f)
+      float v = __ldg(reinterpret_cast<const float*>(w0 + s * WL));
+      if (it.m0 + s >= lim) v = 0.f;
+      w[s] = pack2(make_float2(v, v));
+      if (s % 2) run[(s / 2) * kThreads] = make_ulonglong2(0ull, 0ull);
     }
-  };
-  if (f == 0)
-    for (int b = 0; b < min(kStages - 1, nblk); ++b) issue(b);
-
-  // the weights of block b: (record half, lag) pairs over the CTA's threads
-  const float4* tab = reinterpret_cast<const float4*>(a.table);
-  auto weights = [&](int b) {
-    constexpr int PAIRS = (HALVES ? 2 : 1) * kRec * kAhead;
-#pragma unroll
-    for (int r = 0; r < (PAIRS + kThreads - 1) / kThreads; ++r) {
-      const int i = tid + r * kThreads;
-      if (i < PAIRS) {
-        const int l = i % kAhead, rh = i / kAhead;          // rh: record (x 2 + half)
-        const int x = HALVES ? 2 * rec0 + rh : 2 * (rec0 + rh);
-        const int m = m0 + b * kAhead + l;
-        float w[4] = {0.f, 0.f, 0.f, 0.f};
-        if (m < a.n_cut && (!a.lmax || m < a.lmax[x]))
-          lag_weights(tab, (u64)m * a.ustep[x], reinterpret_cast<const float*>(a.dT)[x], w);
-        unsigned char* p = wsm + (b & 1) * WBUF + rh * kWRow + l * 8;
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          *reinterpret_cast<float2*>(p + k * ((HALVES ? 2 : 1) * kRec * kWRow)) = make_float2(w[k], w[k]);
-      }
-    }
-  };
-  weights(0);
-  weights(1);
-  __syncthreads();
-  const int row = HALVES ? 2 * (lane >> 2) + ((lane >> 1) & 1) : lane >> 2;
-  const unsigned char* wrow = wsm + (kern * (HALVES ? 2 : 1) * kRec + row) * kWRow;
-
-  u64 sum[kAhead], y[kAhead], w[kAhead];
-#pragma unroll
-  for (int s = 0; s < kAhead; ++s) sum[s] = y[s] = 0ull;    // (0.f, 0.f)
-#pragma unroll
-  for (int s = 0; s < kAhead; s += 2) {
-    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(wrow + s * 8);
-    w[s] = v.x;
-    w[s + 1] = v.y;
   }
-
-  bool ok = true;
-  int done = 0;
   for (int b = 0; b < nblk; ++b) {
-    const unsigned gi = gstage + b;
-    const bool landed = tma::mbar_wait(tma::smem_addr(&full[gi % kStages]), (gi / kStages) & 1u, a.err);
-    // every thread has left block b - 1: its stage and its weights may be replaced,
-    // and the weights of block b + 1 are complete
-    if (!__syncthreads_and(landed)) {
-      ok = false;
-      break;
-    }
-    if (f == 0 && b + kStages - 1 < nblk) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      issue(b + kStages - 1);
-    }
-    done = b + 1;
-    const unsigned char* st = smem + (gi % kStages) * STAGE + comp * S::kPlanes * SEG;
-    const unsigned char* wnext = wrow + ((b + 1) & 1) * WBUF;
     const int mb = m0 + b * kAhead;
-    // At lag l output s takes weight l + s of the window; slot l is then replaced
-    // by weight l of the next block.
-    auto block = [&](auto tail) {
+    bool ok = true;
+    // Half a block, one stage: at lag l output s takes weight l + s of the window;
+    // slot l is then replaced by the weight 16 lags on.
+    auto half = [&](auto first, auto tail, auto window) {
       constexpr bool TAIL = decltype(tail)::value;
-      ulonglong2 nw;
+      constexpr int L0 = decltype(first)::value;
+      const int buf = (int)(g % NS);
+      ok = __all_sync(0xffffffffu, tma::mbar_wait(tma::smem_addr(&sync.full[buf]), (g / NS) & 1u, a.err));
+      if (!ok) return;
+      const unsigned char* st = smem + buf * STAGE;
+      float2 dn = IO::smem(st + ((kLags - 1) * 3 + comp) * SEG, PLANE, x);
 #pragma unroll
-      for (int l = 0; l < kAhead; ++l) {
-        float2 d = IO::smem(st + l * 3 * S::kPlanes * SEG, lane);
+      for (int k = 0; k < kLags; ++k) {
+        
+        const int l = L0 + k;
+        float2 d = dn;                           // the next lag's value is on its way
+        if (k + 1 < kLags) dn = IO::smem(st + ((kLags - 2 - k) * 3 + comp) * SEG, PLANE, x);
         if (TAIL && mb + l > m1) d = make_float2(0.f, 0.f);
-        if (l % 2 == 0) nw = *reinterpret_cast<const ulonglong2*>(wnext + l * 8);
         const u64 dd = pack2(d);
+        float v = *reinterpret_cast<const float*>(st + hist_bytes<S>() + woff + k * WL);
+        if (decltype(window)::value && mb + kAhead + l >= lim) v = 0.f;
 #pragma unroll
         for (int s = 0; s < kAhead; ++s) {
           // terms past the cutoff are left out, not multiplied by zero: a
           // non-finite value leaves the sums with its last lag
-          const u64 ds = TAIL && mb + l + s >= a.n_cut ? 0ull : dd;
+          const u64 ds = TAIL && mb + l + s >= n_cut ? 0ull : dd;
           y[s] = fma2r(w[(l + s) % kAhead], ds, y[s]);
         }
-        w[l] = l % 2 == 0 ? nw.x : nw.y;
+        w[l] = pack2(make_float2(v, v));
       }
+      __syncwarp();
+      if (lane == 0) {
+        const int j = 2 * b + L0 / kLags;
+        if (shared_inc(&sync.left[buf]) % kWarps == kWarps - 1 && j + NS < 2 * nblk) {
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          sync.requested = g + NS + 1;
+          request_stage<S, HALVES>(a, j + NS, g + NS, smem, sync);
+        }
+      }
+      ++g;
     };
-    if (mb + 2 * kAhead - 2 < a.n_cut && mb + kAhead - 1 <= m1)
-      block(std::false_type{});
+    using Lo = std::integral_constant<int, 0>;
+    using Hi = std::integral_constant<int, kLags>;
+    auto block = [&](auto tail, auto window) {
+      half(Lo{}, tail, window);
+      if (ok) half(Hi{}, tail, window);
+    };
+    if (mb + 2 * kAhead - 2 >= n_cut || mb + kAhead - 1 > m1)
+      block(std::true_type{}, std::true_type{});
+    else if (a.lmax)
+      block(std::false_type{}, std::true_type{});
     else
-      block(std::true_type{});
-    if (b + 2 <= nblk) weights(b + 2);
-    if ((b & 1) || b + 1 == nblk) {
+      block(std::false_type{}, std::false_type{});
+    if (!ok) return false;
+    if (b % kFold == kFold - 1) {
 #pragma unroll
-      for (int s = 0; s < kAhead; ++s) {
-        const u64 t = add2r(sum[s], y[s]);
-        y[s] = sub2r(y[s], sub2r(t, sum[s]));      // minus the compensation
-        sum[s] = t;
+      for (int s = 0; s < kAhead; s += 2) {
+        const ulonglong2 o = run[(s / 2) * kThreads];
+        const ulonglong2 t = make_ulonglong2(add2r(o.x, y[s]), add2r(o.y, y[s + 1]));
+        y[s] = sub2r(y[s], sub2r(t.x, o.x));     // minus the compensation
+        y[s + 1] = sub2r(y[s + 1], sub2r(t.y, o.y));
+        run[(s / 2) * kThreads] = t;
       }
     }
   }
-  if (!ok) {
-    if (tid == 0) atomicExch(a.err, 1);
-    const int issued = min(nblk, done + kStages - 1);   // land what is in flight
-    for (int s = done; s < issued; ++s) {
-      const unsigned gs = gstage + s;
-      tma::mbar_wait(tma::smem_addr(&full[gs % kStages]), (gs / kStages) & 1u, &tma::kNoError);
-    }
-    return false;
-  }
-  gstage += nblk;
-  float* out = a.ahead + (((long long)chunk * (orb / kOrbitTile) + T) * kAhead * kFields + 2 * f) *
-                             (kOrbitTile * kMembers) + q * (kRec * kMembers) + lane;
+  float* out = a.ahead + (((long long)it.chunk * (a.n_orb_pad / kOrbitTile) + it.T) * kAhead * kFields + 2 * f) *
+                             (kOrbitTile * kMembers) + q * (kRec * kMembers) + x;
 #pragma unroll
   for (int s = 0; s < kAhead; ++s) {
-    const float2 r = unpack2(add2r(sum[s], y[s]));
+    const ulonglong2 o2 = run[(s / 2) * kThreads];
+    const float2 r = unpack2(add2r(s % 2 ? o2.y : o2.x, y[s]));
     float* o = out + (long long)s * kFields * (kOrbitTile * kMembers);
     o[0] = r.x;
     o[kOrbitTile * kMembers] = r.y;
   }
-  __syncthreads();   // the weight buffers are free for the next tile
   return true;
 }
 
-// The tiles 16 i .. 16 i + 15 of one update, records 8 q .. of each, one chunk of
+// The tiles 16 i .. 16 i + 15 of one update, records 32 q .. of each, one chunk of
 // lags: in a running time loop one of the 16 starts a new block at every step.
 template <class S, bool HALVES>
 __device__ __forceinline__ void ahead_tiles(const StepArgs& a, int i, int q, int chunk,
-                                            unsigned char* smem, unsigned long long* full) {
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int b = 0; b < kStages; ++b) tma::mbar_init(tma::smem_addr(&full[b]), 1);
+                                            unsigned char* smem, Sync& sync) {
+  constexpr int NS = stages<HALVES>();
+  const int tid = threadIdx.x;
+  if (tid < NS) {
+    tma::mbar_init(tma::smem_addr(&sync.full[tid]), 1);
+    sync.left[tid] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  __syncthreads();
   const long long n = *a.step;
   const int tiles = a.n_orb_pad / kOrbitTile;
-  unsigned gstage = 0;
-  for (int T = i * kAhead; T < min(tiles, (i + 1) * kAhead); ++T) {
-    const long long base = block_base(n, T);
-    const int m_end = last_lag(a, base, T);
-    if (1 + chunk * a.ahead_lc > m_end) continue;
-    long long* stamp = a.stamp + ((long long)chunk * tiles + T) * kSub + q;
-    const long long mark = base * 65536 + a.config_id;
-    if (*stamp == mark) continue;
-    if (!ahead_item<S, HALVES>(a, T, q, chunk, base, m_end, smem, full, gstage)) return;
-    if (threadIdx.x == 0) *stamp = mark;
+  // lane t looks at tile 16 i + t: is its block due in this chunk, and not yet formed
+  const int lane = tid & 31, Tt = i * kAhead + lane;
+  bool due = false;
+  if (lane < kAhead && Tt < tiles) {
+    const long long base = block_base(n, Tt);
+    due = 1 + chunk * a.ahead_lc <= last_lag(a, base, Tt) &&
+          a.stamp[((long long)chunk * tiles + Tt) * kSub + q] != block_mark(a, base);
+  }
+  unsigned todo = __ballot_sync(0xffffffffu, due);
+  __syncthreads();   // barriers ready; every warp has read the stamps
+  unsigned g = 0;    // stages of the items before this one
+  for (; todo; todo &= todo - 1) {
+    if (tid == 0) sync.it.set(a, i * kAhead + __ffs(todo) - 1, q, chunk, n);
+    __syncthreads();
+    if (tid == 0) {
+      const int first = min(NS, 2 * sync.it.nblk);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      sync.requested = g + first;
+      for (int j = 0; j < first; ++j) request_stage<S, HALVES>(a, j, g + j, smem, sync);
+    }
+    const bool ok = sum_item<S, HALVES>(a, q, smem, sync, g);
+    if (!__syncthreads_and(ok)) {
+      if (tid == 0) {
+        atomicExch(a.err, 1);
+        // land the copies in flight before the CTA's shared memory is released
+        for (unsigned s = sync.requested < NS ? 0 : sync.requested - NS; s < sync.requested; ++s)
+          tma::mbar_wait(tma::smem_addr(&sync.full[s % NS]), (s / NS) & 1u, &tma::kNoError);
+      }
+      return;
+    }
+    g += 2 * sync.it.nblk;
+    if (tid == 0)
+      a.stamp[((long long)chunk * tiles + sync.it.T) * kSub + q] = block_mark(a, sync.it.base);
+    __syncthreads();   // the item is read before the next replaces it
   }
 }
 
+// The weights of every (record half, lag) as the stages read them: [32 records][lag]
+// [record (x 2 halves)][4], zero past the cutoff.  They depend on the handle alone:
+// interpolated once, in double and rounded once (interpolating them in the summing
+// kernel took its FP32 pipe and a warp's latency: 1.21 ms for 1024^2 x 4096 with a
+// warp set aside for it, 1.23 with all, against 1.16).
+template <bool HALVES>
+__global__ void __launch_bounds__(256) ahead_weights_kernel(const StepArgs a, float4* __restrict__ out) {
+  constexpr int ROWS = (HALVES ? 2 : 1) * kRec;
+  const long long lags = ahead_weight_lags(a.n_cut);
+  const long long i = blockIdx.x * 256ll + threadIdx.x;
+  if (i >= (long long)a.n_orb_pad / kRec * lags * ROWS) return;
+  const int m = (int)(i / ROWS % lags);
+  const long long rec0 = i / ROWS / lags * kRec;
+  const long long x = HALVES ? 2 * rec0 + i % ROWS : 2 * (rec0 + i % ROWS);
+  double w[4] = {0.0, 0.0, 0.0, 0.0};
+  if (m < a.n_cut) {
+    const unsigned long long us = a.ustep[x];    // dT / h in 32.32 fixed point
+    lag_weights(reinterpret_cast<const Double4*>(a.table64), (unsigned long long)m * us,
+                (double)us * (a.table_h * (1.0 / 4294967296.0)), w);
+  }
+  out[i] = make_float4((float)w[0], (float)w[1], (float)w[2], (float)w[3]);
+}
+
 template <class S, bool HALVES>
-__global__ void __launch_bounds__(kThreads, 3) ahead_kernel(const StepArgs a) {
+__global__ void __launch_bounds__(kThreads, 1) ahead_kernel(const __grid_constant__ StepArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ __align__(8) unsigned long long full[kStages];
-  ahead_tiles<S, HALVES>(a, blockIdx.x / kSub, blockIdx.x % kSub, blockIdx.y, smem, full);
+  __shared__ __align__(8) Sync sync;
+  ahead_tiles<S, HALVES>(a, blockIdx.x / kSub, blockIdx.x % kSub, blockIdx.y, smem, sync);
 }
 
 // The same over the members of a batch: CTA item_prefix[s] + ... belongs to member s,
 // 16 sub-tiles of each group of 16 tiles, chunk-major.
 template <class S, bool HALVES>
-__global__ void __launch_bounds__(kThreads, 3)
+__global__ void __launch_bounds__(kThreads, 1)
 ahead_batch_kernel(const StepArgs* __restrict__ args, const int* __restrict__ item_prefix, int nb) {
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ __align__(8) unsigned long long full[kStages];
+  __shared__ __align__(8) Sync sync;
   __shared__ StepArgs s_args;
   __shared__ int s_local;
   if (threadIdx.x == 0) {
@@ -347,7 +445,7 @@ ahead_batch_kernel(const StepArgs* __restrict__ args, const int* __restrict__ it
   __syncthreads();
   const int per_chunk = ahead_ctas(s_args.n_orb_pad);
   const int r = s_local % per_chunk;
-  ahead_tiles<S, HALVES>(s_args, r / kSub, r % kSub, s_local / per_chunk, smem, full);
+  ahead_tiles<S, HALVES>(s_args, r / kSub, r % kSub, s_local / per_chunk, smem, sync);
 }
 
 // A step's sums of one member (one thread): the current spectra rotated into the
@@ -384,6 +482,8 @@ __device__ __forceinline__ void near_member(const StepArgs& a, int T, int x) {
   for (int c = 0; c < 3; ++c)
     R[c] = IO::store(a.hist, ((long long)sn * 3 + c) * comp_stride + mi, a.slot_stride, D[c]);
 
+  // weights from the table, which stays in L2 (reading the stored ones, 16 bytes per
+  // record and lag from HBM, took the kernel from 58 to 74 us at 1024^2)
   const float4* tab = reinterpret_cast<const float4*>(a.table);
   const float dT = reinterpret_cast<const float*>(a.dT)[hx];
   const unsigned long long us = a.ustep[hx];
@@ -403,7 +503,7 @@ __device__ __forceinline__ void near_member(const StepArgs& a, int T, int x) {
     kadd<1>(acc[6], cmp[6], w[3], d[1].x); kadd<1>(acc[7], cmp[7], w[3], d[1].y);
     kadd<1>(acc[8], cmp[8], w[3], d[0].x); kadd<1>(acc[9], cmp[9], w[3], d[0].y);
   };
-  // chunks of the block sums, two at a time in flight
+  // the chunks' block sums
   const int m_far = last_lag(a, base, T);
   const int nch = m_far > 0 ? (m_far + a.ahead_lc - 1) / a.ahead_lc : 0;
   const long long chunk_stride = comp_stride * kAhead * kFields;
@@ -429,6 +529,7 @@ __device__ __forceinline__ void near_member(const StepArgs& a, int T, int x) {
 #pragma unroll
     for (int i = 0; i < 4; ++i)
       if (m + i <= M) {
+
         int slot = sn - (m + i);
         if (slot < 0) slot += a.n_cut;
 #pragma unroll
@@ -536,14 +637,24 @@ cudaError_t launch_near(const StepArgs& a, cudaStream_t st, const BatchLaunch* b
   return cudaGetLastError();
 }
 
+template <bool HALVES>
+cudaError_t launch_weights(const StepArgs& a, cudaStream_t st) {
+  const long long total = (long long)ahead_weight_bytes(a.n_orb_pad, a.n_cut, HALVES) / 16;
+  ahead_weights_kernel<HALVES><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(
+      a, reinterpret_cast<float4*>(const_cast<unsigned char*>(a.wts32)));
+  return cudaGetLastError();
+}
+
 // One precision's entry: stage 0 sets the kernels' attributes, 1 launches the
-// block sums, 2 the step's own sums and the assembly (over `tiles` tiles of a batch).
+// block sums, 2 the step's own sums and the assembly (over `tiles` tiles of a
+// batch), 3 fills the handle's weights.
 template <class S>
 cudaError_t run_stage(const StepArgs& a, int stage, bool halves, cudaStream_t st,
                       const BatchLaunch* batch, int tiles) {
   switch (stage) {
     case 0: return halves ? prepare<S, true>() : prepare<S, false>();
     case 1: return halves ? launch_sums<S, true>(a, st, batch) : launch_sums<S, false>(a, st, batch);
+    case 3: return halves ? launch_weights<true>(a, st) : launch_weights<false>(a, st);
     case 2: return launch_near<S>(a, st, batch, tiles);
     default: return cudaErrorInvalidValue;
   }

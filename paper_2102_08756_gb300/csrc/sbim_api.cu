@@ -13,6 +13,7 @@
 //   (3) C2R FFT of the traction spectra    (cuFFT)
 //   (4) traction epilogue                  epilogue_kernel
 // with no host synchronisation.
+#include <cuda.h>
 #include <cufft.h>
 
 #include <algorithm>
@@ -72,7 +73,6 @@ constexpr double kPi = 3.141592653589793238462643383279502884;
 constexpr int kProfRing = 512;
 constexpr int kProfEvents = 6;
 constexpr size_t kSpareBytes = 256ull << 20;
-constexpr int kAheadLags = sbim::kAhead;   // lags per chunk of the block sums: a multiple of this
 
 // 16-point Gauss-Legendre nodes and weights on [-1, 1] (Newton on P_16).
 void gauss_legendre16(double* x, double* w) {
@@ -116,11 +116,13 @@ struct sbim_ctx {
   int lags_per_cta = 0;       // 0: automatic
   size_t part_bytes = 0;
   bool use_ahead = false;     // time-blocked convolution (sbim_ahead.cuh)
-  int ahead_lc = kAheadLags, ahead_chunks = 1;
+  int ahead_lc = sbim::kAhead, ahead_chunks = 1;
   float* d_ahead = nullptr;
   size_t ahead_bytes = 0;
   long long* d_stamp = nullptr;
   size_t stamp_bytes = 0;
+  void* d_tmap = nullptr;     // CUtensorMap of the ring
+  void* d_wts32 = nullptr;    // the block sums' weights
   int config_id = 0;          // counts changes of chunking and window (part of the stamps)
   double tab_h = 0;
   long long tab_n = 0;
@@ -172,6 +174,8 @@ struct sbim_ctx {
 };
 
 namespace {
+
+sbim::StepArgs step_args(const sbim_ctx* c);
 
 // Integer weights (a, b) with L1 / L3 = a / b exactly, a and b coprime and
 // small, so that |k|^2 (L1 L3 / 2 pi)^2 = (j1 b)^2 + (j3 a)^2 is an exact integer
@@ -398,24 +402,24 @@ int alloc_partials(sbim_ctx& c) {
   return SBIM_OK;
 }
 
-// Lag chunks of the block sums.  One chunk is groups x 16 CTAs of 8 records (one
-// tile in 16 is due at a step), 3 CTAs per SM; a CTA takes ~70 ns per lag in a full
-// wave and ~25 lags' worth to fill its pipeline, and every chunk adds partial sums
-// that are written and read once (2 x 160 B per record and step).  The count that
+// Lag chunks of the block sums.  One chunk is groups x 4 CTAs of 32 records (one
+// tile in 16 is due at a step), one CTA per SM; a CTA takes ~80 ns per lag and ~50
+// lags' worth to start and end, and every chunk adds partial sums that are written
+// and read once (2 x 160 B per record and step).  The count that
 // minimises the sum of both keeps the last wave full on small grids and few chunks
 // on large ones (4 at 1024^2 x 4096).
 void choose_ahead(sbim_ctx& c, int sms) {
   const int lags = std::max(1, c.n_cut - 1);
-  auto round16 = [](int x) { return (x + kAheadLags - 1) / kAheadLags * kAheadLags; };
+  auto round16 = [](int x) { return (x + sbim::kAhead - 1) / sbim::kAhead * sbim::kAhead; };
   if (c.lags_per_cta > 0) {
     c.ahead_lc = round16(std::min(c.lags_per_cta, lags));
   } else {
     const double ctas = sbim::ahead_ctas(c.n_orb_pad);
     double best = 0;
-    for (int S = 1; S <= std::min(32, round16(lags) / kAheadLags); ++S) {
+    for (int S = 1; S <= std::min(32, round16(lags) / sbim::kAhead); ++S) {
       const int lc = round16((lags + S - 1) / S);
-      const double waves = std::ceil(ctas * ((lags + lc - 1) / lc) / (3.0 * sms));
-      const double ns = waves * (lc + 25) * 70.0 + S * (double)c.n_orb_pad * 320.0 / 6000.0;
+      const double waves = std::ceil(ctas * ((lags + lc - 1) / lc) / sms);
+      const double ns = waves * (lc + 50) * 80.0 + S * (double)c.n_orb_pad * 320.0 / 6000.0;
       if (S == 1 || ns < best) {
         best = ns;
         c.ahead_lc = lc;
@@ -435,19 +439,56 @@ int forget_ahead(sbim_ctx* c) {
   return SBIM_OK;
 }
 
-// Room for the block sums of the current chunking, leaving `spare` bytes of the
+// The ring as a 2D tensor of 4-byte words for the tiled copies of the block sums:
+// one row per (plane, slot, component), a box of 8 slots x 3 components x 32 records.
+int make_ring_map(sbim_ctx& c) {
+  void* fn = nullptr;
+  cudaDriverEntryPointQueryResult found;
+  CU(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found));
+  if (found != cudaDriverEntryPointSuccess) return fail(SBIM_ERR_CUDA, "cuTensorMapEncodeTiled not found");
+  const int planes = c.prec == SBIM_BF16X2 ? 2 : 1, words = c.prec == SBIM_FP32 ? 8 : 4;
+  const cuuint64_t dims[2] = {(cuuint64_t)c.n_orb_pad * words, (cuuint64_t)planes * c.n_cut * 3};
+  const cuuint64_t pitch[1] = {dims[0] * 4};
+  const cuuint32_t box[2] = {(cuuint32_t)(sbim::kAheadRec * words), 3 * sbim::kAheadLags}, step[2] = {1, 1};
+  CUtensorMap map;
+  const CUresult r = ((decltype(&cuTensorMapEncodeTiled))fn)(
+      &map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, c.d_hist, dims, pitch, box, step,
+      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return fail(SBIM_ERR_CUDA, "cuTensorMapEncodeTiled: %d", (int)r);
+  CU(cudaMalloc(&c.d_tmap, sizeof map));
+  CU(cudaMemcpyAsync(c.d_tmap, &map, sizeof map, cudaMemcpyHostToDevice, c.stream));
+  CU(cudaStreamSynchronize(c.stream));   // map leaves scope
+  return SBIM_OK;
+}
+
+// Room for the block sums of the current chunking (and, once, for the weights they
+// take, 16 bytes per record and lag beside its 96 of FP32 history), leaving `spare` bytes of the
 // device free; false if there is none (the caller then convolves step by step).
 bool alloc_ahead(sbim_ctx& c, size_t spare) {
   const size_t need = ahead_need(c);
   const size_t sneed = (size_t)c.ahead_chunks * c.n_orb_pad / sbim::kAheadRec * sizeof(long long);
   if (need <= c.ahead_bytes && sneed <= c.stamp_bytes) return forget_ahead(&c) == SBIM_OK;
+  const size_t wneed = c.d_wts32 ? 0 : sbim::ahead_weight_bytes(c.n_orb_pad, c.n_cut, c.halves);
   size_t free_b = 0, total_b = 0;
-  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || need + sneed + spare > free_b) return false;
-  void *fresh = nullptr, *stamps = nullptr;
-  if (cudaMalloc(&fresh, need) != cudaSuccess || cudaMalloc(&stamps, sneed) != cudaSuccess) {
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || need + sneed + wneed + spare > free_b) return false;
+  void *fresh = nullptr, *stamps = nullptr, *wts = nullptr;
+  if (cudaMalloc(&fresh, need) != cudaSuccess || cudaMalloc(&stamps, sneed) != cudaSuccess ||
+      (wneed && cudaMalloc(&wts, wneed) != cudaSuccess)) {
     cudaGetLastError();
     if (fresh) cudaFree(fresh);
+    if (stamps) cudaFree(stamps);
     return false;
+  }
+  if (wneed) {
+    c.d_wts32 = wts;
+    if (sbim::launch_ahead(step_args(&c), c.prec, 3, c.halves, c.stream) != cudaSuccess) {
+      c.d_wts32 = nullptr;
+      cudaFree(wts);
+      cudaFree(fresh);
+      cudaFree(stamps);
+      return false;
+    }
   }
   if (c.d_ahead) {
     cudaStreamSynchronize(c.stream);
@@ -472,6 +513,8 @@ int configure_conv(sbim_ctx& c, size_t spare) {
     CU(cudaGetDevice(&dev));
     CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     choose_ahead(c, sms);
+    if (!c.d_tmap && c.n_cut >= sbim::kAheadLags)   // shorter rings always wrap: copied row by row
+      if (const int rc2 = make_ring_map(c)) return rc2;
     CU(sbim::launch_ahead(sbim::StepArgs{}, c.prec, 0, c.halves, nullptr));
     if (alloc_ahead(c, spare)) {
       c.use_ahead = true;
@@ -488,7 +531,7 @@ void release(sbim_ctx* c) {
   void* ptrs[] = {c->d_bin, c->d_dir, c->d_wout, c->d_dT, c->d_ustep, c->d_muq,
                   c->d_tab64, c->d_tab32, c->d_gl, c->d_hist, c->d_part, c->d_uhat,
                   c->d_fhat, c->d_s, c->d_step, c->d_err, c->d_io, c->d_lmax,
-                  c->d_tile_lmax, c->d_nonfinite, c->d_wts, c->d_ahead, c->d_stamp};
+                  c->d_tile_lmax, c->d_nonfinite, c->d_wts, c->d_ahead, c->d_stamp, c->d_tmap, c->d_wts32};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
@@ -512,8 +555,6 @@ int harvest(sbim_ctx* c, long long upto) {
   }
   return SBIM_OK;
 }
-
-sbim::StepArgs step_args(const sbim_ctx* c);
 
 int create_impl(sbim_ctx* c) {
   c->mu = c->rho * c->cs * c->cs;
@@ -601,8 +642,6 @@ int create_impl(sbim_ctx* c) {
   CU(cudaMalloc(&c->d_step, sizeof(long long)));
   CU(cudaMalloc(&c->d_err, sizeof(int)));
   if (c->wts_bytes) CU(cudaMalloc(&c->d_wts, c->wts_bytes));
-  if (const int rc = configure_conv(*c, kSpareBytes)) return rc == SBIM_ERR_CUDA ? rc : SBIM_ERR_OOM;
-
   cudaStream_t st = c->stream;
   CU(cudaMemcpyAsync(c->d_bin, h_bin.data(), h_bin.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   if (dbl)
@@ -629,6 +668,7 @@ int create_impl(sbim_ctx* c) {
   CU(sbim::launch_table_build(c->d_tab64, c->d_tab32, c->tab_n, c->tab_h, c->eta, c->d_gl,
                               c->d_gl + 16, st));
   if (c->d_wts) CU(sbim::launch_weights64(step_args(c), c->d_wts, st));
+  if (const int rc = configure_conv(*c, kSpareBytes)) return rc == SBIM_ERR_CUDA ? rc : SBIM_ERR_OOM;
   CU(cudaMemsetAsync(c->d_step, 0, sizeof(long long), st));
   CU(cudaMemsetAsync(c->d_err, 0, sizeof(int), st));
   CU(cudaStreamSynchronize(st));
@@ -662,6 +702,10 @@ sbim::StepArgs step_args(const sbim_ctx* c) {
   a.step = c->d_step;
   a.err = c->d_err;
   a.part = c->d_part;
+  a.table64 = c->d_tab64;
+  a.table_h = c->tab_h;
+  a.tmap = c->d_tmap;
+  a.wts32 = (const unsigned char*)c->d_wts32;
   a.ahead = c->d_ahead;
   a.stamp = c->d_stamp;
   a.ahead_lc = c->ahead_lc;

@@ -63,7 +63,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // of wall time, or at once when the device error word is already set (another
 // CTA gave up), so a failure costs every CTA at most one second.
 __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, const int* err) {
-  const unsigned long long t0 = global_ns();
+  unsigned long long t0 = 0;   // read only once the first polls have failed
   for (unsigned it = 0;; ++it) {
     unsigned ok;
     asm volatile(
@@ -74,9 +74,11 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, const i
         : "r"(bar), "r"(parity)
         : "memory");
     if (ok) return true;
-    if ((it & 63u) == 63u &&
-        (global_ns() - t0 > kWaitNs || *(volatile const int*)err != 0))
-      return false;
+    if ((it & 63u) == 63u) {
+      const unsigned long long now = global_ns();
+      if (t0 == 0) t0 = now;
+      if (now - t0 > kWaitNs || *(volatile const int*)err != 0) return false;
+    }
   }
 }
 

@@ -31,7 +31,8 @@ constexpr int kFields = 10;      // real accumulators per member: 5 complex sums
 constexpr int kOrbitTile = 128;  // orbits per CTA of the assembly and of the default convolution
                                  // (the TMA convolution also runs 64 or 256: "modes per CTA")
 constexpr int kAhead = 16;       // steps per block of the time-blocked convolution
-constexpr int kAheadRec = 8;     // records per CTA of its block sums
+constexpr int kAheadRec = 32;    // records per CTA of its block sums
+constexpr int kAheadLags = 8;    // lags per copy of the ring
 
 // Everything the per-step kernels read; device pointers unless noted.
 struct StepArgs {
@@ -49,6 +50,10 @@ struct StepArgs {
                                    // (11, 22, 33, 12) as 4 doubles, or NULL
   // state
   void* hist;                      // ring buffer (layout per precision)
+  const void* table64;             // the kernel table in double
+  double table_h;                  // its spacing
+  const unsigned char* wts32;      // the block sums' weights (ahead_weights_kernel)
+  const void* tmap;                // device CUtensorMap of the ring: rows slot x component, box 24 rows x 32 records
   long long* step;                 // device step counter n
   int* err;                        // device error word (bounded waits that gave up)
   void* part;                      // [nchunks][40][n_orb_pad] partial sums
@@ -87,12 +92,18 @@ struct BatchLaunch {
 __host__ __device__ constexpr int ahead_groups(int n_orb_pad) {
   return (n_orb_pad / kOrbitTile + kAhead - 1) / kAhead;
 }
+// The block sums' weights: lags per 32 records (a block of lags past the cutoff is
+// read), and bytes in all.
+__host__ __device__ constexpr long long ahead_weight_lags(int n_cut) { return n_cut + 2 * kAhead; }
+__host__ __device__ constexpr long long ahead_weight_bytes(int n_orb_pad, int n_cut, bool halves) {
+  return n_orb_pad * ahead_weight_lags(n_cut) * (halves ? 32 : 16);
+}
 // CTAs of one lag chunk of the block sums.
 __host__ __device__ constexpr int ahead_ctas(int n_orb_pad) {
   return ahead_groups(n_orb_pad) * (kOrbitTile / kAheadRec);
 }
 // Time-blocked convolution of float-class histories (sbim_ahead.cuh): stage 0
-// prepares the kernels, stage 1 forms the block sums that are due, stage 2 adds the
+// prepares the kernels, stage 3 fills wts32, stage 1 forms the block sums that are due, stage 2 adds the
 // step's own lags, stores the current spectra and assembles the output spectra.
 // With `batch`, over its members (items and tiles as its prefix sums count them).
 cudaError_t launch_ahead(const StepArgs& a, int precision, int stage, bool halves, cudaStream_t st,
