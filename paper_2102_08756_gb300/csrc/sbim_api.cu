@@ -128,6 +128,9 @@ struct sbim_ctx {
   long long tab_n = 0;
   size_t real_size = 4;
 
+  // One allocation holds the plan, tables, ring, spectra and weights below (a handle
+  // with 18 of its own took 2 ms more to create and destroy on GB300).
+  void* d_arena = nullptr;
   int* d_bin = nullptr;
   void* d_dir = nullptr;  // float2, or double2 for the FP64 path
   float* d_wout = nullptr;
@@ -441,7 +444,7 @@ int forget_ahead(sbim_ctx* c) {
 
 // The ring as a 2D tensor of 4-byte words for the tiled copies of the block sums:
 // one row per (plane, slot, component), a box of 8 slots x 3 components x 32 records.
-int make_ring_map(sbim_ctx& c) {
+int make_ring_map(const sbim_ctx& c, CUtensorMap* map) {
   void* fn = nullptr;
   cudaDriverEntryPointQueryResult found;
   CU(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found));
@@ -450,73 +453,53 @@ int make_ring_map(sbim_ctx& c) {
   const cuuint64_t dims[2] = {(cuuint64_t)c.n_orb_pad * words, (cuuint64_t)planes * c.n_cut * 3};
   const cuuint64_t pitch[1] = {dims[0] * 4};
   const cuuint32_t box[2] = {(cuuint32_t)(sbim::kAheadRec * words), 3 * sbim::kAheadLags}, step[2] = {1, 1};
-  CUtensorMap map;
   const CUresult r = ((decltype(&cuTensorMapEncodeTiled))fn)(
-      &map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, c.d_hist, dims, pitch, box, step,
+      map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, c.d_hist, dims, pitch, box, step,
       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(SBIM_ERR_CUDA, "cuTensorMapEncodeTiled: %d", (int)r);
-  CU(cudaMalloc(&c.d_tmap, sizeof map));
-  CU(cudaMemcpyAsync(c.d_tmap, &map, sizeof map, cudaMemcpyHostToDevice, c.stream));
-  CU(cudaStreamSynchronize(c.stream));   // map leaves scope
   return SBIM_OK;
 }
 
-// Room for the block sums of the current chunking (and, once, for the weights they
-// take, 16 bytes per record and lag beside its 96 of FP32 history), leaving `spare` bytes of the
-// device free; false if there is none (the caller then convolves step by step).
-bool alloc_ahead(sbim_ctx& c, size_t spare) {
-  const size_t need = ahead_need(c);
+// Room for the block sums of the current chunking in at most `budget` bytes; false if
+// there is none, or none was left at creation for their weights (the caller then
+// convolves step by step).
+bool alloc_ahead(sbim_ctx& c, size_t budget) {
+  if (!c.d_wts32) return false;
   const size_t sneed = (size_t)c.ahead_chunks * c.n_orb_pad / sbim::kAheadRec * sizeof(long long);
-  if (need <= c.ahead_bytes && sneed <= c.stamp_bytes) return forget_ahead(&c) == SBIM_OK;
-  const size_t wneed = c.d_wts32 ? 0 : sbim::ahead_weight_bytes(c.n_orb_pad, c.n_cut, c.halves);
-  size_t free_b = 0, total_b = 0;
-  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || need + sneed + wneed + spare > free_b) return false;
-  void *fresh = nullptr, *stamps = nullptr, *wts = nullptr;
-  if (cudaMalloc(&fresh, need) != cudaSuccess || cudaMalloc(&stamps, sneed) != cudaSuccess ||
-      (wneed && cudaMalloc(&wts, wneed) != cudaSuccess)) {
-    cudaGetLastError();
-    if (fresh) cudaFree(fresh);
-    if (stamps) cudaFree(stamps);
-    return false;
-  }
-  if (wneed) {
-    c.d_wts32 = wts;
-    if (sbim::launch_ahead(step_args(&c), c.prec, 3, c.halves, c.stream) != cudaSuccess) {
-      c.d_wts32 = nullptr;
-      cudaFree(wts);
-      cudaFree(fresh);
-      cudaFree(stamps);
+  const size_t need = ahead_need(c) + sneed;     // stamps behind the sums
+  if (need > c.ahead_bytes) {
+    void* fresh = nullptr;
+    if (need > budget || cudaMalloc(&fresh, need) != cudaSuccess) {
+      cudaGetLastError();
       return false;
     }
+    if (c.d_ahead) {
+      cudaStreamSynchronize(c.stream);
+      cudaFree(c.d_ahead);
+    }
+    c.d_ahead = (float*)fresh;
+    c.ahead_bytes = need;
   }
-  if (c.d_ahead) {
-    cudaStreamSynchronize(c.stream);
-    cudaFree(c.d_ahead);
-    cudaFree(c.d_stamp);
-  }
-  c.d_ahead = (float*)fresh;
-  c.ahead_bytes = need;
-  c.d_stamp = (long long*)stamps;
+  c.d_stamp = (long long*)((char*)c.d_ahead + ahead_need(c));
   c.stamp_bytes = sneed;
   return forget_ahead(&c) == SBIM_OK;
 }
 
 // Launch, chunking and sums buffer for the current variant, tile and lags_per_cta.
-int configure_conv(sbim_ctx& c, size_t spare) {
+int configure_conv(sbim_ctx& c) {
   ++c.config_id;
   c.use_ahead = false;
   int rc = choose_chunks(c);
   if (rc != SBIM_OK) return rc;
-  if (c.prec != SBIM_FP64 && c.variant >= 1) {
+  if (c.d_wts32 && c.variant >= 1) {
     int dev = 0, sms = 148;
     CU(cudaGetDevice(&dev));
     CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     choose_ahead(c, sms);
-    if (!c.d_tmap && c.n_cut >= sbim::kAheadLags)   // shorter rings always wrap: copied row by row
-      if (const int rc2 = make_ring_map(c)) return rc2;
-    CU(sbim::launch_ahead(sbim::StepArgs{}, c.prec, 0, c.halves, nullptr));
-    if (alloc_ahead(c, spare)) {
+    size_t free_b = 0, total_b = 0;
+    CU(cudaMemGetInfo(&free_b, &total_b));
+    if (alloc_ahead(c, free_b > kSpareBytes ? free_b - kSpareBytes : 0)) {
       c.use_ahead = true;
       return SBIM_OK;
     }
@@ -528,10 +511,7 @@ void release(sbim_ctx* c) {
   if (!c) return;
   if (c->have_fwd) cufftDestroy(c->plan_fwd);
   if (c->have_inv) cufftDestroy(c->plan_inv);
-  void* ptrs[] = {c->d_bin, c->d_dir, c->d_wout, c->d_dT, c->d_ustep, c->d_muq,
-                  c->d_tab64, c->d_tab32, c->d_gl, c->d_hist, c->d_part, c->d_uhat,
-                  c->d_fhat, c->d_s, c->d_step, c->d_err, c->d_io, c->d_lmax,
-                  c->d_tile_lmax, c->d_nonfinite, c->d_wts, c->d_ahead, c->d_stamp, c->d_tmap, c->d_wts32};
+  void* ptrs[] = {c->d_arena, c->d_part, c->d_io, c->d_lmax, c->d_tile_lmax, c->d_nonfinite, c->d_ahead};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
@@ -591,17 +571,6 @@ int create_impl(sbim_ctx* c) {
       c->tab_n > (1LL << 31))
     return fail(SBIM_ERR_ARG, "history too long for the kernel table (n_cut x |k|max c_s dt)");
 
-  std::vector<int> h_bin(mem.size());
-  std::vector<float2> h_dir(mem.size());
-  std::vector<double2> h_dir64(mem.size());
-  std::vector<float> h_w(mem.size());
-  for (size_t i = 0; i < mem.size(); ++i) {
-    h_bin[i] = mem[i].bin;
-    h_dir[i] = make_float2((float)mem[i].e1, (float)mem[i].e3);
-    h_dir64[i] = make_double2(mem[i].e1, mem[i].e3);
-    h_w[i] = mem[i].w;
-  }
-
   if (choose_chunks(*c) != SBIM_OK) return SBIM_ERR_CUDA;
   if (c->variant >= 1)
     CU(sbim::prepare_conv_tma(c->prec, c->kahan, c->variant, c->tile, c->halves));
@@ -626,51 +595,75 @@ int create_impl(sbim_ctx* c) {
     if (need + wb + (512ull << 20) <= free_b) c->wts_bytes = wb;
   }
 
-  CU(cudaMalloc(&c->d_bin, h_bin.size() * sizeof(int)));
-  CU(cudaMalloc(&c->d_dir, h_dir.size() * (dbl ? sizeof(double2) : sizeof(float2))));
-  CU(cudaMalloc(&c->d_wout, h_w.size() * sizeof(float)));
-  CU(cudaMalloc(&c->d_dT, 2 * c->n_orb_pad * c->real_size));
-  CU(cudaMalloc(&c->d_muq, 2 * c->n_orb_pad * c->real_size));
-  CU(cudaMalloc(&c->d_ustep, 2 * c->n_orb_pad * sizeof(unsigned long long)));
-  CU(cudaMalloc(&c->d_tab64, (size_t)c->tab_n * 4 * sizeof(double)));
-  if (!dbl) CU(cudaMalloc(&c->d_tab32, (size_t)c->tab_n * 4 * sizeof(float)));
-  CU(cudaMalloc(&c->d_gl, 32 * sizeof(double)));
-  CU(cudaMalloc(&c->d_hist, c->hist_bytes));
-  CU(cudaMalloc(&c->d_uhat, 3 * (size_t)c->nbins * cplx));
-  CU(cudaMalloc(&c->d_fhat, 3 * (size_t)c->nbins * cplx));
-  CU(cudaMalloc(&c->d_s, c->field_elems() * c->real_size));
-  CU(cudaMalloc(&c->d_step, sizeof(long long)));
-  CU(cudaMalloc(&c->d_err, sizeof(int)));
-  if (c->wts_bytes) CU(cudaMalloc(&c->d_wts, c->wts_bytes));
-  cudaStream_t st = c->stream;
-  CU(cudaMemcpyAsync(c->d_bin, h_bin.data(), h_bin.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-  if (dbl)
-    CU(cudaMemcpyAsync(c->d_dir, h_dir64.data(), h_dir64.size() * sizeof(double2),
-                       cudaMemcpyHostToDevice, st));
-  else
-    CU(cudaMemcpyAsync(c->d_dir, h_dir.data(), h_dir.size() * sizeof(float2),
-                       cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(c->d_wout, h_w.data(), h_w.size() * sizeof(float), cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(c->d_ustep, ustep.data(), ustep.size() * sizeof(unsigned long long),
-                     cudaMemcpyHostToDevice, st));
-  if (dbl) {
-    CU(cudaMemcpyAsync(c->d_dT, dT.data(), dT.size() * 8, cudaMemcpyHostToDevice, st));
-    CU(cudaMemcpyAsync(c->d_muq, muq.data(), muq.size() * 8, cudaMemcpyHostToDevice, st));
-  } else {
-    std::vector<float> f1(dT.begin(), dT.end()), f2(muq.begin(), muq.end());
-    CU(cudaMemcpyAsync(c->d_dT, f1.data(), f1.size() * 4, cudaMemcpyHostToDevice, st));
-    CU(cudaMemcpyAsync(c->d_muq, f2.data(), f2.size() * 4, cudaMemcpyHostToDevice, st));
-    CU(cudaStreamSynchronize(st));  // f1, f2 leave scope
+  // The block sums' weights (16 B per record and lag beside 96 of FP32 history, 32 for
+  // half records) and the least room for the sums themselves; a handle that has none
+  // left convolves step by step.
+  const size_t w32 = dbl ? 0 : sbim::ahead_weight_bytes(c->n_orb_pad, c->n_cut, c->halves);
+  const bool blocked = w32 && need + w32 + (size_t)c->n_orb_pad * 4096 + kSpareBytes <= free_b;
+
+  // Lay the arena out: what the host fills in first, in one copy, then the rest.
+  size_t at = 0;
+  std::vector<std::pair<void**, size_t>> place;
+  auto put = [&](void** p, size_t bytes) {
+    place.push_back({p, at});
+    at += (bytes + 255) / 256 * 256;
+    return place.back().second;
+  };
+  const size_t m4 = mem.size(), o2 = 2 * (size_t)c->n_orb_pad;
+  const size_t o_bin = put((void**)&c->d_bin, m4 * sizeof(int));
+  const size_t o_dir = put(&c->d_dir, m4 * 2 * c->real_size);
+  const size_t o_w = put((void**)&c->d_wout, m4 * sizeof(float));
+  const size_t o_dT = put(&c->d_dT, o2 * c->real_size);
+  const size_t o_muq = put(&c->d_muq, o2 * c->real_size);
+  const size_t o_us = put((void**)&c->d_ustep, o2 * sizeof(unsigned long long));
+  const size_t o_gl = put((void**)&c->d_gl, 32 * sizeof(double));
+  const size_t o_map = put(&c->d_tmap, sizeof(CUtensorMap));
+  put((void**)&c->d_step, sizeof(long long));   // zero, like the error word
+  put((void**)&c->d_err, sizeof(int));
+  const size_t filled = at;
+  put((void**)&c->d_tab64, (size_t)c->tab_n * 4 * sizeof(double));
+  if (!dbl) put((void**)&c->d_tab32, (size_t)c->tab_n * 4 * sizeof(float));
+  put(&c->d_uhat, 3 * (size_t)c->nbins * cplx);
+  put(&c->d_fhat, 3 * (size_t)c->nbins * cplx);
+  put(&c->d_s, c->field_elems() * c->real_size);
+  if (blocked) put(&c->d_wts32, w32);
+  if (c->wts_bytes) put(&c->d_wts, c->wts_bytes);
+  put(&c->d_hist, c->hist_bytes);
+  CU(cudaMalloc(&c->d_arena, at));
+  for (auto& x : place) *x.first = (char*)c->d_arena + x.second;
+
+  std::vector<unsigned char> host(filled, 0);
+  auto real = [&](size_t off, size_t i, double v) {
+    if (dbl) ((double*)&host[off])[i] = v;
+    else ((float*)&host[off])[i] = (float)v;
+  };
+  for (size_t i = 0; i < m4; ++i) {
+    ((int*)&host[o_bin])[i] = mem[i].bin;
+    real(o_dir, 2 * i, mem[i].e1);
+    real(o_dir, 2 * i + 1, mem[i].e3);
+    ((float*)&host[o_w])[i] = mem[i].w;
   }
-  double gl[32];
-  gauss_legendre16(gl, gl + 16);
-  CU(cudaMemcpyAsync(c->d_gl, gl, sizeof gl, cudaMemcpyHostToDevice, st));
+  for (size_t o = 0; o < o2; ++o) {
+    real(o_dT, o, dT[o]);
+    real(o_muq, o, muq[o]);
+  }
+  std::memcpy(&host[o_us], ustep.data(), o2 * sizeof(unsigned long long));
+  gauss_legendre16((double*)&host[o_gl], (double*)&host[o_gl] + 16);
+  if (blocked && c->n_cut >= sbim::kAheadLags) {   // shorter rings always wrap: copied row by row
+    CUtensorMap map;
+    if (const int rc = make_ring_map(*c, &map)) return rc;
+    std::memcpy(&host[o_map], &map, sizeof map);
+  }
+  cudaStream_t st = c->stream;
+  CU(cudaMemcpyAsync(c->d_arena, host.data(), filled, cudaMemcpyHostToDevice, st));
   CU(sbim::launch_table_build(c->d_tab64, c->d_tab32, c->tab_n, c->tab_h, c->eta, c->d_gl,
                               c->d_gl + 16, st));
   if (c->d_wts) CU(sbim::launch_weights64(step_args(c), c->d_wts, st));
-  if (const int rc = configure_conv(*c, kSpareBytes)) return rc == SBIM_ERR_CUDA ? rc : SBIM_ERR_OOM;
-  CU(cudaMemsetAsync(c->d_step, 0, sizeof(long long), st));
-  CU(cudaMemsetAsync(c->d_err, 0, sizeof(int), st));
+  if (blocked) {
+    CU(sbim::launch_ahead(step_args(c), c->prec, 0, c->halves, st));
+    CU(sbim::launch_ahead(step_args(c), c->prec, 3, c->halves, st));
+  }
+  if (const int rc = configure_conv(*c)) return rc == SBIM_ERR_CUDA ? rc : SBIM_ERR_OOM;
   CU(cudaStreamSynchronize(st));
 
   // cuFFT plans: batch of 3 components, [n3][n1] real <-> [n3][n1/2+1] complex
@@ -1122,7 +1115,7 @@ int sbim_set_conv_config(sbim_handle h, int variant, int lags_per_cta) {
       return fail(SBIM_ERR_CUDA, "kernel attributes: %s", cudaGetErrorString(e));
     }
   }
-  const int rc = configure_conv(*h, kSpareBytes);
+  const int rc = configure_conv(*h);
   if (rc != SBIM_OK) {
     h->variant = old_v; h->lags_per_cta = old_l; h->lc = old_lc; h->nchunks = old_nc;
     h->ahead_lc = old_alc; h->ahead_chunks = old_anc; h->use_ahead = old_ahead;
@@ -1150,7 +1143,7 @@ int sbim_set_conv_tile(sbim_handle h, int orbits_per_cta) {
       return fail(SBIM_ERR_CUDA, "kernel attributes: %s", cudaGetErrorString(e));
     }
   }
-  const int rc = configure_conv(*h, kSpareBytes);
+  const int rc = configure_conv(*h);
   if (rc != SBIM_OK) {
     h->tile = old_t; h->lc = old_lc; h->nchunks = old_nc;
     h->ahead_lc = old_alc; h->ahead_chunks = old_anc; h->use_ahead = old_ahead;
