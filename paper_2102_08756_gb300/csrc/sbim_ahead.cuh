@@ -468,15 +468,7 @@ __device__ __forceinline__ void near_member(const StepArgs& a, int T, int x) {
   const int b = a.bin[mi];
   const float2 e = reinterpret_cast<const float2*>(a.dir)[mi];
   float2 D[3];
-  if (b >= 0) {
-    const float2* uh = reinterpret_cast<const float2*>(a.uhat);
-    const float2 u1 = uh[b], u2 = uh[a.nbins + b], u3 = uh[2 * (long long)a.nbins + b];
-    D[0] = make_float2(e.x * u1.x + e.y * u3.x, e.x * u1.y + e.y * u3.y);
-    D[1] = u2;
-    D[2] = make_float2(-e.y * u1.x + e.x * u3.x, -e.y * u1.y + e.x * u3.y);
-  } else {
-    D[0] = D[1] = D[2] = make_float2(0.f, 0.f);
-  }
+  rotate_member(a, (int)mi, D);
   float2 R[3];   // as stored
 #pragma unroll
   for (int c = 0; c < 3; ++c)

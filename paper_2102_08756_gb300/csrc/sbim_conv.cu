@@ -124,143 +124,114 @@ conv_kernel(const StepArgs a) {
           KAHAN ? acc[g][k] - cmp[g][k] : acc[g][k];
 }
 
+// The chunk reduction and the modal operator for 32 records, one thread per member
+// (warp g holds member g of each record, so the partial sums are read coalesced).  The
+// chunk loop keeps four chunks' 10 sums in flight; each sum's order over the chunks,
+// and its compensation, are those of a loop over single chunks.  A thread per record
+// with all 40 sums left a 64^2 plane 5 blocks of 4 warps: 105 us of its 163 us step in
+// FP64 (16 chunks); with one per member the step takes 106 us.
+constexpr int kAsmRec = 32, kAsmThreads = kAsmRec * kMembers;
+
 template <class S, int KAHAN>
-__device__ __forceinline__ void assemble_orbit(const StepArgs& a, int o) {
+__device__ __forceinline__ void assemble_records(const StepArgs& a, int o0) {
   using R = typename S::real;
   using C = typename S::cplx;
+  __shared__ R shF[kMembers][6][kAsmRec];
+  __shared__ int shB[kMembers][kAsmRec];
+  const int r = threadIdx.x % kAsmRec, g = threadIdx.x / kAsmRec;
+  const int o = o0 + r;
   const long long n = *a.step;
   const int n_valid = (n + 1 < (long long)a.n_cut) ? (int)(n + 1) : a.n_cut;
-  const int m_end = a.tile_lmax ? min(n_valid, a.tile_lmax[o / kOrbitTile]) : n_valid;
+  const int m_end = a.tile_lmax ? min(n_valid, a.tile_lmax[o0 / kOrbitTile]) : n_valid;
   const int nch = (m_end + a.lc - 1) / a.lc;
   const long long orb = a.n_orb_pad;
-  const R muq0 = reinterpret_cast<const R*>(a.muq)[2 * o];
-  const R muq1 = reinterpret_cast<const R*>(a.muq)[2 * o + 1];
+  const R muq = reinterpret_cast<const R*>(a.muq)[2 * o + g / 2];
   const R sd = (R)a.side;
   const R inst = (R)(2.0 - a.eta);
-  const R* part = reinterpret_cast<const R*>(a.part);
-  C* fh = reinterpret_cast<C*>(a.fhat);
+  const R* part = reinterpret_cast<const R*>(a.part) + (long long)g * kFields * orb + o;
 
-  C D[3][4];
-  rotate_current(a, o, D);
+  C D[3];
+  rotate_member(a, o * kMembers + g, D);
 
-  // Chunk reduction of the 4 x kFields sums: the chunk loop is outermost so that
-  // each iteration issues 40 independent loads (each sum's own order over the
-  // chunks, and its compensation, are those of a per-sum loop).
-  R sum[4][kFields], cmp[4][kFields];
+  R v[kFields], cmp[kFields];
 #pragma unroll
-  for (int g = 0; g < 4; ++g)
+  for (int k = 0; k < kFields; ++k) v[k] = cmp[k] = (R)0;
+  constexpr int W = 4;
+  for (int c0 = 0; c0 < nch; c0 += W) {
+    R x[W][kFields];
 #pragma unroll
-    for (int k = 0; k < kFields; ++k) { sum[g][k] = (R)0; cmp[g][k] = (R)0; }
-  auto load_chunk = [&](int ch, R (&x)[4][kFields]) {
+    for (int i = 0; i < W; ++i)
+      if (c0 + i < nch)
 #pragma unroll
-    for (int g = 0; g < 4; ++g)
+        for (int k = 0; k < kFields; ++k)
+          x[i][k] = part[((long long)(c0 + i) * (kMembers * kFields) + k) * orb];
 #pragma unroll
-      for (int k = 0; k < kFields; ++k)
-        x[g][k] = part[((long long)ch * (4 * kFields) + g * kFields + k) * orb + o];
-  };
-  if constexpr (KAHAN) {
-    for (int ch = 0; ch < nch; ++ch) {
-      R x[4][kFields];
-      load_chunk(ch, x);
-#pragma unroll
-      for (int g = 0; g < 4; ++g)
+    for (int i = 0; i < W; ++i)
+      if (c0 + i < nch)
 #pragma unroll
         for (int k = 0; k < kFields; ++k) {
-          const R y = x[g][k] - cmp[g][k];
-          const R t = sum[g][k] + y;
-          cmp[g][k] = (t - sum[g][k]) - y;
-          sum[g][k] = t;
+          if constexpr (KAHAN) {
+            const R y = x[i][k] - cmp[k];
+            const R t = v[k] + y;
+            cmp[k] = (t - v[k]) - y;
+            v[k] = t;
+          } else {
+            v[k] += x[i][k];
+          }
         }
-    }
-  } else if constexpr (sizeof(R) == 8) {
-    // FP64 sums (their step is bound by the FP64 pipe): one chunk at a time
-    for (int ch = 0; ch < nch; ++ch) {
-      R x[4][kFields];
-      load_chunk(ch, x);
-#pragma unroll
-      for (int g = 0; g < 4; ++g)
-#pragma unroll
-        for (int k = 0; k < kFields; ++k) sum[g][k] += x[g][k];
-    }
-  } else if (nch > 0) {
-    // Plain float sums: the next chunk's 40 loads are issued before this chunk's
-    // adds (left to the compiler, the uncompensated loop kept few loads in flight
-    // and ran at a third of the compensated one's rate on GB300).
-    R x[4][kFields], xn[4][kFields];
-    load_chunk(0, x);
-    for (int ch = 0; ch < nch; ++ch) {
-      const bool more = ch + 1 < nch;
-      if (more) load_chunk(ch + 1, xn);
-#pragma unroll
-      for (int g = 0; g < 4; ++g)
-#pragma unroll
-        for (int k = 0; k < kFields; ++k) sum[g][k] += x[g][k];
-      if (more)
-#pragma unroll
-        for (int g = 0; g < 4; ++g)
-#pragma unroll
-          for (int k = 0; k < kFields; ++k) x[g][k] = xn[g][k];
-    }
   }
 
-  int pend = -1;
-  C P1, P2, P3;
+  const int b = a.bin[o * kMembers + g];
+  const C dxi = D[0], d2 = D[1];
+  // F_xi = -side mu q C11 + i mu q [(2 - eta) D_2 + C12a]
+  const R bxr = inst * d2.x + v[6], bxi = inst * d2.y + v[7];
+  C fxi, fp, f2;
+  fxi.x = muq * (-sd * v[0] - bxi);
+  fxi.y = muq * (-sd * v[1] + bxr);
+  // F_perp = -side mu q C33
+  fp.x = -sd * muq * v[2];
+  fp.y = -sd * muq * v[3];
+  // F_2 = -i mu q [(2 - eta) D_xi + C12b] - side mu q C22
+  const R b2r = inst * dxi.x + v[8], b2i = inst * dxi.y + v[9];
+  f2.x = muq * (b2i - sd * v[4]);
+  f2.y = muq * (-b2r - sd * v[5]);
+  const C e = reinterpret_cast<const C*>(a.dir)[o * kMembers + g];
+  const R wsc = (R)a.wout[o * kMembers + g] * (R)a.inv_n;
+  const R F[6] = {wsc * (e.x * fxi.x - e.y * fp.x), wsc * (e.x * fxi.y - e.y * fp.y), f2.x * wsc,
+                  f2.y * wsc, wsc * (e.y * fxi.x + e.x * fp.x), wsc * (e.y * fxi.y + e.x * fp.y)};
+  shB[g][r] = b;
 #pragma unroll
-  for (int g = 0; g < 4; ++g) {
-    const int b = a.bin[o * 4 + g];
-    if (b < 0) continue;
-    const R muq = g < 2 ? muq0 : muq1;
-    const R* v = sum[g];
-    const C dxi = D[0][g], d2 = D[1][g];
-    // F_xi = -side mu q C11 + i mu q [(2 - eta) D_2 + C12a]
-    const R bxr = inst * d2.x + v[6], bxi = inst * d2.y + v[7];
-    C fxi, fp, f2;
-    fxi.x = muq * (-sd * v[0] - bxi);
-    fxi.y = muq * (-sd * v[1] + bxr);
-    // F_perp = -side mu q C33
-    fp.x = -sd * muq * v[2];
-    fp.y = -sd * muq * v[3];
-    // F_2 = -i mu q [(2 - eta) D_xi + C12b] - side mu q C22
-    const R b2r = inst * dxi.x + v[8], b2i = inst * dxi.y + v[9];
-    f2.x = muq * (b2i - sd * v[4]);
-    f2.y = muq * (-b2r - sd * v[5]);
-    const C e = reinterpret_cast<const C*>(a.dir)[o * 4 + g];
-    const R e1 = e.x, e3 = e.y;
-    const R wsc = (R)a.wout[o * 4 + g] * (R)a.inv_n;
-    C f1, f3;
-    f1.x = wsc * (e1 * fxi.x - e3 * fp.x); f1.y = wsc * (e1 * fxi.y - e3 * fp.y);
-    f3.x = wsc * (e3 * fxi.x + e1 * fp.x); f3.y = wsc * (e3 * fxi.y + e1 * fp.y);
-    f2.x *= wsc; f2.y *= wsc;
-    if (b == pend) {
-      P1.x += f1.x; P1.y += f1.y; P2.x += f2.x; P2.y += f2.y; P3.x += f3.x; P3.y += f3.y;
-    } else {
-      if (pend >= 0) {
-        fh[pend] = P1; fh[a.nbins + pend] = P2; fh[2 * (long long)a.nbins + pend] = P3;
-      }
-      pend = b; P1 = f1; P2 = f2; P3 = f3;
-    }
-  }
-  if (pend >= 0) {
-    fh[pend] = P1; fh[a.nbins + pend] = P2; fh[2 * (long long)a.nbins + pend] = P3;
-  }
+  for (int k = 0; k < 6; ++k) shF[g][k][r] = F[k];
+  __syncthreads();
+  // the virtual members of one Nyquist bin are neighbours: the first adds them up
+  if (b < 0 || (g > 0 && shB[g - 1][r] == b)) return;
+  R G[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) G[k] = F[k];
+  for (int h = g + 1; h < kMembers && shB[h][r] == b; ++h)
+#pragma unroll
+    for (int k = 0; k < 6; ++k) G[k] += shF[h][k][r];
+  C* fh = reinterpret_cast<C*>(a.fhat);
+  fh[b] = make_cplx(G[0], G[1]);
+  fh[a.nbins + b] = make_cplx(G[2], G[3]);
+  fh[2 * (long long)a.nbins + b] = make_cplx(G[4], G[5]);
 }
 
 template <class S, int KAHAN>
-__global__ void __launch_bounds__(kOrbitTile) assemble_kernel(const StepArgs a) {
-  const int o = blockIdx.x * kOrbitTile + threadIdx.x;
-  if (o >= a.n_orb_pad) return;
-  assemble_orbit<S, KAHAN>(a, o);
+__global__ void __launch_bounds__(kAsmThreads) assemble_kernel(const StepArgs a) {
+  assemble_records<S, KAHAN>(a, blockIdx.x * kAsmRec);
 }
 
-// One CTA per orbit tile of every member of a batch.
+// The same over the orbit tiles of every member of a batch.
 template <class S, int KAHAN>
-__global__ void __launch_bounds__(kOrbitTile)
+__global__ void __launch_bounds__(kAsmThreads)
 assemble_batch_kernel(const StepArgs* __restrict__ args, const int* __restrict__ tile_prefix, int nb) {
-  const int t = blockIdx.x;
+  constexpr int SUB = kOrbitTile / kAsmRec;
+  const int t = blockIdx.x / SUB;
   int s = 0;
   while (s + 1 < nb && tile_prefix[s + 1] <= t) ++s;
   const StepArgs a = args[s];
-  assemble_orbit<S, KAHAN>(a, (t - tile_prefix[s]) * kOrbitTile + threadIdx.x);
+  assemble_records<S, KAHAN>(a, (t - tile_prefix[s]) * kOrbitTile + (blockIdx.x % SUB) * kAsmRec);
 }
 
 template <class R>
@@ -386,8 +357,7 @@ cudaError_t conv_dispatch(const StepArgs& a, cudaStream_t st) {
 
 template <class S, int KAHAN>
 cudaError_t assemble_dispatch(const StepArgs& a, cudaStream_t st) {
-  const int grid = a.n_orb_pad / kOrbitTile;
-  assemble_kernel<S, KAHAN><<<grid, kOrbitTile, 0, st>>>(a);
+  assemble_kernel<S, KAHAN><<<a.n_orb_pad / kAsmRec, kAsmThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -425,7 +395,8 @@ cudaError_t launch_assemble(const StepArgs& a, int precision, int kahan, cudaStr
 
 template <class S, int KAHAN>
 cudaError_t assemble_batch_dispatch(const BatchLaunch& b, int tiles, cudaStream_t st) {
-  assemble_batch_kernel<S, KAHAN><<<tiles, kOrbitTile, 0, st>>>(b.args, b.tile_prefix, b.nb);
+  assemble_batch_kernel<S, KAHAN><<<tiles * (kOrbitTile / kAsmRec), kAsmThreads, 0, st>>>(
+      b.args, b.tile_prefix, b.nb);
   return cudaGetLastError();
 }
 

@@ -247,6 +247,25 @@ template <> __device__ __forceinline__ double2 cmake<double2>(double re, double 
   return make_double2(re, im);
 }
 
+__device__ __forceinline__ float2 make_cplx(float re, float im) { return make_float2(re, im); }
+__device__ __forceinline__ double2 make_cplx(double re, double im) { return make_double2(re, im); }
+
+// Current spectra of one member rotated into (xi, 2, perp); zero for padding.
+template <class C>
+__device__ __forceinline__ void rotate_member(const StepArgs& a, int i, C (&D)[3]) {
+  using R = typename RealOf<C>::type;
+  const C* uh = reinterpret_cast<const C*>(a.uhat);
+  const int b = a.bin[i];
+  D[0] = D[1] = D[2] = cmake<C>(0, 0);
+  if (b < 0) return;
+  const C e = reinterpret_cast<const C*>(a.dir)[i];
+  const R e1 = e.x, e3 = e.y;
+  const C u1 = uh[b], u2 = uh[a.nbins + b], u3 = uh[2 * (long long)a.nbins + b];
+  D[0].x = e1 * u1.x + e3 * u3.x;  D[0].y = e1 * u1.y + e3 * u3.y;
+  D[1] = u2;
+  D[2].x = -e3 * u1.x + e1 * u3.x; D[2].y = -e3 * u1.y + e1 * u3.y;
+}
+
 // Current spectra of the orbit's members rotated into (xi, 2, perp).
 template <class C>
 __device__ __forceinline__ void rotate_current(const StepArgs& a, int o, C (&D)[3][4]) {
