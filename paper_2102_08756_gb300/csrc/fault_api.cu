@@ -30,6 +30,7 @@ struct sbim_fault_ctx {
   double cs = 0, cp = 0, rho = 0, dt = 0;
   cudaStream_t stream = nullptr;
   sbim_handle up = nullptr, lo = nullptr;
+  sbim::PairStreams pair;    // the lower half-space's stages run beside the upper's
   void* u = nullptr;         // [2][3][n3][n1]: face 0 upper (+), face 1 lower (-)
   void* v = nullptr;
   void* u_pred = nullptr;    // [2][3][n3][n1] predictor displacement
@@ -184,6 +185,7 @@ void release(sbim_fault_ctx* c) {
   if (!c) return;
   sbim_destroy(c->up);
   sbim_destroy(c->lo);
+  sbim::pair_release(c->pair);
   for (void* p : {c->u, c->v, c->u_pred, c->v_pred, c->s_up, c->s_lo, c->zero, c->mu_s, c->tau0, c->traction, c->rate})
     if (p) cudaFree(p);
   delete c;
@@ -196,13 +198,14 @@ template <class R>
 int solve(sbim_fault_ctx* h, const R* u, R* v_out, bool again) {
   const long long np = h->plane();
   const size_t face = 3 * (size_t)np;
-  auto eval = again ? sbim_step_repeat : sbim_step;
-  int rc = eval(h->up, u, h->zero, h->s_up);
-  if (rc != SBIM_OK) return rc;
+  const int kind = again ? 2 : 0;
+  if (!h->symmetric) FCU(sbim::pair_begin(h->pair, h->stream));
+  int rc = sbim::handle_step_on(h->up, u, h->zero, h->s_up, kind, h->stream);
   if (!h->symmetric) {
-    rc = eval(h->lo, u + face, h->zero, h->s_lo);
-    if (rc != SBIM_OK) return rc;
+    if (rc == SBIM_OK) rc = sbim::handle_step_on(h->lo, u + face, h->zero, h->s_lo, kind, h->pair.side);
+    FCU(sbim::pair_end(h->pair, h->stream));
   }
+  if (rc != SBIM_OK) return rc;
   const R mu = (R)(h->rho * h->cs * h->cs);
   const R z_s = mu / (R)h->cs, z_p = z_s * (R)(h->cp / h->cs);
   Law<R> law{(const R*)h->mu_s, (const R*)h->tau0, (R)h->mu_k, (R)h->Dc, (R)h->sigma0,
@@ -274,6 +277,8 @@ int sbim_fault_create(sbim_fault* out, int n1, int n3, double L1, double L3, dou
   const int kahan = precision == SBIM_BF16 ? 0 : 1;
   if (rc == SBIM_OK)
     rc = sbim_create(&c->up, n1, n3, L1, L3, cs, cp, rho, dt, n_cut, +1, precision, kahan, stream);
+  if (rc == SBIM_OK && !c->symmetric && sbim::pair_init(c->pair) != cudaSuccess)
+    rc = ffail(SBIM_ERR_CUDA, "side stream");
   if (rc == SBIM_OK && !c->symmetric)
     rc = sbim_create(&c->lo, n1, n3, L1, L3, cs, cp, rho, dt, n_cut, -1, precision, kahan, stream);
   if (rc == SBIM_OK && cudaStreamSynchronize(c->stream) != cudaSuccess) rc = ffail(SBIM_ERR_CUDA, "sync");

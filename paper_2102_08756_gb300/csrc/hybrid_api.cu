@@ -23,6 +23,7 @@ struct sbim_hybrid_ctx {
   double h = 0, cs = 0, cp = 0, rho = 0, dt = 0;
   cudaStream_t stream = nullptr;
   sbim_handle top = nullptr, bot = nullptr;
+  sbim::PairStreams pair;   // the bottom half-space's stages run beside the top's
   void* u = nullptr;
   void* v = nullptr;
   void* a = nullptr;
@@ -35,7 +36,7 @@ struct sbim_hybrid_ctx {
   sbim::fem::Stencil<float> stencil_f;
   sbim::fem::Stencil<double> stencil_d;
   void* adj[8] = {};        // reverse sweep: un, vp, af, lun, lvp, lan, lao, lF
-  void* adjp[4] = {};       // tb_top, tb_bot, ub, vb ([3][n3][n1])
+  void* adjp[6] = {};       // tb_top, tb_bot, ub, vb (top), ub, vb (bottom) ([3][n3][n1])
   double mu_k = 0, Dc = 1, sigma0 = 0;
   bool have_law = false;
   long long n = 0;
@@ -207,6 +208,18 @@ int stage_finish(sbim_hybrid_ctx* c, const void* src) {
   return stage_finish<R>(c, src, c->stream);
 }
 
+// One step (kind 0) or transposed step (1) of both half-spaces, side by side: each is
+// a chain of short kernels that leave most of the chip idle on small grids.
+int half_spaces(sbim_hybrid_ctx* c, int kind, const void* in_t, const void* aux_t, void* out_t,
+                const void* in_b, const void* aux_b, void* out_b) {
+  HCU(sbim::pair_begin(c->pair, c->stream));
+  int rc = sbim::handle_step_on(c->top, in_t, aux_t, out_t, kind, c->stream);
+  // (joined after an error too: the side stream must not be left forked)
+  if (rc == SBIM_OK) rc = sbim::handle_step_on(c->bot, in_b, aux_b, out_b, kind, c->pair.side);
+  HCU(sbim::pair_end(c->pair, c->stream));
+  return rc;
+}
+
 template <class R>
 int step_impl(sbim_hybrid_ctx* c, const void* src) {
   int rc = stage_predict<R>(c);
@@ -214,8 +227,7 @@ int step_impl(sbim_hybrid_ctx* c, const void* src) {
   if (c->boundaries) {
     const void *ut, *vt, *ub, *vb;
     boundary_ptrs(c, &ut, &vt, &ub, &vb);
-    rc = sbim_step(c->top, ut, vt, c->tau_top);
-    if (rc == SBIM_OK) rc = sbim_step(c->bot, ub, vb, c->tau_bot);
+    rc = half_spaces(c, 0, ut, vt, c->tau_top, ub, vb, c->tau_bot);
     if (rc != SBIM_OK) return rc;
   }
   rc = stage_finish<R>(c, src);
@@ -272,14 +284,14 @@ int adjoint_impl(sbim_hybrid_ctx* c, const void* u, const void* v, const void* a
     const long long lay = 3 * c->plane();
     R* ub = (R*)c->adjp[2];
     R* vb = (R*)c->adjp[3];
-    int rc = sbim_step_adjoint(c->top, j.tb_top, ub, vb);
+    R* ub2 = (R*)c->adjp[4];
+    R* vb2 = (R*)c->adjp[5];
+    const int rc = half_spaces(c, 1, j.tb_top, vb, ub, j.tb_bot, vb2, ub2);
     if (rc != SBIM_OK) return rc;
     HCU(sbim::fem::layer_add<R>(j.lun + (c->L - 1) * lay, ub, lay, st));
     HCU(sbim::fem::layer_add<R>(j.lvp + (c->L - 1) * lay, vb, lay, st));
-    rc = sbim_step_adjoint(c->bot, j.tb_bot, ub, vb);
-    if (rc != SBIM_OK) return rc;
-    HCU(sbim::fem::layer_add<R>(j.lun, ub, lay, st));
-    HCU(sbim::fem::layer_add<R>(j.lvp, vb, lay, st));
+    HCU(sbim::fem::layer_add<R>(j.lun, ub2, lay, st));
+    HCU(sbim::fem::layer_add<R>(j.lvp, vb2, lay, st));
   }
   HCU(sbim::fem::adjoint_stages<R>(j, g, stencil_of(c, R()), fa, 5, st));
   ++c->n;
@@ -290,6 +302,7 @@ void hrelease(sbim_hybrid_ctx* c) {
   if (!c) return;
   sbim_destroy(c->top);
   sbim_destroy(c->bot);
+  sbim::pair_release(c->pair);
   void* p[] = {c->u,     c->v,     c->a,        c->an,      c->tau_top,
                c->tau_bot, c->mu_s, c->tau0, c->traction};
   for (void* x : p)
@@ -333,6 +346,9 @@ int sbim_hybrid_create(sbim_hybrid* out, int n1, int n2, int n3, double h, doubl
   alloc(&c->u, fb); alloc(&c->v, fb); alloc(&c->a, fb); alloc(&c->an, fb);
   alloc(&c->tau_top, pb); alloc(&c->tau_bot, pb); alloc(&c->traction, pb);
   alloc(&c->mu_s, c->plane() * c->rs); alloc(&c->tau0, c->plane() * c->rs);
+  if (rc == SBIM_OK && c->boundaries) {
+    if (sbim::pair_init(c->pair) != cudaSuccess) rc = hfail(SBIM_ERR_CUDA, "side stream");
+  }
   if (rc == SBIM_OK && c->boundaries) {
     rc = sbim_create(&c->top, n1, n3, n1 * h, n3 * h, cs, cp, rho, dt, n_cut, +1, precision, 1, stream);
     if (rc == SBIM_OK)

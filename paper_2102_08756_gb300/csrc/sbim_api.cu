@@ -161,6 +161,7 @@ struct sbim_ctx {
   int* h_err = nullptr;  // pinned copy of the error word, read with tau by sbim_step_host
   cudaStream_t io_stream = nullptr;          // sbim_step_host: copies in + forward FFT
   cudaEvent_t io_fork = nullptr, io_join = nullptr;
+  sbim::PairStreams sums;                    // the block sums, beside the forward transform
   cufftHandle plan_fwd = 0, plan_inv = 0;
   bool have_fwd = false, have_inv = false;
 
@@ -518,6 +519,7 @@ void release(sbim_ctx* c) {
   if (c->io_fork) cudaEventDestroy(c->io_fork);
   if (c->io_join) cudaEventDestroy(c->io_join);
   if (c->io_stream) cudaStreamDestroy(c->io_stream);
+  sbim::pair_release(c->sums);
   if (c->h_err) cudaFreeHost(c->h_err);
   delete c;
 }
@@ -660,6 +662,7 @@ int create_impl(sbim_ctx* c) {
                               c->d_gl + 16, st));
   if (c->d_wts) CU(sbim::launch_weights64(step_args(c), c->d_wts, st));
   if (blocked) {
+    CU(sbim::pair_init(c->sums));
     CU(sbim::launch_ahead(step_args(c), c->prec, 0, c->halves, st));
     CU(sbim::launch_ahead(step_args(c), c->prec, 3, c->halves, st));
   }
@@ -740,13 +743,14 @@ int handle_fft_forward(sbim_handle c, const void* u, cudaStream_t st) {
   return SBIM_OK;
 }
 
-int handle_fft_inverse(sbim_handle c, cudaStream_t st) {
+int handle_fft_inverse(sbim_handle c, cudaStream_t st, void* out) {
+  if (!out) out = c->d_s;
   if (st != c->stream) CF(cufftSetStream(c->plan_inv, st));
   cufftResult r;
   if (c->prec == SBIM_FP64)
-    r = cufftExecZ2D(c->plan_inv, (cufftDoubleComplex*)c->d_fhat, (cufftDoubleReal*)c->d_s);
+    r = cufftExecZ2D(c->plan_inv, (cufftDoubleComplex*)c->d_fhat, (cufftDoubleReal*)out);
   else
-    r = cufftExecC2R(c->plan_inv, (cufftComplex*)c->d_fhat, (cufftReal*)c->d_s);
+    r = cufftExecC2R(c->plan_inv, (cufftComplex*)c->d_fhat, (cufftReal*)out);
   if (st != c->stream) CF(cufftSetStream(c->plan_inv, c->stream));
   CF(r);
   return SBIM_OK;
@@ -855,23 +859,32 @@ namespace {
 // The opt-in input check: a reduction over the step's inputs, read back on the
 // host before anything of the step is enqueued, so a refused step leaves the
 // handle exactly as it was.
-int check_inputs(sbim_ctx* c, const void* a, const void* b) {
-  CU(sbim::launch_nonfinite_check(c->prec, a, b, (long long)c->field_elems(), c->d_nonfinite,
-                                  c->stream));
+int check_inputs(sbim_ctx* c, const void* a, const void* b, cudaStream_t st) {
+  CU(sbim::launch_nonfinite_check(c->prec, a, b, (long long)c->field_elems(), c->d_nonfinite, st));
   int flag = 0;
-  CU(cudaMemcpyAsync(&flag, c->d_nonfinite, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  CU(cudaStreamSynchronize(c->stream));
+  CU(cudaMemcpyAsync(&flag, c->d_nonfinite, sizeof(int), cudaMemcpyDeviceToHost, st));
+  CU(cudaStreamSynchronize(st));
   if (flag)
     return fail(SBIM_ERR_NONFINITE, "non-finite value (NaN or infinity) in the step's input; "
                                     "the step was not taken");
   return SBIM_OK;
 }
 
+// The block sums that are due, beside the forward transform on `st`: they need only
+// the stored history (a step of 128^2 x 48 is a chain of short kernels, 46.9 us with
+// the sums in it against 37.5).
+int fork_sums(sbim_ctx* c, const sbim::StepArgs& a, cudaStream_t st) {
+  CU(sbim::pair_begin(c->sums, st));
+  CU(sbim::launch_ahead(a, c->prec, 1, c->halves, c->sums.side));
+  CU(cudaEventRecord(c->sums.join, c->sums.side));
+  return SBIM_OK;
+}
+
+// (On `st`, which is the handle's stream or one forked from it and joined to it.)
 int run_step(sbim_ctx* c, const void* in, const void* aux, void* out, bool adjoint,
-             bool repeat = false) {
-  cudaStream_t st = c->stream;
+             bool repeat, cudaStream_t st) {
   if (c->check_finite) {
-    const int rc = check_inputs(c, in, adjoint ? nullptr : aux);
+    const int rc = check_inputs(c, in, adjoint ? nullptr : aux, st);
     if (rc != SBIM_OK) return rc;
   }
   if (repeat) {                     // back to the level being re-evaluated
@@ -887,15 +900,18 @@ int run_step(sbim_ctx* c, const void* in, const void* aux, void* out, bool adjoi
     e = &c->ev[(c->prof_issued % kProfRing) * kProfEvents];
     CU(cudaEventRecord(e[0], st));
   }
-  if (c->prec == SBIM_FP64)
-    CF(cufftExecD2Z(c->plan_fwd, (cufftDoubleReal*)in, (cufftDoubleComplex*)c->d_uhat));
-  else
-    CF(cufftExecR2C(c->plan_fwd, (cufftReal*)in, (cufftComplex*)c->d_uhat));
-  if (e) CU(cudaEventRecord(e[1], st));
   const sbim::StepArgs a = step_args(c);
+  // (a repeated level finds its block sums formed: they end before the block)
+  const bool sums = c->use_ahead && !repeat, beside = sums && !e;
+  if (beside)
+    if (const int rc = fork_sums(c, a, st)) return rc;
+  if (const int rc = sbim::handle_fft_forward(c, in, st)) return rc;
+  if (e) CU(cudaEventRecord(e[1], st));
+  if (beside)
+    CU(cudaStreamWaitEvent(st, c->sums.join, 0));
+  else if (sums)
+    CU(sbim::launch_ahead(a, c->prec, 1, c->halves, st));
   if (c->use_ahead) {
-    // a repeated level finds its block sums formed: they end before the block
-    if (!repeat) CU(sbim::launch_ahead(a, c->prec, 1, c->halves, st));
   } else if (repeat)
     CU(sbim::launch_repeat_lag0(a, c->prec, st));
   else if (c->variant >= 1)
@@ -908,11 +924,7 @@ int run_step(sbim_ctx* c, const void* in, const void* aux, void* out, bool adjoi
   else
     CU(sbim::launch_assemble(a, c->prec, c->kahan, st));
   if (e) CU(cudaEventRecord(e[3], st));
-  void* s_dst = adjoint ? out : c->d_s;
-  if (c->prec == SBIM_FP64)
-    CF(cufftExecZ2D(c->plan_inv, (cufftDoubleComplex*)c->d_fhat, (cufftDoubleReal*)s_dst));
-  else
-    CF(cufftExecC2R(c->plan_inv, (cufftComplex*)c->d_fhat, (cufftReal*)s_dst));
+  if (const int rc = sbim::handle_fft_inverse(c, st, adjoint ? out : c->d_s)) return rc;
   if (e) CU(cudaEventRecord(e[4], st));
   const double k = c->side * c->mu / c->cs;
   const double coef[3] = {k, k * c->eta, k};
@@ -930,6 +942,38 @@ int run_step(sbim_ctx* c, const void* in, const void* aux, void* out, bool adjoi
   c->can_repeat = !adjoint;
   return SBIM_OK;
 }
+
+}  // namespace
+
+namespace sbim {
+cudaError_t pair_init(PairStreams& p) {
+  cudaError_t e = cudaStreamCreateWithFlags(&p.side, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p.fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p.join, cudaEventDisableTiming);
+  return e;
+}
+cudaError_t pair_begin(PairStreams& p, cudaStream_t st) {
+  const cudaError_t e = cudaEventRecord(p.fork, st);
+  return e == cudaSuccess ? cudaStreamWaitEvent(p.side, p.fork, 0) : e;
+}
+cudaError_t pair_end(PairStreams& p, cudaStream_t st) {
+  const cudaError_t e = cudaEventRecord(p.join, p.side);
+  return e == cudaSuccess ? cudaStreamWaitEvent(st, p.join, 0) : e;
+}
+void pair_release(PairStreams& p) {
+  if (p.fork) cudaEventDestroy(p.fork);
+  if (p.join) cudaEventDestroy(p.join);
+  if (p.side) cudaStreamDestroy(p.side);
+}
+
+int handle_step_on(sbim_handle c, const void* in, const void* aux, void* out, int kind, cudaStream_t st) {
+  if (kind == 2 && (!c->can_repeat || c->n == 0))
+    return fail(SBIM_ERR_STATE, "nothing to repeat on this handle");
+  return run_step(c, in, aux, out, kind == 1, kind == 2, st);
+}
+}  // namespace sbim
+
+namespace {
 
 // The device error word as read after the stream drained: clears it and
 // reports SBIM_ERR_TIMEOUT when a bounded wait gave up.
@@ -949,7 +993,7 @@ extern "C" {
 int sbim_step(sbim_handle h, const void* u, const void* v, void* tau) {
   if (!h) return fail(SBIM_ERR_ARG, "NULL handle");
   if (!u || !v || !tau) return fail(SBIM_ERR_ARG, "NULL field pointer");
-  return run_step(h, u, v, tau, false);
+  return run_step(h, u, v, tau, false, false, h->stream);
 }
 
 int sbim_step_repeat(sbim_handle h, const void* u, const void* v, void* tau) {
@@ -958,7 +1002,7 @@ int sbim_step_repeat(sbim_handle h, const void* u, const void* v, void* tau) {
   if (!h->can_repeat || h->n == 0)
     return fail(SBIM_ERR_STATE, "sbim_step_repeat needs a preceding sbim_step on this handle "
                                 "(with no other call that changes its state in between)");
-  return run_step(h, u, v, tau, false, true);
+  return run_step(h, u, v, tau, false, true, h->stream);
 }
 
 int sbim_step_adjoint(sbim_handle h, const void* tau_bar, void* u_bar, void* v_bar) {
@@ -966,7 +1010,7 @@ int sbim_step_adjoint(sbim_handle h, const void* tau_bar, void* u_bar, void* v_b
   if (!tau_bar || !u_bar || !v_bar) return fail(SBIM_ERR_ARG, "NULL field pointer");
   if (tau_bar == u_bar || tau_bar == v_bar || u_bar == v_bar)
     return fail(SBIM_ERR_ARG, "tau_bar, u_bar and v_bar must be distinct buffers");
-  return run_step(h, tau_bar, v_bar, u_bar, true);
+  return run_step(h, tau_bar, v_bar, u_bar, true, false, h->stream);
 }
 
 int sbim_step_host(sbim_handle h, const void* u, const void* v, void* tau) {

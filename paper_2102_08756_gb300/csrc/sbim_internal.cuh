@@ -157,7 +157,19 @@ void set_last_error(const char* msg);
 // several handles (each returns an sbim_status).
 StepArgs handle_step_args(sbim_handle h);
 int handle_fft_forward(sbim_handle h, const void* u, cudaStream_t st);
-int handle_fft_inverse(sbim_handle h, cudaStream_t st);
+int handle_fft_inverse(sbim_handle h, cudaStream_t st, void* out = nullptr);   // default: the handle's buffer
+// One sbim_step (kind 0), sbim_step_adjoint (1: in = tau_bar, aux = v_bar, out = u_bar)
+// or sbim_step_repeat (2) on a stream forked from the handle's and joined to it.
+int handle_step_on(sbim_handle h, const void* in, const void* aux, void* out, int kind, cudaStream_t st);
+// A side stream for the second of two half-spaces that step side by side.
+struct PairStreams {
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
+};
+cudaError_t pair_init(PairStreams& p);                     // at creation: steps may be captured
+cudaError_t pair_begin(PairStreams& p, cudaStream_t st);   // the side stream follows st
+cudaError_t pair_end(PairStreams& p, cudaStream_t st);     // st follows the side stream
+void pair_release(PairStreams& p);
 int handle_epilogue(sbim_handle h, const void* v, void* tau, cudaStream_t st);
 void handle_advance(sbim_handle h);
 bool handle_uses_ahead(sbim_handle h);
