@@ -70,10 +70,14 @@ template <class R> cudaError_t predict(R* u, R* v, const R* a, long long n, R dt
 template <class R>
 cudaError_t force(const R* u, R* an, const MeshArgs& g, const Stencil<R>& S, const R* tau_top,
                   const R* tau_bot, const R* src, cudaStream_t st);
+// Forces, and the velocity correction of the node layers off the split plane; the
+// split layers' accelerations are left in `an` for fault(), which corrects those two.
 template <class R>
-cudaError_t fault(const R* u, const R* vpred, const R* a, R* an, const MeshArgs& g,
+cudaError_t force_correct(const R* u, R* v, R* a, R* an, const MeshArgs& g, const Stencil<R>& S,
+                          const R* tau_top, const R* tau_bot, const R* src, R dt, cudaStream_t st);
+template <class R>
+cudaError_t fault(const R* u, R* vpred, R* a, const R* an, const MeshArgs& g,
                   const FaultArgs<R>& fa, R dt, int weld, cudaStream_t st);
-template <class R> cudaError_t correct(R* v, R* a, const R* an, long long n, R dt, cudaStream_t st);
 template <class R>
 cudaError_t fault_fields(const R* u, const R* v, const MeshArgs& g, R* slip, R* rate,
                          cudaStream_t st);

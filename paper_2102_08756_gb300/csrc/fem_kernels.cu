@@ -150,11 +150,12 @@ __device__ __forceinline__ void apply_side(const Stencil<R>& S, const Window<R>&
 // before the barrier of layer l-1), and is waited for one layer later.  A
 // layer's element blocks below (down) and above (up) exist unless they cross
 // the split fault plane or the slab's faces.  Per node of a column inside the
-// grid, epi(l, q0, down, up, F) finishes; threads of columns outside it still
-// copy and synchronise.
-template <class R, class Epi>
+// grid, pre(l, q0) runs before the layer's arithmetic (loads that epi needs) and
+// epi(l, q0, down, up, F) finishes; threads of columns outside it still copy and
+// synchronise.
+template <class R, class Pre, class Epi>
 __device__ __forceinline__ void stencil_columns(const R* __restrict__ x, const MeshArgs& g,
-                                                const Stencil<R>& S, Epi epi) {
+                                                const Stencil<R>& S, Pre pre, Epi epi) {
   __shared__ __align__(16) R tiles[kStages][kLayerTile];
   const int tx = threadIdx.x % kTX, tz = threadIdx.x / kTX;
   const int x0 = blockIdx.x * kTX, z0 = blockIdx.y * kTZ;
@@ -197,6 +198,7 @@ __device__ __forceinline__ void stencil_columns(const R* __restrict__ x, const M
     const bool down = l > 0 && !(g.fault && l == g.f + 1);
     const bool up = l < g.L - 1 && !(g.fault && l == g.f);
     R F[3] = {(R)0, (R)0, (R)0};
+    if (inside) pre(l, q0);
     if (down) apply_side<0>(S, prev, cur, F);
     cp_async_wait<1>();    // layer l+1 landed (layer l+2 may still be in flight)
     __syncthreads();
@@ -215,18 +217,35 @@ __device__ __forceinline__ void stencil_columns(const R* __restrict__ x, const M
 
 // an = (-K u + f_boundary) / m: the acceleration without fault traction.
 // f_boundary = +A tau_top on the top layer, -A tau_bot on the bottom layer.
-template <class R>
+// CORRECT: node layers off the split plane take their velocity correction
+// v = v_pred + dt/2 (a_{t+1} - a_t), a = a_{t+1} here (Eq. (fecorr)); only the split
+// layers' accelerations go to `an`, for the fault kernel.  As a pass of its own the
+// correction read back every acceleration and took 43 us at 512 x 18 x 512, of 143
+// with predictor and forces; fused with the forces the two take 78 us instead of 99.
+template <class R, bool CORRECT>
 __global__ void __launch_bounds__(kColThreads) force_kernel(const R* __restrict__ u, R* __restrict__ an,
                                                     MeshArgs g, const __grid_constant__ Stencil<R> S,
                                                     const R* __restrict__ tau_top,
                                                     const R* __restrict__ tau_bot,
-                                                    const R* __restrict__ src) {
+                                                    const R* __restrict__ src, R* __restrict__ v,
+                                                    R* __restrict__ a, R dt) {
   const long long plane = (long long)g.n1 * g.n3;
   // 1 / lumped mass of a node with elements on both sides or on one (every node
   // of a slab has elements on at least one side), converted and divided once
   const R hm = (R)g.half_mass;
   const R inv_m1 = (R)1 / hm, inv_m2 = (R)1 / (hm + hm);
-  stencil_columns(u, g, S, [&](int l, long long q0, bool down, bool up, R(&F)[3]) {
+  R vo[3], ao[3];   // this layer's, loaded before its arithmetic
+  auto pre = [&](int l, long long q0) {
+    if constexpr (CORRECT) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const long long i = ((long long)l * 3 + c) * plane + q0;
+        vo[c] = v[i];
+        ao[c] = a[i];
+      }
+    }
+  };
+  stencil_columns(u, g, S, pre, [&](int l, long long q0, bool down, bool up, R(&F)[3]) {
     if (l == g.L - 1 && tau_top)
 #pragma unroll
       for (int c = 0; c < 3; ++c) F[c] += g.area * tau_top[c * plane + q0];
@@ -238,7 +257,14 @@ __global__ void __launch_bounds__(kColThreads) force_kernel(const R* __restrict_
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const R extra = src ? src[((long long)l * 3 + c) * plane + q0] : (R)0;
-      al[c * plane + q0] = (F[c] + extra) * inv_m;
+      const R x = (F[c] + extra) * inv_m;
+      if (CORRECT && !(g.fault && (l == g.f || l == g.f + 1))) {
+        const long long i = ((long long)l * 3 + c) * plane + q0;
+        v[i] = vo[c] + (R)0.5 * dt * (x - ao[c]);
+        a[i] = x;
+      } else {
+        al[c * plane + q0] = x;
+      }
     }
   });
 }
@@ -247,10 +273,11 @@ __global__ void __launch_bounds__(kColThreads) force_kernel(const R* __restrict_
 // (sticktraction), (stickslip)) with linear slip weakening (Eq. (slipweak)), in
 // the perturbation formulation: shear traction tau0 + tau, normal stress
 // (compression positive) sigma0 - tau_2; the normal component always sticks.
-// Applies -A tau / m+ to the plus copy and +A tau / m- to the minus copy.
+// Applies -A tau / m+ to the plus copy and +A tau / m- to the minus copy, and corrects
+// the two layers' velocities (v holds v_pred, an the accelerations without traction).
 template <class R>
-__global__ void fault_kernel(const R* __restrict__ u, const R* __restrict__ vpred,
-                             const R* __restrict__ a, R* __restrict__ an, MeshArgs g,
+__global__ void fault_kernel(const R* __restrict__ u, R* __restrict__ vpred,
+                             R* __restrict__ a, const R* __restrict__ an, MeshArgs g,
                              FaultArgs<R> fa, R dt, int weld) {
   const long long plane = (long long)g.n1 * g.n3;
   const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -258,12 +285,14 @@ __global__ void fault_kernel(const R* __restrict__ u, const R* __restrict__ vpre
   const long long P = (long long)(g.f + 1) * 3 * plane + q;   // plus copy, component 0
   const long long M = (long long)g.f * 3 * plane + q;         // minus copy
   const R m = (R)g.half_mass;                                 // each copy: 4 elements
-  R stick[3], slipc[3];
+  R stick[3], slipc[3], v2[3][2], a2[3][2], f2[3][2];   // plus, minus
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const long long o = c * plane;
-    const R vp = vpred[P + o] - (R)0.5 * dt * a[P + o] + dt * an[P + o];
-    const R vm = vpred[M + o] - (R)0.5 * dt * a[M + o] + dt * an[M + o];
+    v2[c][0] = vpred[P + o]; a2[c][0] = a[P + o]; f2[c][0] = an[P + o];
+    v2[c][1] = vpred[M + o]; a2[c][1] = a[M + o]; f2[c][1] = an[M + o];
+    const R vp = v2[c][0] - (R)0.5 * dt * a2[c][0] + dt * f2[c][0];
+    const R vm = v2[c][1] - (R)0.5 * dt * a2[c][1] + dt * f2[c][1];
     stick[c] = (vp - vm) / (dt * (R)g.area * ((R)2 / m));
     slipc[c] = u[P + o] - u[M + o];
   }
@@ -284,21 +313,13 @@ __global__ void fault_kernel(const R* __restrict__ u, const R* __restrict__ vpre
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const long long o = c * plane;
-    an[P + o] -= (R)g.area * tau[c] / m;
-    an[M + o] += (R)g.area * tau[c] / m;
+    const R ap = f2[c][0] - (R)g.area * tau[c] / m;
+    const R am = f2[c][1] + (R)g.area * tau[c] / m;
+    vpred[P + o] = v2[c][0] + (R)0.5 * dt * (ap - a2[c][0]);
+    vpred[M + o] = v2[c][1] + (R)0.5 * dt * (am - a2[c][1]);
+    a[P + o] = ap;
+    a[M + o] = am;
     if (fa.traction) fa.traction[o + q] = tau[c];
-  }
-}
-
-// v = v_pred + dt/2 (a_{t+1} - a_t)  (Eq. (fecorr)); a = a_{t+1}.
-template <class R>
-__global__ void correct_kernel(R* __restrict__ v, R* __restrict__ a, const R* __restrict__ an,
-                               long long n, R dt) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    const R anew = an[i];
-    v[i] += (R)0.5 * dt * (anew - a[i]);
-    a[i] = anew;
   }
 }
 
@@ -448,7 +469,7 @@ __global__ void __launch_bounds__(kColThreads) stiffness_add_kernel(const R* __r
                                                             R* __restrict__ out, MeshArgs g,
                                                             const __grid_constant__ Stencil<R> S) {
   const long long plane = (long long)g.n1 * g.n3;
-  stencil_columns(x, g, S, [&](int l, long long q0, bool, bool, R(&F)[3]) {
+  stencil_columns(x, g, S, [](int, long long) {}, [&](int l, long long q0, bool, bool, R(&F)[3]) {
     R* ol = out + (long long)l * 3 * plane + q0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) ol[c * plane] += F[c];
@@ -497,21 +518,24 @@ cudaError_t predict(R* u, R* v, const R* a, long long n, R dt, cudaStream_t st) 
 template <class R>
 cudaError_t force(const R* u, R* an, const MeshArgs& g, const Stencil<R>& S, const R* tau_top,
                   const R* tau_bot, const R* src, cudaStream_t st) {
-  force_kernel<R><<<column_grid(g), kColThreads, 0, st>>>(u, an, g, S, tau_top, tau_bot, src);
+  force_kernel<R, false><<<column_grid(g), kColThreads, 0, st>>>(u, an, g, S, tau_top, tau_bot, src,
+                                                                 nullptr, nullptr, (R)0);
   return cudaGetLastError();
 }
 
 template <class R>
-cudaError_t fault(const R* u, const R* vpred, const R* a, R* an, const MeshArgs& g,
+cudaError_t force_correct(const R* u, R* v, R* a, R* an, const MeshArgs& g, const Stencil<R>& S,
+                          const R* tau_top, const R* tau_bot, const R* src, R dt, cudaStream_t st) {
+  force_kernel<R, true><<<column_grid(g), kColThreads, 0, st>>>(u, an, g, S, tau_top, tau_bot, src, v,
+                                                                a, dt);
+  return cudaGetLastError();
+}
+
+template <class R>
+cudaError_t fault(const R* u, R* vpred, R* a, const R* an, const MeshArgs& g,
                   const FaultArgs<R>& fa, R dt, int weld, cudaStream_t st) {
   const long long plane = (long long)g.n1 * g.n3;
   fault_kernel<R><<<(unsigned)((plane + 255) / 256), 256, 0, st>>>(u, vpred, a, an, g, fa, dt, weld);
-  return cudaGetLastError();
-}
-
-template <class R>
-cudaError_t correct(R* v, R* a, const R* an, long long n, R dt, cudaStream_t st) {
-  correct_kernel<R><<<grid1(n, 256), 256, 0, st>>>(v, a, an, n, dt);
   return cudaGetLastError();
 }
 
@@ -571,9 +595,11 @@ cudaError_t layer_add(R* dst, const R* src, long long n, cudaStream_t st) {
   template cudaError_t force<R>(const R*, R*, const MeshArgs&, const Stencil<R>&, const R*,  \
                                 const R*, const R*,                                          \
                                 cudaStream_t);                                               \
-  template cudaError_t fault<R>(const R*, const R*, const R*, R*, const MeshArgs&,           \
+  template cudaError_t force_correct<R>(const R*, R*, R*, R*, const MeshArgs&,               \
+                                        const Stencil<R>&, const R*, const R*, const R*, R,  \
+                                        cudaStream_t);                                       \
+  template cudaError_t fault<R>(const R*, R*, R*, const R*, const MeshArgs&,                 \
                                 const FaultArgs<R>&, R, int, cudaStream_t);                  \
-  template cudaError_t correct<R>(R*, R*, const R*, long long, R, cudaStream_t);             \
   template cudaError_t fault_fields<R>(const R*, const R*, const MeshArgs&, R*, R*, cudaStream_t); \
   template cudaError_t adjoint_stages<R>(const AdjointArgs<R>&, const MeshArgs&,                  \
                                          const Stencil<R>&, const FaultArgs<R>&, int,            \

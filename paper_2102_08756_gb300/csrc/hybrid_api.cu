@@ -5,9 +5,10 @@
 //   (1) FE predictor (Eq. (fepred), central-difference displacement update)
 //   (2)-(3) sbim_step of the top (side +1) and bottom (side -1) half-spaces with
 //       u_{t+1} and the predicted velocity of the boundary layers
-//   (4) internal force + boundary forces f = +A tau_top / -A tau_bot
-//   (5) fault traction (forward Lagrange multiplier, slip weakening)
-//   (6)-(7) acceleration increment and velocity correction (Eqs. (tintf), (fecorr))
+//   (4) internal force + boundary forces f = +A tau_top / -A tau_bot, and
+//       (6)-(7) acceleration and velocity correction off the fault (Eqs. (tintf), (fecorr))
+//   (5) fault traction (forward Lagrange multiplier, slip weakening), then (6)-(7) of
+//       the two fault layers
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -182,14 +183,14 @@ void boundary_ptrs(sbim_hybrid_ctx* c, const void** u_top, const void** v_top,
 template <class R>
 int stage_finish(sbim_hybrid_ctx* c, const void* src, cudaStream_t st) {
   const R dt = (R)c->dt;
-  const long long n = c->elems();
   R* u = (R*)c->u;
   R* v = (R*)c->v;
   R* a = (R*)c->a;
   R* an = (R*)c->an;
   const sbim::fem::MeshArgs g = mesh_args(c);
-  HCU(sbim::fem::force<R>(u, an, g, stencil_of(c, R()), c->boundaries ? (const R*)c->tau_top : nullptr,
-                          c->boundaries ? (const R*)c->tau_bot : nullptr, (const R*)src, st));
+  HCU(sbim::fem::force_correct<R>(u, v, a, an, g, stencil_of(c, R()),
+                                  c->boundaries ? (const R*)c->tau_top : nullptr,
+                                  c->boundaries ? (const R*)c->tau_bot : nullptr, (const R*)src, dt, st));
   if (c->fault) {
     sbim::fem::FaultArgs<R> fa;
     fa.mu_s = (const R*)c->mu_s;
@@ -200,7 +201,6 @@ int stage_finish(sbim_hybrid_ctx* c, const void* src, cudaStream_t st) {
     fa.traction = (R*)c->traction;
     HCU(sbim::fem::fault<R>(u, v, a, an, g, fa, dt, c->have_law ? 0 : 1, st));
   }
-  HCU(sbim::fem::correct<R>(v, a, an, n, dt, st));
   return SBIM_OK;
 }
 template <class R>
