@@ -966,6 +966,38 @@ void pair_release(PairStreams& p) {
   if (p.side) cudaStreamDestroy(p.side);
 }
 
+bool handle_raw_ok(sbim_handle c) { return !c->prof && !c->check_finite; }
+
+// s of a level, written to `out`, without the radiation term, the far field or the step
+// counter: the first evaluation of a level forms the block sums (or convolves), `again`
+// re-evaluates it with another displacement.  The caller adds handle_far_field and
+// advances the counter (handle_counter on the device, handle_advanced on the host) once
+// the level is final.
+int handle_raw_step(sbim_handle c, const void* in, void* out, bool again, cudaStream_t st) {
+  const sbim::StepArgs a = step_args(c);
+  const bool sums = c->use_ahead && !again;
+  if (sums)
+    if (const int rc = fork_sums(c, a, st)) return rc;
+  if (const int rc = handle_fft_forward(c, in, st)) return rc;
+  if (sums) CU(cudaStreamWaitEvent(st, c->sums.join, 0));
+  if (c->use_ahead) {
+    CU(launch_ahead(a, c->prec, 2, c->halves, st));
+  } else {
+    if (again) CU(launch_repeat_lag0(a, c->prec, st));
+    else if (c->variant >= 1)
+      CU(launch_conv_tma(a, c->prec, c->kahan, c->variant, st, nullptr, c->tile, c->halves));
+    else CU(launch_conv(a, c->prec, c->kahan, st));
+    CU(launch_assemble(a, c->prec, c->kahan, st));
+  }
+  return handle_fft_inverse(c, st, out);
+}
+const double* handle_far_field(sbim_handle c) { return c->tau_inf; }
+long long* handle_counter(sbim_handle c) { return c->d_step; }
+void handle_advanced(sbim_handle c) {
+  ++c->n;
+  c->can_repeat = true;
+}
+
 int handle_step_on(sbim_handle c, const void* in, const void* aux, void* out, int kind, cudaStream_t st) {
   if (kind == 2 && (!c->can_repeat || c->n == 0))
     return fail(SBIM_ERR_STATE, "nothing to repeat on this handle");

@@ -161,6 +161,11 @@ int handle_fft_inverse(sbim_handle h, cudaStream_t st, void* out = nullptr);   /
 // One sbim_step (kind 0), sbim_step_adjoint (1: in = tau_bar, aux = v_bar, out = u_bar)
 // or sbim_step_repeat (2) on a stream forked from the handle's and joined to it.
 int handle_step_on(sbim_handle h, const void* in, const void* aux, void* out, int kind, cudaStream_t st);
+bool handle_raw_ok(sbim_handle h);
+int handle_raw_step(sbim_handle h, const void* in, void* out, bool again, cudaStream_t st);
+const double* handle_far_field(sbim_handle h);
+long long* handle_counter(sbim_handle h);
+void handle_advanced(sbim_handle h);
 // A side stream for the second of two half-spaces that step side by side.
 struct PairStreams {
   cudaStream_t side = nullptr;
