@@ -428,7 +428,9 @@ __global__ void __launch_bounds__(kThreads, 1) ahead_kernel(const __grid_constan
 }
 
 // The same over the members of a batch: CTA item_prefix[s] + ... belongs to member s,
-// 16 sub-tiles of each group of 16 tiles, chunk-major.
+// 4 sub-tiles of each group of 16 tiles, chunk-major.  The weights of whole and half
+// records are laid out differently: a batch that holds both is launched once for each,
+// and the CTAs of the other members return at once.
 template <class S, bool HALVES>
 __global__ void __launch_bounds__(kThreads, 1)
 ahead_batch_kernel(const StepArgs* __restrict__ args, const int* __restrict__ item_prefix, int nb) {
@@ -443,6 +445,7 @@ ahead_batch_kernel(const StepArgs* __restrict__ args, const int* __restrict__ it
     s_local = blockIdx.x - item_prefix[s];
   }
   __syncthreads();
+  if ((s_args.halves != 0) != HALVES) return;
   const int per_chunk = ahead_ctas(s_args.n_orb_pad);
   const int r = s_local % per_chunk;
   ahead_tiles<S, HALVES>(s_args, r / kSub, r % kSub, s_local / per_chunk, smem, sync);
@@ -645,7 +648,12 @@ cudaError_t run_stage(const StepArgs& a, int stage, bool halves, cudaStream_t st
                       const BatchLaunch* batch, int tiles) {
   switch (stage) {
     case 0: return halves ? prepare<S, true>() : prepare<S, false>();
-    case 1: return halves ? launch_sums<S, true>(a, st, batch) : launch_sums<S, false>(a, st, batch);
+    case 1: {
+      const bool whole = batch ? batch->whole : !halves;
+      cudaError_t e = whole ? launch_sums<S, false>(a, st, batch) : cudaSuccess;
+      if (e == cudaSuccess && halves) e = launch_sums<S, true>(a, st, batch);
+      return e;
+    }
     case 3: return halves ? launch_weights<true>(a, st) : launch_weights<false>(a, st);
     case 2: return launch_near<S>(a, st, batch, tiles);
     default: return cudaErrorInvalidValue;

@@ -18,6 +18,7 @@ struct sbim_batch_ctx {
   int tile = sbim::kOrbitTile;   // orbits per CTA of the batched convolution
   int lags = 0;                  // lags per work item last configured
   bool halves = false;           // some member's records hold two |k|
+  bool whole = false;            // some member's do not
   bool per_item = false;    // one CTA per work item instead of persistent CTAs
   bool ahead = false;       // every member's convolution is blocked in time
   bool owns = true;
@@ -114,13 +115,15 @@ int configure(sbim_batch_ctx* b, int shape, int lags) {
     const int rc = sbim_set_conv_config(b->h[i], shape, lags);
     if (rc != SBIM_OK) return rc;
   }
-  b->halves = false;
-  for (int i = 0; i < b->nb; ++i) b->halves = b->halves || sbim::handle_step_args(b->h[i]).halves;
+  b->halves = b->whole = false;
+  for (int i = 0; i < b->nb; ++i)
+    (sbim::handle_step_args(b->h[i]).halves ? b->halves : b->whole) = true;
   // time-blocked where every member has room for its block sums
   b->ahead = true;
   for (sbim_handle x : b->h) b->ahead = b->ahead && sbim::handle_uses_ahead(x);
   if (b->ahead) {
-    BCU(sbim::launch_ahead(sbim::StepArgs{}, b->prec, 0, b->halves, nullptr));
+    if (b->whole) BCU(sbim::launch_ahead(sbim::StepArgs{}, b->prec, 0, false, nullptr));
+    if (b->halves) BCU(sbim::launch_ahead(sbim::StepArgs{}, b->prec, 0, true, nullptr));
   } else {
     BCU(sbim::prepare_conv_tma(b->prec, b->kahan, shape, b->tile, b->halves));
     for (sbim_handle x : b->h) {
@@ -199,6 +202,7 @@ int enqueue(sbim_batch_ctx* b, const void* const* u, const void* const* v, void*
   bl.counter = b->d_counter;
   bl.ctas = b->ctas;
   bl.items = b->per_item || b->ahead ? b->total_items : 0;
+  bl.whole = b->whole;
   int rc = fork(b);
   // the block sums need only the stored histories: they run beside the transforms
   if (rc == SBIM_OK && b->ahead) BCU(sbim::launch_ahead(a0, b->prec, 1, b->halves, b->stream, &bl));

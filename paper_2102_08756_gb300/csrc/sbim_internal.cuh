@@ -58,7 +58,7 @@ struct StepArgs {
   int* err;                        // device error word (bounded waits that gave up)
   void* part;                      // [nchunks][40][n_orb_pad] partial sums
   float* ahead;                    // time-blocked sums: [ahead_chunks][tile][16 steps][10][128 records x 4]
-  long long* stamp;                // [ahead_chunks][tile][16] the block and configuration they belong to
+  long long* stamp;                // [chunk][tile][4] the block and configuration they belong to
   const void* uhat;                // [3][nbins] forward spectra
   void* fhat;                      // [3][nbins] output spectra (scaled 1/(n1 n3))
   // sizes (host values)
@@ -86,6 +86,7 @@ struct BatchLaunch {
   int* counter;             // work counter, zero before each launch
   int ctas;                 // persistent CTAs
   int items;                // > 0: one CTA per item (this many), no persistent CTAs
+  bool whole;               // some member has whole records (others may have half records)
 };
 
 // Groups of kAhead tiles: each step renews the block sums of one tile of a group.

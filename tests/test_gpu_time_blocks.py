@@ -113,3 +113,39 @@ def test_non_finite_values_leave_with_their_last_lag():
         assert torch.equal(t, r), m
         seen += int(not bool(r.all()))
     assert seen == n_cut
+
+
+def _batch(members, n_cut, dt, stream):
+    from paper_2102_08756_gb300 import sbim as B
+    k = len(members)
+    n1, n3 = [list(x) for x in zip(*members)]
+    b = B.sbim_batch_create(n1, n3, [100.0 * x for x in n1], [100.0 * x for x in n3], [CS] * k, [CP] * k,
+                            [RHO] * k, [dt] * k, [n_cut] * k, [1] * k, 1, 1, stream.cuda_stream)
+    return B, b
+
+
+def _batch_step(B, b, f):
+    tau = [torch.empty_like(u) for u, _ in f]
+    B.sbim_batch_step(b, [u.data_ptr() for u, _ in f], [v.data_ptr() for _, v in f],
+                      [t.data_ptr() for t in tau])
+    return tau
+
+
+# whole and half records in one batch, in both orders, and each alone
+@pytest.mark.parametrize("members", [[(32, 32), (64, 6), (48, 48)], [(64, 6), (32, 32)], [(64, 6)], [(32, 32)]])
+def test_batches_of_mixed_layouts(members):
+    from paper_2102_08756_gb300.sbim import SBIM
+    n_cut, dt = 40, 0.3 * 100.0 / CP
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        B, b = _batch(members, n_cut, dt, stream)
+        alone = [SBIM(n1, n3, n1 * 100.0, n3 * 100.0, CS, CP, RHO, dt, n_cut, 1, "fp32", True,
+                      stream=stream) for n1, n3 in members]
+        for h in alone:
+            h.set_conv_config(2, 1024)
+        f = [_fields(n1, n3, dt, 60, seed=k) for k, (n1, n3) in enumerate(members)]
+        for m in range(60):
+            tau = _batch_step(B, b, [x[m] for x in f])
+            for k, h in enumerate(alone):
+                assert torch.equal(tau[k], h.step(*f[k][m])), (m, k)
+        B.sbim_batch_destroy(b)
