@@ -467,8 +467,7 @@ int make_ring_map(const sbim_ctx& c, CUtensorMap* map) {
 // convolves step by step).
 bool alloc_ahead(sbim_ctx& c, size_t budget) {
   if (!c.d_wts32) return false;
-  const size_t sneed = (size_t)c.ahead_chunks * c.n_orb_pad / sbim::kAheadRec * sizeof(long long);
-  const size_t need = ahead_need(c) + sneed;     // stamps behind the sums
+  const size_t need = ahead_need(c);
   if (need > c.ahead_bytes) {
     void* fresh = nullptr;
     if (need > budget || cudaMalloc(&fresh, need) != cudaSuccess) {
@@ -482,8 +481,6 @@ bool alloc_ahead(sbim_ctx& c, size_t budget) {
     c.d_ahead = (float*)fresh;
     c.ahead_bytes = need;
   }
-  c.d_stamp = (long long*)((char*)c.d_ahead + ahead_need(c));
-  c.stamp_bytes = sneed;
   return forget_ahead(&c) == SBIM_OK;
 }
 
@@ -599,9 +596,17 @@ int create_impl(sbim_ctx* c) {
 
   // The block sums' weights (16 B per record and lag beside 96 of FP32 history, 32 for
   // half records) and the least room for the sums themselves; a handle that has none
-  // left convolves step by step.
+  // left convolves step by step.  Half-spaces come in pairs (the two sides of a slab or
+  // a fault, an update and its transpose): these extras never take the room of a second
+  // handle of this size that would fit without them.
   const size_t w32 = dbl ? 0 : sbim::ahead_weight_bytes(c->n_orb_pad, c->n_cut, c->halves);
-  const bool blocked = w32 && need + w32 + (size_t)c->n_orb_pad * 4096 + kSpareBytes <= free_b;
+  const size_t extras = w32 + (size_t)c->n_orb_pad * 4096 + kSpareBytes;
+  const bool blocked = w32 && need + extras <= free_b &&
+                       (2 * need + extras <= free_b || 2 * need + kSpareBytes > free_b);
+  // a stamp for every chunk that any chunking can have: they stay where they are when
+  // the chunking changes, so that a batch's own copy of the arguments stays consistent
+  c->stamp_bytes = blocked ? (size_t)((c->n_cut + sbim::kAhead - 1) / sbim::kAhead) *
+                                 (c->n_orb_pad / sbim::kAheadRec) * sizeof(long long) : 0;
 
   // Lay the arena out: what the host fills in first, in one copy, then the rest.
   size_t at = 0;
@@ -628,7 +633,10 @@ int create_impl(sbim_ctx* c) {
   put(&c->d_uhat, 3 * (size_t)c->nbins * cplx);
   put(&c->d_fhat, 3 * (size_t)c->nbins * cplx);
   put(&c->d_s, c->field_elems() * c->real_size);
-  if (blocked) put(&c->d_wts32, w32);
+  if (blocked) {
+    put(&c->d_wts32, w32);
+    put((void**)&c->d_stamp, c->stamp_bytes);
+  }
   if (c->wts_bytes) put(&c->d_wts, c->wts_bytes);
   put(&c->d_hist, c->hist_bytes);
   CU(cudaMalloc(&c->d_arena, at));
@@ -1121,6 +1129,7 @@ int sbim_set_window(sbim_handle h, double window) {
   if (!(window >= 0)) return fail(SBIM_ERR_ARG, "window must be >= 0");
   h->can_repeat = false;
   ++h->config_id;
+  if (const int rc = forget_ahead(h)) return rc;
   if (window == 0) {
     h->window = 0;
     return SBIM_OK;

@@ -149,3 +149,30 @@ def test_batches_of_mixed_layouts(members):
             for k, h in enumerate(alone):
                 assert torch.equal(tau[k], h.step(*f[k][m])), (m, k)
         B.sbim_batch_destroy(b)
+
+
+def test_member_with_its_own_chunking_between_batch_steps():
+    """A batch keeps its copy of a member's chunking; the member, given a coarser one and
+    stepped by itself, and the batch then alternate on the same sums buffer."""
+    n1, n3, n_cut = 48, 32, 70
+    stream = torch.cuda.Stream()
+    err = Worst()
+    with torch.cuda.stream(stream):
+        _, ref, dt = _pair(n1, n3, n_cut, "fp32", side=1)
+        B, b = _batch([(n1, n3)], n_cut, dt, stream)
+        B.sbim_batch_set_conv_config(b, 2, 16)
+        member = B.sbim_batch_member(b, 0)
+        f = _fields(n1, n3, dt, 100, seed=9)
+        for m, (u, v) in enumerate(f):
+            if m == 75:
+                B.sbim_set_conv_config(member, 2, 64)
+            if m >= 75 and m % 3:
+                tau = torch.empty_like(u)
+                B.sbim_step(member, u.data_ptr(), v.data_ptr(), tau.data_ptr())
+            else:
+                tau = _batch_step(B, b, [(u, v)])[0]
+            stream.synchronize()
+            r = ref.step(u.double(), v.double()).cpu().numpy()
+            err.update(rel_l2(tau.double().cpu().numpy(), r))
+        B.sbim_batch_destroy(b)
+    assert err.value < TOL["fp32"], err
