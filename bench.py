@@ -48,7 +48,9 @@ MACS_PER_PAIR = 5
 DEFAULT_VARIANT = {"fp32": 2, "bf16": 2, "bf16x2": 2, "fp64": 1}
 BYTES_PER_PAIR = {"fp64": 48, "fp32": 24, "bf16x2": 24, "bf16": 12}
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-# DRAM bytes (read + write) per convolution launch of the full 1024^2 x 4096
+# 152 SMs x 128 FP32 multiply-adds/clk x 2 flops x 2.07 GHz = 80.5 TFLOP/s
+FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
+# DRAM bytes (read + write) per step-by-step convolution launch of the full 1024^2 x 4096
 # workload, valid only for the kernel source with this hash: ncu's DRAM bytes of
 # one launch at 512^2 x 1024 lags (1.00645 x the ring buffer read, plus the
 # lag-chunk partial sums written), scaled component by component to the full
@@ -370,6 +372,25 @@ def cpu_workers():
     return max(1, os.cpu_count() or 1)
 
 
+def conv_roofline(pairs, alg_bytes, ms, kernel, traffic=None):
+    """Roofline of a float-class convolution that took `ms` a step.  Step by step it is bound by the
+    history's bytes; blocked in time (one pass over the history forms the sums of 16 steps) by the FP32
+    pipe: 10 real multiply-adds (20 flops) per (mode, lag) pair.  A step that beats the copy bandwidth
+    by 15 % on the step-by-step bytes has not read them all, so it ran blocked."""
+    peak, kind = peaks()
+    hbm = alg_bytes / (ms * 1e-3) / 1e9
+    if hbm <= 1.15 * peak:
+        return {"bound": "hbm", "achieved": hbm, "peak": peak, "unit": "GB/s", "frac": hbm / peak,
+                "traffic": traffic, "kernel": kernel, "peak_kind": kind,
+                "algorithmic_bytes_per_launch": alg_bytes, "launch_ms": ms}
+    tf = pairs * 20 / (ms * 1e-3) / 1e12
+    return {"bound": "alu", "achieved": tf, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
+            "frac": tf / FP32_PEAK_TFLOPS, "traffic": None,
+            "kernel": kernel.replace("conv_tma_kernel", "ahead_kernel"),
+            "peak_kind": "nominal (unit count x clock)", "algorithmic_flops_per_launch": pairs * 20,
+            "launch_ms": ms}
+
+
 def cpu_baseline_leg(c, modes_per_worker=1024, seconds=10.0):
     """The FP64 oracle timed on the host: every core at once (the reported
     value), and one thread alone beside it."""
@@ -546,7 +567,7 @@ def run_native(args):
     bpp = BYTES_PER_PAIR[prec]
     alg_bytes = (pairs + modes) * bpp
     achieved = alg_bytes / (conv_ms * 1e-3) / 1e9
-    peak, peak_kind = peaks()
+    peak, _ = peaks()
     # the FP64 history is bound by the FP64 pipe: 10 real FMAs (20 flops) per
     # (mode, lag) pair against GB300's FP64 rate (152 SMs x 2 DFMA/clk x 2 flops
     # x 2.07 GHz = 1.259 TFLOP/s, nominal)
@@ -611,11 +632,8 @@ def run_native(args):
                    "modes": modes, "history_bytes": hist_bytes,
                    "l2": "inputs larger than L2 (history ring buffer >> 129 MB)",
                    "parallelism": f"replicas x{world}"},
-        "roofline": alu or {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                            "frac": achieved / peak, "traffic": traffic,
-                            "kernel": "conv_tma_kernel" if (args.variant != 0) else "conv_kernel",
-                            "peak_kind": peak_kind,
-                            "algorithmic_bytes_per_launch": alg_bytes, "launch_ms": conv_ms},
+        "roofline": alu or conv_roofline(pairs, alg_bytes, conv_ms,
+                                         "conv_tma_kernel" if args.variant != 0 else "conv_kernel", traffic),
         "stage_ms_per_step": {k: v / nprof for k, v in stage.items()},
         "hbm_gbs_step": alg_bytes / (ms_step * 1e-3) / 1e9,
         "cpu_baseline": cpu,
@@ -711,9 +729,7 @@ def run_coupled(args):
     slip, rate, _ = g.fault_fields()
     modes = n3 * (n1 // 2 + 1)
     macs = 2 * modes * n_cut * MACS_PER_PAIR
-    conv_ms = stage["convolution"] / nprof
-    alg = (modes * n_cut + modes) * BYTES_PER_PAIR["fp32"]
-    peak, peak_kind = peaks()
+    alg = 2 * (modes * n_cut + modes) * BYTES_PER_PAIR["fp32"]
     line = {
         "metric": "coupled hybrid steps/s", "value": 1e3 / ms, "unit": "steps/s", "n_gpus": 1,
         "steps": K, "warmup": W, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
@@ -722,11 +738,8 @@ def run_coupled(args):
                                f"slip-weakening fault, two SBIM half-spaces, {n_cut}-lag history",
                    "elements": n1 * n2 * n3, "l2": "history (12.6 GB) >> L2"},
         "sbim_macs_per_s": macs / (ms * 1e-3),
-        "roofline": {"bound": "hbm", "achieved": alg / (conv_ms * 1e-3) / 1e9, "peak": peak,
-                     "unit": "GB/s", "frac": alg / (conv_ms * 1e-3) / 1e9 / peak, "traffic": None,
-                     "kernel": "conv_tma_kernel (one half-space's launch, its stage events)",
-                     "peak_kind": peak_kind, "algorithmic_bytes_per_launch": alg,
-                     "launch_ms": conv_ms},
+        # the two half-spaces run side by side: the whole step, a lower bound
+        "roofline": conv_roofline(2 * modes * n_cut, alg, ms, "whole coupled step (FE stages included)"),
         "stage_ms_per_step_top": {k: v / nprof for k, v in stage.items()},
         "fault": {"max_slip_m": float(slip.abs().max()), "max_slip_rate_m_s": float(rate.abs().max()),
                   "simulated_s": (n_cut + W + K) * dt},
@@ -808,7 +821,6 @@ def run_tpv3(args):
                                                               dt, steps, "fp32", True))
     modes = n3 * (n1 // 2 + 1)
     alg = (modes * steps + modes) * BYTES_PER_PAIR["fp32"]
-    peak, peak_kind = peaks()
     slots = B.sbim_plan(n1, n3, n1 * h, n3 * h, steps, "fp32")["n_slots"]
     both = np.isfinite(t_h) & np.isfinite(t_p)
     either = np.isfinite(t_h) | np.isfinite(t_p)
@@ -821,11 +833,7 @@ def run_tpv3(args):
                                f"(symmetry plane) vs hybrid with a 4-element slab",
                    "l2": "history >> L2"},
         "hybrid_ms_per_step": ms_h,
-        "roofline": {"bound": "hbm", "achieved": alg / (conv_p * 1e-3) / 1e9, "peak": peak,
-                     "unit": "GB/s", "frac": alg / (conv_p * 1e-3) / 1e9 / peak, "traffic": None,
-                     "kernel": "conv_tma_kernel + repeat_lag0_kernel (the step's one history pass)",
-                     "peak_kind": peak_kind, "algorithmic_bytes_per_launch": alg,
-                     "launch_ms": conv_p},
+        "roofline": conv_roofline(modes * steps, alg, conv_p, "conv_tma_kernel (the step's one history pass)"),
         "layout": {"modes": modes, "slots": slots, "padding": slots / modes},
         "agreement": {
             "ruptured_nodes": int(both.sum()), "ruptured_either": int(either.sum()),
@@ -921,11 +929,8 @@ def run_ensemble(args):
         "sbim_macs_per_s": macs / (ms * 1e-3), "hbm_gbs_history": hist_bytes / (ms * 1e-3) / 1e9,
         # the batched convolution runs inside the replayed graph, so only the
         # whole step is timed: a lower bound on the convolution's own rate
-        "roofline": {"bound": "hbm", "achieved": hist_bytes / (ms * 1e-3) / 1e9, "peak": peaks()[0],
-                     "unit": "GB/s", "frac": hist_bytes / (ms * 1e-3) / 1e9 / peaks()[0],
-                     "traffic": None, "peak_kind": peaks()[1],
-                     "kernel": "whole ensemble step (graph replay, FE stages included)",
-                     "algorithmic_bytes_per_launch": hist_bytes, "launch_ms": ms},
+        "roofline": conv_roofline(macs // MACS_PER_PAIR, hist_bytes, ms,
+                                  "whole ensemble step (graph replay, FE stages included)"),
         "max_slip_rate_m_s": peak_rate, "clocks": clk.summary(),
     }
     if tuned is not None:
