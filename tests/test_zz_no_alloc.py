@@ -144,3 +144,25 @@ def test_noalloc_rejects_misaligned_and_host_pointers(sbim):
     sbim.sbim_spectral_response_noalloc(*args, h.data_ptr(), o.data_ptr(), None)
     torch.cuda.synchronize()
     assert float(o.abs().max()) == 0.0
+
+
+# grids with no pair of bins (j1, +-j3), with one, and with ragged last threads; lags around the 4 in flight
+@pytest.mark.parametrize("n1,n3", [(4, 2), (2, 4), (6, 4), (258, 6), (16, 130)])
+@pytest.mark.parametrize("n_lags", [1, 3, 4, 5, 66])
+def test_noalloc_pairs_of_bins(sbim, n1, n3, n_lags):
+    """Bins of one |k| share a thread: every bin against the oracle, and nothing written past the output."""
+    dx, cp, side = 100.0, 6000.0, -1
+    dt = 0.3 * dx / cp
+    nh = n1 // 2 + 1
+    rng = np.random.default_rng(n1 * n3 + n_lags)
+    spec = np.fft.rfft2(rng.standard_normal((n_lags, 3, n3, n1))).astype(np.complex64)
+    hist = torch.from_numpy(spec.view(np.float32)).cuda()
+    out = torch.full((3 * n3 * nh + 32, 2), 7.0, device="cuda")
+    sbim.sbim_spectral_response_noalloc(n1, n3, n1 * dx, n3 * dx, CS, cp, RHO, dt, side, n_lags,
+                                        hist.data_ptr(), out.data_ptr(),
+                                        torch.cuda.current_stream().cuda_stream)
+    got = out.cpu().numpy()
+    assert np.all(got[3 * n3 * nh:] == 7.0)
+    got = got[:3 * n3 * nh].copy().view(np.complex64).reshape(3, n3, nh).astype(np.complex128)
+    ref = _oracle_spectrum(n1, n3, n1 * dx, n3 * dx, cp, dt, side, spec.astype(np.complex128))
+    assert np.linalg.norm(got - ref) < 1e-5 * np.linalg.norm(ref)
