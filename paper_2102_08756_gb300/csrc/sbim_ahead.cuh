@@ -10,7 +10,13 @@
 // and each step of the block adds the at most 16 lags that lie inside the block
 // (near_kernel).  The history is read once per 16 steps and the work per step is
 // the same multiply-adds, now bound by the FP32 pipe (39-40 T multiply-adds/s
-// measured on GB300, 0.54 ms for 1024^2 x 4096 against 7.1 ms for the bytes).
+// measured on GB300: 0.54 ms for 1024^2 x 4096 against 7.1 ms for the bytes).  The kernel
+// takes 1.11 ms there, 155 ns per lag of a CTA against 77 on the pipe alone: 17 of a
+// warp's 41 instructions per lag are the two-lane multiply-adds (ncu, 512^2 x 1024), and
+// the pipe is busy 59 % of the time.  A warp set aside for the requests (spills: 21 warps
+// leave 80 registers), the requests in turns behind an mbarrier (+3 %), a skew of at most
+// one (+15 %) or two stages (+1 %) between the warps, and weights loaded into both halves
+// of a register pair (same) were measured and not kept.
 //
 // Blocks are aligned and staggered: tile T (128 records) starts its blocks at the
 // steps with (n + T) mod 16 = 0, so every step renews 1/16 of the tiles and costs
@@ -498,6 +504,8 @@ __device__ __forceinline__ void near_member(const StepArgs& a, int T, int x) {
     kadd<1>(acc[6], cmp[6], w[3], d[1].x); kadd<1>(acc[7], cmp[7], w[3], d[1].y);
     kadd<1>(acc[8], cmp[8], w[3], d[0].x); kadd<1>(acc[9], cmp[9], w[3], d[0].y);
   };
+  // (issuing the next four lags' loads ahead of these took 56.6 instead of 52.3 us at
+  // 1024^2, 123 registers against 92, and changed nothing below 512^2)
   // the chunks' block sums
   const int m_far = last_lag(a, base, T);
   const int nch = m_far > 0 ? (m_far + a.ahead_lc - 1) / a.ahead_lc : 0;
