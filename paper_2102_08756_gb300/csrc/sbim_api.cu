@@ -601,7 +601,12 @@ int create_impl(sbim_ctx* c) {
   // handle of this size that would fit without them.
   const size_t w32 = dbl ? 0 : sbim::ahead_weight_bytes(c->n_orb_pad, c->n_cut, c->halves);
   const size_t extras = w32 + (size_t)c->n_orb_pad * 4096 + kSpareBytes;
-  const bool blocked = w32 && need + extras <= free_b &&
+  // On large planes of whole records a very short BF16 history is read faster than the lags
+  // inside a block are added (1024^2, hi-only, us a step: 16 lags 129 step by step against
+  // 143, 24 lags 141 / 150, 39 lags 162 / 151; hi/lo, 16 lags: 163 / 152; half records,
+  // 1024 x 500, 20 lags: 96 / 90).
+  const int least = c->prec == SBIM_BF16 && !c->halves && c->n_orb_pad >= 16384 ? 28 : 0;
+  const bool blocked = w32 && c->n_cut >= least && need + extras <= free_b &&
                        (2 * need + extras <= free_b || 2 * need + kSpareBytes > free_b);
   // a stamp for every chunk that any chunking can have: they stay where they are when
   // the chunking changes, so that a batch's own copy of the arguments stays consistent

@@ -176,3 +176,28 @@ def test_member_with_its_own_chunking_between_batch_steps():
             err.update(rel_l2(tau.double().cpu().numpy(), r))
         B.sbim_batch_destroy(b)
     assert err.value < TOL["fp32"], err
+
+
+# few lags and many; large planes with short BF16 histories (whole records: 384^2 convolves step by step)
+@pytest.mark.parametrize("precision,grid,n_cut", [("fp32", (48, 32), 40), ("fp32", (48, 32), 90),
+                                                  ("bf16", (48, 32), 40), ("bf16x2", (48, 32), 130),
+                                                  ("bf16", (384, 384), 20), ("bf16x2", (512, 256), 24)])
+def test_host_direct_and_repeated_steps_in_turn(precision, grid, n_cut):
+    """Host-buffer, direct and repeated steps of one handle against the FP64 handle."""
+    from paper_2102_08756_gb300 import sbim as B
+    n1, n3 = grid
+    g, ref, dt = _pair(n1, n3, n_cut, precision)
+    err = Worst()
+    for m, (u, v) in enumerate(_fields(n1, n3, dt, n_cut + 20, seed=3)):
+        r = ref.step(u.double(), v.double()).cpu().numpy()
+        if m % 5 in (0, 1, 3):
+            t = torch.from_numpy(g.step_host(u.cpu().numpy(), v.cpu().numpy()))
+        else:
+            t = g.step(u, v)
+        err.update(rel_l2(t.double().cpu().numpy(), r))
+        if m % 5 in (1, 4):
+            out = torch.empty_like(u)
+            B.sbim_step_repeat(g.h, u.data_ptr(), v.data_ptr(), out.data_ptr())
+            err.update(rel_l2(out.double().cpu().numpy(), r))
+    g.check()
+    assert err.value < TOL[precision], err
