@@ -27,7 +27,9 @@
 // of the block its sums belong to and of the arguments' chunking and window; sums
 // whose stamp is not the current one are formed again, all on the device, so that a
 // captured graph renews them as a direct step does.  sbim_reset and sbim_load, which
-// change the ring itself, mark every stamp invalid.
+// change the ring itself, mark every stamp invalid, and sbim_rewind those of blocks
+// that begin after the step it goes back to: a level before them may be written again,
+// and a block whose predecessor has no history in a chunk finds its old stamp there.
 #pragma once
 
 #include <type_traits>
@@ -157,7 +159,7 @@ __device__ __forceinline__ long long block_base(long long n, int T) {
 }
 // The stamp of sums formed for a block with these arguments' chunking and window.
 __device__ __forceinline__ long long block_mark(const StepArgs& a, long long base) {
-  return base * 65536 + a.config_id;
+  return stamp_of(base, a.config_id);
 }
 // Largest lag m of the block sums A[s] of tile T: the history before `base`, the
 // cutoff, and the tile's truncation window.

@@ -1260,7 +1260,8 @@ int sbim_reset(sbim_handle h) {
 int sbim_rewind(sbim_handle h) {
   if (!h) return fail(SBIM_ERR_ARG, "NULL handle");
   if (h->n == 0) return fail(SBIM_ERR_STATE, "no step to rewind");
-  CU(sbim::launch_rewind(h->d_step, h->stream));
+  CU(sbim::launch_rewind(h->d_step, h->stream, h->d_stamp,
+                         (long long)(h->stamp_bytes / sizeof(long long))));
   --h->n;
   h->can_repeat = false;
   return SBIM_OK;

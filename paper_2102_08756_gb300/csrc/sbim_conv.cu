@@ -345,6 +345,14 @@ __global__ void rewind_kernel(long long* step) {
   if (threadIdx.x == 0 && *step > 0) *step -= 1;
 }
 
+// Block sums that begin after the step the counter is about to go back to: the levels
+// they were formed from may be written again before their block comes round.
+__global__ void forget_after_kernel(const long long* __restrict__ step, long long* __restrict__ stamp,
+                                    long long n) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i < n && stamp[i] >= 0 && stamp_base(stamp[i]) > *step - 1) stamp[i] = -1;
+}
+
 template <class S, int KAHAN>
 cudaError_t conv_dispatch(const StepArgs& a, cudaStream_t st) {
   const dim3 grid(a.n_orb_pad / kOrbitTile, a.nchunks);
@@ -472,7 +480,9 @@ cudaError_t launch_nonfinite_check(int precision, const void* a, const void* b, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_rewind(long long* step, cudaStream_t st) {
+cudaError_t launch_rewind(long long* step, cudaStream_t st, long long* stamp, long long stamps) {
+  if (stamp)
+    forget_after_kernel<<<(unsigned)((stamps + 255) / 256), 256, 0, st>>>(step, stamp, stamps);
   rewind_kernel<<<1, 32, 0, st>>>(step);
   return cudaGetLastError();
 }

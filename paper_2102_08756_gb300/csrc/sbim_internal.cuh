@@ -103,6 +103,9 @@ __host__ __device__ constexpr long long ahead_weight_bytes(int n_orb_pad, int n_
 __host__ __device__ constexpr int ahead_ctas(int n_orb_pad) {
   return ahead_groups(n_orb_pad) * (kOrbitTile / kAheadRec);
 }
+// A block's stamp holds its first step and 16 bits for the chunking and window.
+__host__ __device__ constexpr long long stamp_of(long long base, int config_id) { return base * 65536 + config_id; }
+__host__ __device__ constexpr long long stamp_base(long long stamp) { return stamp / 65536; }
 // Time-blocked convolution of float-class histories (sbim_ahead.cuh): stage 0
 // prepares the kernels, stage 3 fills wts32, stage 1 forms the block sums that are due, stage 2 adds the
 // step's own lags, stores the current spectra and assembles the output spectra.
@@ -129,7 +132,9 @@ cudaError_t prepare_conv_tma(int precision, int kahan, int shape, int tile = kOr
 // One CTA whose bounded mbarrier wait can never complete (sbim_selftest_wait_timeout).
 cudaError_t launch_wait_selftest(int* err, cudaStream_t st);
 cudaError_t launch_assemble(const StepArgs& a, int precision, int kahan, cudaStream_t s);
-cudaError_t launch_rewind(long long* step, cudaStream_t st);
+// The step counter one back; the stamps of block sums that begin after it are cleared.
+cudaError_t launch_rewind(long long* step, cudaStream_t st, long long* stamp = nullptr,
+                          long long stamps = 0);
 // FP64 path: out[m][o] = the four convolution weights of orbit o at lag m,
 // m < n_cut (the cubic interpolation of the FP64 table the kernels would do).
 cudaError_t launch_weights64(const StepArgs& a, void* out, cudaStream_t st);

@@ -201,3 +201,29 @@ def test_host_direct_and_repeated_steps_in_turn(precision, grid, n_cut):
             err.update(rel_l2(out.double().cpu().numpy(), r))
     g.check()
     assert err.value < TOL[precision], err
+
+
+# rewinds to before a block whose predecessor has no history in some chunk: the first blocks
+# of a run (levels 0 .. 15, staggered over 18 tiles) and, with 16-lag chunks, the second chunk
+# of a block at 32; then other displacements
+@pytest.mark.parametrize("steps,back,lags", [(17, 2, 0), (17, 9, 0), (17, 17, 0), (2, 2, 0), (33, 23, 16),
+                                             (33, 30, 0), (20, 6, 16)])
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+def test_rewinds_to_before_the_first_blocks(precision, steps, back, lags):
+    n1, n3 = 176, 96
+    g, ref, dt = _pair(n1, n3, 48, precision)
+    if lags:
+        g.set_conv_config(2, lags)
+    f = _fields(n1, n3, dt, 60, seed=31)
+    other = _fields(n1, n3, dt, 60, seed=32)
+    for u, v in f[:steps]:
+        g.step(u, v)
+        ref.step(u.double(), v.double())
+    for h in (g, ref):
+        for _ in range(back):
+            h.rewind()
+    err = Worst()
+    for u, v in other[steps - back:46]:
+        r = ref.step(u.double(), v.double()).cpu().numpy()
+        err.update(rel_l2(g.step(u, v).double().cpu().numpy(), r))
+    assert err.value < TOL[precision], err
