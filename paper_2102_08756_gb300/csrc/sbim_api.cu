@@ -115,6 +115,10 @@ struct sbim_ctx {
   bool halves = false;        // records may hold two |k| (half-record layout)
   int lags_per_cta = 0;       // 0: automatic
   size_t part_bytes = 0;
+  // A batch keeps a copy of this handle's arguments, and a captured graph replays with
+  // it: buffers that a new chunking outgrows then stay until the handle is destroyed.
+  bool held = false;
+  std::vector<void*> outgrown;
   bool use_ahead = false;     // time-blocked convolution (sbim_ahead.cuh)
   int ahead_lc = sbim::kAhead, ahead_chunks = 1;
   float* d_ahead = nullptr;
@@ -390,6 +394,18 @@ int choose_chunks(sbim_ctx& c) {
   return SBIM_OK;
 }
 
+// Frees a buffer that a larger one replaces, or keeps it where a batch still uses it.
+int outgrow(sbim_ctx& c, void* p) {
+  if (!p) return SBIM_OK;
+  if (c.held) {
+    c.outgrown.push_back(p);
+    return SBIM_OK;
+  }
+  CU(cudaStreamSynchronize(c.stream));
+  CU(cudaFree(p));
+  return SBIM_OK;
+}
+
 // (Re)allocate the lag-chunk partial sums for the current chunking; on failure
 // the previous buffer is kept.
 int alloc_partials(sbim_ctx& c) {
@@ -397,10 +413,7 @@ int alloc_partials(sbim_ctx& c) {
   if (need <= c.part_bytes && c.d_part) return SBIM_OK;
   void* fresh = nullptr;
   CU(cudaMalloc(&fresh, need));
-  if (c.d_part) {
-    CU(cudaStreamSynchronize(c.stream));
-    CU(cudaFree(c.d_part));
-  }
+  if (const int rc = outgrow(c, c.d_part)) return rc;
   c.d_part = fresh;
   c.part_bytes = need;
   return SBIM_OK;
@@ -474,10 +487,7 @@ bool alloc_ahead(sbim_ctx& c, size_t budget) {
       cudaGetLastError();
       return false;
     }
-    if (c.d_ahead) {
-      cudaStreamSynchronize(c.stream);
-      cudaFree(c.d_ahead);
-    }
+    outgrow(c, c.d_ahead);
     c.d_ahead = (float*)fresh;
     c.ahead_bytes = need;
   }
@@ -512,6 +522,7 @@ void release(sbim_ctx* c) {
   void* ptrs[] = {c->d_arena, c->d_part, c->d_io, c->d_lmax, c->d_tile_lmax, c->d_nonfinite, c->d_ahead};
   for (void* p : ptrs)
     if (p) cudaFree(p);
+  for (void* p : c->outgrown) cudaFree(p);
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
   if (c->io_fork) cudaEventDestroy(c->io_fork);
   if (c->io_join) cudaEventDestroy(c->io_join);
@@ -783,6 +794,8 @@ void handle_advance(sbim_handle c) {
 }
 
 bool handle_uses_ahead(sbim_handle c) { return c->use_ahead; }
+
+void handle_hold(sbim_handle c) { c->held = true; }
 
 int handle_step_by_step(sbim_handle c) {
   c->use_ahead = false;

@@ -137,6 +137,7 @@ int configure(sbim_batch_ctx* b, int shape, int lags) {
   std::vector<int> items(b->nb + 1, 0), tiles(b->nb + 1, 0);
   for (int i = 0; i < b->nb; ++i) {
     args[i] = sbim::handle_step_args(b->h[i]);
+    sbim::handle_hold(b->h[i]);
     tiles[i + 1] = tiles[i] + args[i].n_orb_pad / sbim::kOrbitTile;   // assembly tiles
     items[i + 1] = items[i] + (b->ahead ? sbim::ahead_ctas(args[i].n_orb_pad) * args[i].ahead_chunks
                                         : args[i].n_orb_pad / b->tile * args[i].nchunks);

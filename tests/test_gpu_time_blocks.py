@@ -227,3 +227,37 @@ def test_rewinds_to_before_the_first_blocks(precision, steps, back, lags):
         r = ref.step(u.double(), v.double()).cpu().numpy()
         err.update(rel_l2(g.step(u, v).double().cpu().numpy(), r))
     assert err.value < TOL[precision], err
+
+
+def test_member_with_a_finer_chunking_leaves_the_batch_its_buffers():
+    """A member given a finer chunking by itself needs larger buffers; the batch, and a graph
+    captured before, go on with the arguments they hold."""
+    n1, n3, n_cut = 48, 32, 90
+    stream = torch.cuda.Stream()
+    err = Worst()
+    with torch.cuda.stream(stream):
+        _, ref, dt = _pair(n1, n3, n_cut, "fp32", side=1)
+        B, b = _batch([(n1, n3)], n_cut, dt, stream)
+        member = B.sbim_batch_member(b, 0)
+        ub, vb, tb = [torch.zeros((3, n3, n1), device="cuda") for _ in range(3)]
+        B.sbim_batch_capture(b, [ub.data_ptr()], [vb.data_ptr()], [tb.data_ptr()])
+        keep = []
+        for m, (u, v) in enumerate(_fields(n1, n3, dt, 120, seed=12)):
+            if m in (40, 95):
+                B.sbim_set_conv_config(member, 2, 32 if m == 40 else 16)
+                keep.append(torch.full((1 << 22,), float("nan"), device="cuda"))
+            ub.copy_(u)
+            vb.copy_(v)
+            if m % 4 == 3 and m >= 40:
+                tau = torch.empty_like(u)
+                B.sbim_step(member, u.data_ptr(), v.data_ptr(), tau.data_ptr())
+            elif m % 2:
+                tau = _batch_step(B, b, [(u, v)])[0]
+            else:
+                B.sbim_batch_replay(b)
+                tau = tb
+            stream.synchronize()
+            r = ref.step(u.double(), v.double()).cpu().numpy()
+            err.update(rel_l2(tau.double().cpu().numpy(), r))
+        B.sbim_batch_destroy(b)
+    assert err.value < TOL["fp32"], err
