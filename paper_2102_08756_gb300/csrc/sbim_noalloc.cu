@@ -79,7 +79,8 @@ struct BinGeom {
 // multiply-adds per SM and clock: the library's square root and the quotients of the
 // bin's whole geometry, formed here for every chunk, took most of the kernel (188 us
 // for 256 x 256 x 500 lags, 141 without).  One Newton step from the float reciprocal
-// root (relative error 1.5 e^2, e ~ 1e-7) gives |k| to ~2e-14.
+// root (relative error 1.5 e^2, e ~ 1e-7) gives |k| to ~2e-14, and one step of Heron's
+// method with the residual s - q^2 in one rounding makes it a double's.
 __device__ __forceinline__ double bin_dT(const NAArgs& a, int b) {
   const int j1 = b % a.nh, r3 = b / a.nh;
   const int j3 = r3 <= a.n3 / 2 ? r3 : r3 - a.n3;
@@ -87,7 +88,8 @@ __device__ __forceinline__ double bin_dT(const NAArgs& a, int b) {
   const double s = k1 * k1 + k3 * k3;
   if (!(s > 1e-30 && s < 1e30)) return sqrt(s) * a.cs_dt;   // k = 0, and past a float's range
   const double r = rsqrtf((float)s);
-  return s * (r * (1.5 - 0.5 * s * r * r)) * a.cs_dt;
+  const double q = s * (r * (1.5 - 0.5 * s * r * r));
+  return fma(fma(-q, q, s), 0.5 * r, q) * a.cs_dt;
 }
 
 __device__ BinGeom bin_geom(const NAArgs& a, int b) {
