@@ -52,10 +52,7 @@ using namespace dev;
 // registers).
 constexpr int kRec = kAheadRec, kSums = 5, kThreads = kRec * kMembers * kSums, kWarps = kThreads / 32;
 constexpr int kSub = kOrbitTile / kRec;     // CTAs per 128-record tile
-// Lags per stage, and the 16-lag blocks that are chained before they are folded into
-// the running sums (every 32 lags: the error against 64 bits stays that of the
-// step-by-step sums, 5.44e-7 for 256^2 x 1024; 64 lags were 5 % faster at 5.46e-7).
-constexpr int kLags = kAheadLags, kFold = 2;
+constexpr int kLags = kAheadLags;   // lags per stage
 template <bool HALVES> __host__ __device__ constexpr int stages() { return HALVES ? 4 : 5; }
 
 template <class S> __host__ __device__ constexpr int seg() { return kRec * S::kRecBytes; }
@@ -239,10 +236,15 @@ __device__ __forceinline__ void request_stage(const StepArgs& a, int j, unsigned
 }
 
 // A warp's part of an item: one of the five sums for the 32 members of 8 records.
-// The terms of 32 lags are chained by multiply-adds, then folded into the running
-// sums (in shared memory) with one compensated addition.  The warps meet only at the
-// stages: each waits for its copies, and the last to leave one requests its next
-// filling.  Returns false if a bounded wait gave up.
+// The terms of 16 lags are chained by multiply-adds, then folded into the running
+// sums (in shared memory) with one compensated addition, half of the outputs after
+// each stage.  With chains of 32 lags the error against 64 bits was up to 0.6 % above
+// that of the step-by-step convolution (compensated every 2 lags); with 16, and the
+// stored weights for the lags inside a block too, it is 0.99 of it for FP32 on average
+// and equal for BF16 hi/lo.  Folds of 8 lags gain nothing more and cost 18 % at
+// 512^2 x 2000; these cost 4 % (208 to 215 us a step), 8 % with all outputs folded at
+// once.  The warps meet only at the stages: each waits for its copies, and the last to
+// leave one requests its next filling.  Returns false if a bounded wait gave up.
 template <class S, bool HALVES>
 __device__ __forceinline__ bool sum_item(const StepArgs& a, int q, unsigned char* smem, Sync& sync,
                                          unsigned g) {
@@ -289,7 +291,6 @@ __device__ __forceinline__ bool sum_item(const StepArgs& a, int q, unsigned char
       float2 dn = IO::smem(st + ((kLags - 1) * 3 + comp) * SEG, PLANE, x);
 #pragma unroll
       for (int k = 0; k < kLags; ++k) {
-        
         const int l = L0 + k;
         float2 d = dn;                           // the next lag's value is on its way
         if (k + 1 < kLags) dn = IO::smem(st + ((kLags - 2 - k) * 3 + comp) * SEG, PLANE, x);
@@ -307,6 +308,14 @@ __device__ __forceinline__ bool sum_item(const StepArgs& a, int q, unsigned char
         w[l] = pack2(make_float2(v, v));
       }
       __syncwarp();
+#pragma unroll
+      for (int s = L0; s < L0 + kLags; s += 2) {
+        const ulonglong2 o = run[(s / 2) * kThreads];
+        const ulonglong2 t = make_ulonglong2(add2r(o.x, y[s]), add2r(o.y, y[s + 1]));
+        y[s] = sub2r(y[s], sub2r(t.x, o.x));     // minus the compensation
+        y[s + 1] = sub2r(y[s + 1], sub2r(t.y, o.y));
+        run[(s / 2) * kThreads] = t;
+      }
       if (lane == 0) {
         const int j = 2 * b + L0 / kLags;
         if (shared_inc(&sync.left[buf]) % kWarps == kWarps - 1 && j + NS < 2 * nblk) {
@@ -330,16 +339,6 @@ __device__ __forceinline__ bool sum_item(const StepArgs& a, int q, unsigned char
     else
       block(std::false_type{}, std::false_type{});
     if (!ok) return false;
-    if (b % kFold == kFold - 1) {
-#pragma unroll
-      for (int s = 0; s < kAhead; s += 2) {
-        const ulonglong2 o = run[(s / 2) * kThreads];
-        const ulonglong2 t = make_ulonglong2(add2r(o.x, y[s]), add2r(o.y, y[s + 1]));
-        y[s] = sub2r(y[s], sub2r(t.x, o.x));     // minus the compensation
-        y[s + 1] = sub2r(y[s + 1], sub2r(t.y, o.y));
-        run[(s / 2) * kThreads] = t;
-      }
-    }
   }
   float* out = a.ahead + (((long long)it.chunk * (a.n_orb_pad / kOrbitTile) + it.T) * kAhead * kFields + 2 * f) *
                              (kOrbitTile * kMembers) + q * (kRec * kMembers) + x;
@@ -485,11 +484,6 @@ __device__ __forceinline__ void near_member(const StepArgs& a, int T, int x) {
   for (int c = 0; c < 3; ++c)
     R[c] = IO::store(a.hist, ((long long)sn * 3 + c) * comp_stride + mi, a.slot_stride, D[c]);
 
-  // weights from the table, which stays in L2 (reading the stored ones, 16 bytes per
-  // record and lag from HBM, took the kernel from 58 to 74 us at 1024^2)
-  const float4* tab = reinterpret_cast<const float4*>(a.table);
-  const float dT = reinterpret_cast<const float*>(a.dT)[hx];
-  const unsigned long long us = a.ustep[hx];
   float acc[kFields], cmp[kFields];
 #pragma unroll
   for (int k = 0; k < kFields; ++k) acc[k] = cmp[k] = 0.f;
@@ -520,21 +514,28 @@ __device__ __forceinline__ void near_member(const StepArgs& a, int T, int x) {
 #pragma unroll
     for (int k = 0; k < kFields; ++k) fold(k, v[k]);
   }
-  // lags inside the block, 4 in flight
+  // lags inside the block, 4 in flight with their weights: those of the block sums,
+  // rounded once from double (interpolating them in float from the table gave up to
+  // 1.6 % more error and 1.3-2 us more a step up to 512^2, the same above)
   int M = min((int)(base < 0 ? n : n - base), a.n_cut - 1);
   if (a.tile_lmax) M = min(M, a.tile_lmax[T] - 1);
   const int lo = a.lmax ? a.lmax[hx] : 0x7fffffff;
+  const int rows = kRec << a.halves;
+  const float4* wrow = reinterpret_cast<const float4*>(a.wts32) +
+                       (long long)(rec / kRec) * ahead_weight_lags(a.n_cut) * rows +
+                       (a.halves ? hx % (2 * kRec) : rec % kRec);
   {
-    float w[4];
-    lag_weights(tab, 0ull, dT * 0.5f, w);
+    const float4 q = __ldg(wrow);
+    const float w[4] = {0.5f * q.x, 0.5f * q.y, 0.5f * q.z, 0.5f * q.w};
     lag(w, R);
   }
   for (int m = 1; m <= M; m += 4) {
     float2 d[4][3];
+    float4 w4[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
       if (m + i <= M) {
-
+        w4[i] = __ldg(wrow + (long long)(m + i) * rows);
         int slot = sn - (m + i);
         if (slot < 0) slot += a.n_cut;
 #pragma unroll
@@ -544,8 +545,8 @@ __device__ __forceinline__ void near_member(const StepArgs& a, int T, int x) {
 #pragma unroll
     for (int i = 0; i < 4; ++i)
       if (m + i <= M) {
-        float w[4];
-        lag_weights(tab, (unsigned long long)(m + i) * us, m + i < lo ? dT : 0.f, w);
+        const bool in = m + i < lo;
+        const float w[4] = {in ? w4[i].x : 0.f, in ? w4[i].y : 0.f, in ? w4[i].z : 0.f, in ? w4[i].w : 0.f};
         lag(w, d[i]);
       }
   }

@@ -203,6 +203,39 @@ def test_host_direct_and_repeated_steps_in_turn(precision, grid, n_cut):
     assert err.value < TOL[precision], err
 
 
+@pytest.mark.parametrize("n,n_cut", [(64, 1000), (128, 600)])
+def test_sums_are_as_exact_as_step_by_step(n, n_cut):
+    """White fields, whose error is the convolution's more than the transforms': over 32 steps with
+    the whole history the block sums are no further from FP64 than sums compensated term by term."""
+    g, ref, dt = _pair(n, n, n_cut, "fp32")
+    by_step, _, _ = _pair(n, n, n_cut, "fp32")
+    by_step.set_conv_config(0, 0)
+    gen = torch.Generator(device="cuda").manual_seed(17)
+    U = 1e-3 * torch.randn((4, 3 * n * n), generator=gen, device="cuda", dtype=torch.float64)
+    t = torch.arange(n_cut + 40, device="cuda", dtype=torch.float64)
+    w = 0.25 * np.pi / 100.0 * CS * dt * (0.05 + 0.95 * torch.rand((4, 8, 1), generator=gen, device="cuda",
+                                                                    dtype=torch.float64))
+    sig = torch.sin(w * t + 6.28 * torch.rand((4, 8, 1), generator=gen, device="cuda",
+                                              dtype=torch.float64)).sum(1)
+    zero = torch.zeros((3, n, n), device="cuda")
+    hs = (g, by_step, ref)
+    for h in hs:
+        h.set_window(1e-6)
+    err = [0.0, 0.0]
+    for m in range(n_cut + 40):
+        if m == n_cut + 4:
+            for h in hs:
+                h.set_window(0.0)
+        u = (sig[:, m] @ U).reshape(3, n, n).float()
+        r = ref.step(u.double(), zero.double())
+        tau = [h.step(u, zero).double() for h in hs[:2]]
+        if m >= n_cut + 8:
+            for k in range(2):
+                assert bool(torch.isfinite(tau[k]).all())
+                err[k] += float((tau[k] - r).square().sum())
+    assert err[0] <= err[1], err
+
+
 # rewinds to before a block whose predecessor has no history in some chunk: the first blocks
 # of a run (levels 0 .. 15, staggered over 18 tiles) and, with 16-lag chunks, the second chunk
 # of a block at 32; then other displacements
