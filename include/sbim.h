@@ -80,8 +80,9 @@ typedef enum {
  * fit in free device memory.  An SBIM_FP64 handle also keeps its convolution
  * weights, computed once (n_cut x n_slots x 8 bytes; 17.3 GB at 1024^2 x 4096),
  * when they fit with 512 MB to spare; otherwise it interpolates them from the
- * table every step, with the same result to rounding.  *out is written on
- * success only.
+ * table every step, with the same result to rounding.  A float-class handle takes
+ * the memory of its block sums at its first step, if there is room
+ * (sbim_set_time_blocks).  *out is written on success only.
  */
 int sbim_create(sbim_handle* out, int n1, int n3, double L1, double L3,
                 double cs, double cp, double rho, double dt, int n_cut,
@@ -275,6 +276,31 @@ int sbim_stage_times(sbim_handle h, double ms[5], long long* steps);
  * previous configuration is kept.
  */
 int sbim_set_conv_config(sbim_handle h, int variant, int lags_per_cta);
+
+/*
+ * sbim_set_time_blocks / sbim_get_time_blocks -- how a float-class handle forms the
+ * convolution of Eq. (SBI) (Section 2.3): blocked in time (enable != 0, the
+ * default), one pass over the history forming the sums of 16 consecutive steps, or
+ * step by step (0).  Block sums need device memory beside the handle's own: their
+ * weights (16 bytes per record and lag, 32 for half records: 17 % of an FP32 ring, 33
+ * or 67 % of a BF16 hi-only one; a record is 4 slots of sbim_get_info) and the sums
+ * (2,560 bytes per record and lag chunk).  It is taken at the handle's first step (or
+ * when a batch is made of it), not at its creation, and only where at least as much
+ * stays free, and room for another handle of this size if there was any; otherwise
+ * the handle convolves step by step, several times slower on long histories, with
+ * the same result to rounding.  Both forms may serve one handle in turn.
+ *   set 0 returns the memory (synchronising the stream; a handle in a batch keeps it)
+ *     and steps step by step from then on; set 1 lets the next step decide again, as
+ *     sbim_set_conv_config does.  The batch itself follows its members at its next
+ *     sbim_batch_set_conv_config or sbim_batch_set_conv_tile.  Graphs that a caller
+ *     captured from this handle's steps must be captured again.
+ *   get tells whether the next step takes block sums (deciding it if no step has yet).
+ * A first step under stream capture allocates nothing and goes step by step.  FP64
+ * handles, variant 0 and very short hi-only BF16 histories (n_cut < 28) on planes of
+ * 16,384 whole records and more always do.  Library utility: the paper has no counterpart.
+ */
+int sbim_set_time_blocks(sbim_handle h, int enable);
+int sbim_get_time_blocks(sbim_handle h, int* enabled);
 
 /*
  * sbim_set_conv_tile -- orbit records per CTA of the TMA-staged convolution

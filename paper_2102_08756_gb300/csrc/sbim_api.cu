@@ -119,21 +119,28 @@ struct sbim_ctx {
   // it: buffers that a new chunking outgrows then stay until the handle is destroyed.
   bool held = false;
   std::vector<void*> outgrown;
-  bool use_ahead = false;     // time-blocked convolution (sbim_ahead.cuh)
+  // Time-blocked convolution (sbim_ahead.cuh): 1, step by step: 0, or decided by the
+  // memory that is free at the next step: -1.
+  int blocks = -1;
+  bool blocks_off = false;    // the caller wants no block sums
   int ahead_lc = sbim::kAhead, ahead_chunks = 1;
-  float* d_ahead = nullptr;
-  size_t ahead_bytes = 0;
-  long long* d_stamp = nullptr;
-  size_t stamp_bytes = 0;
+  // One allocation of its own, made at the first step: ring map, weights, stamps, sums.
+  void* d_extra = nullptr;
   void* d_tmap = nullptr;     // CUtensorMap of the ring
   void* d_wts32 = nullptr;    // the block sums' weights
+  long long* d_stamp = nullptr;
+  size_t stamp_bytes = 0;
+  float* d_ahead = nullptr;   // the sums: in d_extra, or d_ahead_own once a finer chunking outgrew that
+  float* d_ahead_own = nullptr;
+  size_t ahead_bytes = 0;
+  size_t need = 0;            // device memory of a handle without block sums
   int config_id = 0;          // counts changes of chunking and window (part of the stamps)
   double tab_h = 0;
   long long tab_n = 0;
   size_t real_size = 4;
 
-  // One allocation holds the plan, tables, ring, spectra and weights below (a handle
-  // with 18 of its own took 2 ms more to create and destroy on GB300).
+  // One allocation holds the plan, tables, ring, spectra, partial sums and FP64 weights
+  // below (a handle with 18 of its own took 2 ms more to create and destroy on GB300).
   void* d_arena = nullptr;
   int* d_bin = nullptr;
   void* d_dir = nullptr;  // float2, or double2 for the FP64 path
@@ -147,7 +154,8 @@ struct sbim_ctx {
   void* d_hist = nullptr;
   size_t hist_bytes = 0;
   long long plane_records = 0;
-  void* d_part = nullptr;
+  void* d_part = nullptr;      // in the arena, or d_part_own once a finer chunking outgrew that
+  void* d_part_own = nullptr;
   void* d_uhat = nullptr;
   void* d_fhat = nullptr;
   void* d_s = nullptr;
@@ -170,7 +178,8 @@ struct sbim_ctx {
   bool have_fwd = false, have_inv = false;
 
   long long n = 0;
-  bool can_repeat = false;    // the partial sums hold the last forward level
+  bool can_repeat = false;    // the sums hold the last forward level,
+  bool level_blocks = false;  // which took block sums
   double tau_inf[3] = {0, 0, 0};
 
   bool prof = false;
@@ -410,11 +419,11 @@ int outgrow(sbim_ctx& c, void* p) {
 // the previous buffer is kept.
 int alloc_partials(sbim_ctx& c) {
   const size_t need = (size_t)c.nchunks * 4 * sbim::kFields * c.n_orb_pad * c.real_size;
-  if (need <= c.part_bytes && c.d_part) return SBIM_OK;
+  if (need <= c.part_bytes) return SBIM_OK;
   void* fresh = nullptr;
   CU(cudaMalloc(&fresh, need));
-  if (const int rc = outgrow(c, c.d_part)) return rc;
-  c.d_part = fresh;
+  if (const int rc = outgrow(c, c.d_part_own)) return rc;
+  c.d_part = c.d_part_own = fresh;
   c.part_bytes = need;
   return SBIM_OK;
 }
@@ -451,8 +460,8 @@ size_t ahead_need(const sbim_ctx& c) {
 }
 
 // Marks every block sum as not formed.
-int forget_ahead(sbim_ctx* c) {
-  if (c->d_stamp) CU(cudaMemsetAsync(c->d_stamp, 0xff, c->stamp_bytes, c->stream));
+int forget_ahead(sbim_ctx* c, cudaStream_t st) {
+  if (c->d_stamp) CU(cudaMemsetAsync(c->d_stamp, 0xff, c->stamp_bytes, st));
   return SBIM_OK;
 }
 
@@ -475,51 +484,128 @@ int make_ring_map(const sbim_ctx& c, CUtensorMap* map) {
   return SBIM_OK;
 }
 
-// Room for the block sums of the current chunking in at most `budget` bytes; false if
-// there is none, or none was left at creation for their weights (the caller then
-// convolves step by step).
-bool alloc_ahead(sbim_ctx& c, size_t budget) {
-  if (!c.d_wts32) return false;
-  const size_t need = ahead_need(c);
-  if (need > c.ahead_bytes) {
-    void* fresh = nullptr;
-    if (need > budget || cudaMalloc(&fresh, need) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    outgrow(c, c.d_ahead);
-    c.d_ahead = (float*)fresh;
-    c.ahead_bytes = need;
-  }
-  return forget_ahead(&c) == SBIM_OK;
+// Whether `bytes` for block sums may be taken: at most half of what is free, never the
+// last 256 MB, and never the room of another handle of this size.
+int have_room(const sbim_ctx& c, size_t bytes, bool* room) {
+  size_t free_b = 0, total_b = 0;
+  CU(cudaMemGetInfo(&free_b, &total_b));
+  const size_t another = c.need + kSpareBytes;
+  *room = bytes + kSpareBytes <= free_b && bytes <= free_b / 2 &&
+          (free_b < another || free_b - bytes >= another);
+  return SBIM_OK;
 }
 
-// Launch, chunking and sums buffer for the current variant, tile and lags_per_cta.
-int configure_conv(sbim_ctx& c) {
-  ++c.config_id;
-  c.use_ahead = false;
-  int rc = choose_chunks(c);
-  if (rc != SBIM_OK) return rc;
-  if (c.d_wts32 && c.variant >= 1) {
-    int dev = 0, sms = 148;
-    CU(cudaGetDevice(&dev));
-    CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    choose_ahead(c, sms);
-    size_t free_b = 0, total_b = 0;
-    CU(cudaMemGetInfo(&free_b, &total_b));
-    if (alloc_ahead(c, free_b > kSpareBytes ? free_b - kSpareBytes : 0)) {
-      c.use_ahead = true;
+// Room for the sums of the current chunking, and everything that goes with them if this
+// is the first time; *ok is false where there is none.
+int start_blocks(sbim_ctx* c, cudaStream_t st, bool* ok) {
+  *ok = false;
+  // On large planes of whole records a very short BF16 history is read faster than the lags
+  // inside a block are added (1024^2, hi-only, us a step: 16 lags 129 step by step against
+  // 143, 24 lags 141 / 150, 39 lags 162 / 151; hi/lo, 16 lags: 163 / 152; half records,
+  // 1024 x 500, 20 lags: 96 / 90).
+  const int least = c->prec == SBIM_BF16 && !c->halves && c->n_orb_pad >= 16384 ? 28 : 0;
+  if (c->prec == SBIM_FP64 || c->variant < 1 || c->blocks_off || c->n_cut < least) return SBIM_OK;
+  const size_t sums = ahead_need(*c);
+  if (!c->d_extra) {
+    const size_t w32 = sbim::ahead_weight_bytes(c->n_orb_pad, c->n_cut, c->halves);
+    // a stamp for every chunk that any chunking can have: they stay where they are when
+    // the chunking changes, so that a batch's own copy of the arguments stays consistent
+    const size_t stamps = (size_t)((c->n_cut + sbim::kAhead - 1) / sbim::kAhead) *
+                          (c->n_orb_pad / sbim::kAheadRec) * sizeof(long long);
+    const size_t o_stamp = 256 + w32, o_sums = o_stamp + (stamps + 255) / 256 * 256;
+    bool room;
+    if (const int rc = have_room(*c, o_sums + sums, &room)) return rc;
+    if (!room) return SBIM_OK;
+    if (!c->sums.side) CU(sbim::pair_init(c->sums));
+    CU(sbim::launch_ahead(sbim::StepArgs{}, c->prec, 0, c->halves, st));
+    CUtensorMap map;
+    std::memset(&map, 0, sizeof map);
+    if (c->n_cut >= sbim::kAheadLags)   // shorter rings always wrap: copied row by row
+      if (const int rc = make_ring_map(*c, &map)) return rc;
+    if (cudaMalloc(&c->d_extra, o_sums + sums) != cudaSuccess) {
+      c->d_extra = nullptr;
+      cudaGetLastError();
       return SBIM_OK;
     }
+    c->d_tmap = c->d_extra;
+    c->d_wts32 = (char*)c->d_extra + 256;
+    c->d_stamp = (long long*)((char*)c->d_extra + o_stamp);
+    c->stamp_bytes = stamps;
+    c->d_ahead = (float*)((char*)c->d_extra + o_sums);
+    c->ahead_bytes = sums;
+    CU(cudaMemcpyAsync(c->d_tmap, &map, sizeof map, cudaMemcpyHostToDevice, st));
+    CU(sbim::launch_ahead(step_args(c), c->prec, 3, c->halves, st));
+  } else if (sums > c->ahead_bytes) {
+    bool room;
+    if (const int rc = have_room(*c, sums, &room)) return rc;
+    void* fresh = nullptr;
+    if (!room || cudaMalloc(&fresh, sums) != cudaSuccess) {
+      cudaGetLastError();
+      return SBIM_OK;
+    }
+    if (const int rc = outgrow(*c, c->d_ahead_own)) return rc;
+    c->d_ahead = c->d_ahead_own = (float*)fresh;
+    c->ahead_bytes = sums;
   }
-  return alloc_partials(c);
+  *ok = true;
+  return forget_ahead(c, st);
+}
+
+// Decides, before a step on `st`, how an undecided handle convolves.  Block sums need
+// memory that no handle needs to be created: it is taken at the first step, when a
+// program's other handles usually exist.  Nothing is allocated under stream capture: a
+// handle that is first stepped there goes step by step and stays undecided.
+int ready(sbim_ctx* c, cudaStream_t st) {
+  if (c->blocks >= 0) return SBIM_OK;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return SBIM_OK;
+  }
+  if (cap != cudaStreamCaptureStatusNone) return SBIM_OK;
+  // (allocations would break a capture that another thread has under way)
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  CU(cudaThreadExchangeStreamCaptureMode(&mode));
+  bool ok = false;
+  const int rc = start_blocks(c, st, &ok);
+  CU(cudaThreadExchangeStreamCaptureMode(&mode));
+  if (rc == SBIM_OK) c->blocks = ok ? 1 : 0;
+  return rc;
+}
+
+// Gives the block sums' memory back.
+int drop_blocks(sbim_ctx* c) {
+  if (c->held || !c->d_extra) return SBIM_OK;
+  CU(cudaStreamSynchronize(c->stream));
+  CU(cudaFree(c->d_ahead_own));
+  c->d_ahead_own = nullptr;
+  CU(cudaFree(c->d_extra));
+  c->d_extra = c->d_tmap = c->d_wts32 = nullptr;
+  c->d_stamp = nullptr;
+  c->d_ahead = nullptr;
+  c->stamp_bytes = c->ahead_bytes = 0;
+  return SBIM_OK;
+}
+
+// Chunking and buffers for the current variant, tile and lags_per_cta.
+int configure_conv(sbim_ctx& c) {
+  if (const int rc = choose_chunks(c)) return rc;
+  if (const int rc = alloc_partials(c)) return rc;
+  int dev = 0, sms = 148;
+  CU(cudaGetDevice(&dev));
+  CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  choose_ahead(c, sms);
+  ++c.config_id;
+  c.blocks = -1;
+  return SBIM_OK;
 }
 
 void release(sbim_ctx* c) {
   if (!c) return;
   if (c->have_fwd) cufftDestroy(c->plan_fwd);
   if (c->have_inv) cufftDestroy(c->plan_inv);
-  void* ptrs[] = {c->d_arena, c->d_part, c->d_io, c->d_lmax, c->d_tile_lmax, c->d_nonfinite, c->d_ahead};
+  void* ptrs[] = {c->d_arena,  c->d_part_own,  c->d_io,    c->d_lmax, c->d_tile_lmax,
+                  c->d_nonfinite, c->d_ahead_own, c->d_extra};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (void* p : c->outgrown) cudaFree(p);
@@ -592,8 +678,8 @@ int create_impl(sbim_ctx* c) {
   const size_t cplx = 2 * c->real_size;
   size_t free_b = 0, total_b = 0;
   CU(cudaMemGetInfo(&free_b, &total_b));
-  // (the partial sums of a step-by-step convolution: the least a handle needs)
-  const size_t need = c->hist_bytes + part_bytes + 2 * 3 * (size_t)c->nbins * cplx +
+  // (block sums take memory of their own, if there is any, at the first step)
+  const size_t need = c->need = c->hist_bytes + part_bytes + 2 * 3 * (size_t)c->nbins * cplx +
                       4 * c->field_elems() * c->real_size + (size_t)c->tab_n * 48;
   if (need + kSpareBytes > free_b)
     return fail(SBIM_ERR_OOM, "need %.2f GB of device memory, %.2f GB free",
@@ -604,25 +690,6 @@ int create_impl(sbim_ctx* c) {
     const size_t wb = (size_t)c->n_cut * c->n_orb_pad * 32;
     if (need + wb + (512ull << 20) <= free_b) c->wts_bytes = wb;
   }
-
-  // The block sums' weights (16 B per record and lag beside 96 of FP32 history, 32 for
-  // half records) and the least room for the sums themselves; a handle that has none
-  // left convolves step by step.  Half-spaces come in pairs (the two sides of a slab or
-  // a fault, an update and its transpose): these extras never take the room of a second
-  // handle of this size that would fit without them.
-  const size_t w32 = dbl ? 0 : sbim::ahead_weight_bytes(c->n_orb_pad, c->n_cut, c->halves);
-  const size_t extras = w32 + (size_t)c->n_orb_pad * 4096 + kSpareBytes;
-  // On large planes of whole records a very short BF16 history is read faster than the lags
-  // inside a block are added (1024^2, hi-only, us a step: 16 lags 129 step by step against
-  // 143, 24 lags 141 / 150, 39 lags 162 / 151; hi/lo, 16 lags: 163 / 152; half records,
-  // 1024 x 500, 20 lags: 96 / 90).
-  const int least = c->prec == SBIM_BF16 && !c->halves && c->n_orb_pad >= 16384 ? 28 : 0;
-  const bool blocked = w32 && c->n_cut >= least && need + extras <= free_b &&
-                       (2 * need + extras <= free_b || 2 * need + kSpareBytes > free_b);
-  // a stamp for every chunk that any chunking can have: they stay where they are when
-  // the chunking changes, so that a batch's own copy of the arguments stays consistent
-  c->stamp_bytes = blocked ? (size_t)((c->n_cut + sbim::kAhead - 1) / sbim::kAhead) *
-                                 (c->n_orb_pad / sbim::kAheadRec) * sizeof(long long) : 0;
 
   // Lay the arena out: what the host fills in first, in one copy, then the rest.
   size_t at = 0;
@@ -640,7 +707,6 @@ int create_impl(sbim_ctx* c) {
   const size_t o_muq = put(&c->d_muq, o2 * c->real_size);
   const size_t o_us = put((void**)&c->d_ustep, o2 * sizeof(unsigned long long));
   const size_t o_gl = put((void**)&c->d_gl, 32 * sizeof(double));
-  const size_t o_map = put(&c->d_tmap, sizeof(CUtensorMap));
   put((void**)&c->d_step, sizeof(long long));   // zero, like the error word
   put((void**)&c->d_err, sizeof(int));
   const size_t filled = at;
@@ -649,10 +715,8 @@ int create_impl(sbim_ctx* c) {
   put(&c->d_uhat, 3 * (size_t)c->nbins * cplx);
   put(&c->d_fhat, 3 * (size_t)c->nbins * cplx);
   put(&c->d_s, c->field_elems() * c->real_size);
-  if (blocked) {
-    put(&c->d_wts32, w32);
-    put((void**)&c->d_stamp, c->stamp_bytes);
-  }
+  put(&c->d_part, part_bytes);
+  c->part_bytes = part_bytes;
   if (c->wts_bytes) put(&c->d_wts, c->wts_bytes);
   put(&c->d_hist, c->hist_bytes);
   CU(cudaMalloc(&c->d_arena, at));
@@ -675,21 +739,11 @@ int create_impl(sbim_ctx* c) {
   }
   std::memcpy(&host[o_us], ustep.data(), o2 * sizeof(unsigned long long));
   gauss_legendre16((double*)&host[o_gl], (double*)&host[o_gl] + 16);
-  if (blocked && c->n_cut >= sbim::kAheadLags) {   // shorter rings always wrap: copied row by row
-    CUtensorMap map;
-    if (const int rc = make_ring_map(*c, &map)) return rc;
-    std::memcpy(&host[o_map], &map, sizeof map);
-  }
   cudaStream_t st = c->stream;
   CU(cudaMemcpyAsync(c->d_arena, host.data(), filled, cudaMemcpyHostToDevice, st));
   CU(sbim::launch_table_build(c->d_tab64, c->d_tab32, c->tab_n, c->tab_h, c->eta, c->d_gl,
                               c->d_gl + 16, st));
   if (c->d_wts) CU(sbim::launch_weights64(step_args(c), c->d_wts, st));
-  if (blocked) {
-    CU(sbim::pair_init(c->sums));
-    CU(sbim::launch_ahead(step_args(c), c->prec, 0, c->halves, st));
-    CU(sbim::launch_ahead(step_args(c), c->prec, 3, c->halves, st));
-  }
   if (const int rc = configure_conv(*c)) return rc == SBIM_ERR_CUDA ? rc : SBIM_ERR_OOM;
   CU(cudaStreamSynchronize(st));
 
@@ -793,13 +847,17 @@ void handle_advance(sbim_handle c) {
   c->can_repeat = false;   // the batch kept its partial sums in its own buffers
 }
 
-bool handle_uses_ahead(sbim_handle c) { return c->use_ahead; }
+int handle_uses_ahead(sbim_handle c, bool* blocks) {
+  const int rc = ready(c, c->stream);
+  *blocks = c->blocks == 1;
+  return rc;
+}
 
 void handle_hold(sbim_handle c) { c->held = true; }
 
 int handle_step_by_step(sbim_handle c) {
-  c->use_ahead = false;
-  return alloc_partials(*c);
+  c->blocks = 0;
+  return drop_blocks(c);
 }
 
 int handle_shape(sbim_handle c, int* precision, int* kahan, int* variant, void** stream) {
@@ -913,6 +971,11 @@ int run_step(sbim_ctx* c, const void* in, const void* aux, void* out, bool adjoi
     const int rc = check_inputs(c, in, adjoint ? nullptr : aux, st);
     if (rc != SBIM_OK) return rc;
   }
+  if (!repeat) {
+    if (const int rc = ready(c, st)) return rc;
+    c->level_blocks = c->blocks == 1;
+  }
+  const bool blocks = c->level_blocks;
   if (repeat) {                     // back to the level being re-evaluated
     CU(sbim::launch_rewind(c->d_step, st));
     --c->n;
@@ -928,7 +991,7 @@ int run_step(sbim_ctx* c, const void* in, const void* aux, void* out, bool adjoi
   }
   const sbim::StepArgs a = step_args(c);
   // (a repeated level finds its block sums formed: they end before the block)
-  const bool sums = c->use_ahead && !repeat, beside = sums && !e;
+  const bool sums = blocks && !repeat, beside = sums && !e;
   if (beside)
     if (const int rc = fork_sums(c, a, st)) return rc;
   if (const int rc = sbim::handle_fft_forward(c, in, st)) return rc;
@@ -937,7 +1000,7 @@ int run_step(sbim_ctx* c, const void* in, const void* aux, void* out, bool adjoi
     CU(cudaStreamWaitEvent(st, c->sums.join, 0));
   else if (sums)
     CU(sbim::launch_ahead(a, c->prec, 1, c->halves, st));
-  if (c->use_ahead) {
+  if (blocks) {
   } else if (repeat)
     CU(sbim::launch_repeat_lag0(a, c->prec, st));
   else if (c->variant >= 1)
@@ -945,7 +1008,7 @@ int run_step(sbim_ctx* c, const void* in, const void* aux, void* out, bool adjoi
   else
     CU(sbim::launch_conv(a, c->prec, c->kahan, st));
   if (e) CU(cudaEventRecord(e[2], st));
-  if (c->use_ahead)
+  if (blocks)
     CU(sbim::launch_ahead(a, c->prec, 2, c->halves, st));
   else
     CU(sbim::launch_assemble(a, c->prec, c->kahan, st));
@@ -1000,13 +1063,17 @@ bool handle_raw_ok(sbim_handle c) { return !c->prof && !c->check_finite; }
 // advances the counter (handle_counter on the device, handle_advanced on the host) once
 // the level is final.
 int handle_raw_step(sbim_handle c, const void* in, void* out, bool again, cudaStream_t st) {
+  if (!again) {
+    if (const int rc = ready(c, st)) return rc;
+    c->level_blocks = c->blocks == 1;
+  }
   const sbim::StepArgs a = step_args(c);
-  const bool sums = c->use_ahead && !again;
+  const bool blocks = c->level_blocks, sums = blocks && !again;
   if (sums)
     if (const int rc = fork_sums(c, a, st)) return rc;
   if (const int rc = handle_fft_forward(c, in, st)) return rc;
   if (sums) CU(cudaStreamWaitEvent(st, c->sums.join, 0));
-  if (c->use_ahead) {
+  if (blocks) {
     CU(launch_ahead(a, c->prec, 2, c->halves, st));
   } else {
     if (again) CU(launch_repeat_lag0(a, c->prec, st));
@@ -1105,6 +1172,8 @@ int sbim_step_host(sbim_handle h, const void* u, const void* v, void* tau) {
       CU(cudaEventCreateWithFlags(&c->io_fork, cudaEventDisableTiming));
       CU(cudaEventCreateWithFlags(&c->io_join, cudaEventDisableTiming));
     }
+    if (const int rc = ready(c, st)) return rc;
+    const bool blocks = c->level_blocks = c->blocks == 1;
     CU(cudaEventRecord(c->io_fork, st));
     CU(cudaStreamWaitEvent(c->io_stream, c->io_fork, 0));
     CU(cudaMemcpyAsync(du, u, bytes, cudaMemcpyHostToDevice, c->io_stream));
@@ -1114,7 +1183,7 @@ int sbim_step_host(sbim_handle h, const void* u, const void* v, void* tau) {
     CU(cudaEventRecord(c->io_join, c->io_stream));
     sbim::StepArgs a = step_args(c);
     a.uhat = zero_hat;
-    if (c->use_ahead)
+    if (blocks)
       CU(sbim::launch_ahead(a, c->prec, 1, c->halves, st));
     else if (c->variant >= 1)
       CU(sbim::launch_conv_tma(a, c->prec, c->kahan, c->variant, st, nullptr, c->tile, c->halves));
@@ -1122,7 +1191,7 @@ int sbim_step_host(sbim_handle h, const void* u, const void* v, void* tau) {
       CU(sbim::launch_conv(a, c->prec, c->kahan, st));
     CU(cudaStreamWaitEvent(st, c->io_join, 0));
     a.uhat = c->d_uhat;
-    if (c->use_ahead) {
+    if (blocks) {
       CU(sbim::launch_ahead(a, c->prec, 2, c->halves, st));
     } else {
       CU(sbim::launch_repeat_lag0(a, c->prec, st));
@@ -1147,7 +1216,7 @@ int sbim_set_window(sbim_handle h, double window) {
   if (!(window >= 0)) return fail(SBIM_ERR_ARG, "window must be >= 0");
   h->can_repeat = false;
   ++h->config_id;
-  if (const int rc = forget_ahead(h)) return rc;
+  if (const int rc = forget_ahead(h, h->stream)) return rc;
   if (window == 0) {
     h->window = 0;
     return SBIM_OK;
@@ -1206,8 +1275,6 @@ int sbim_set_conv_config(sbim_handle h, int variant, int lags_per_cta) {
   if (lags_per_cta < 0) return fail(SBIM_ERR_ARG, "lags_per_cta must be >= 0");
   h->can_repeat = false;
   const int old_v = h->variant, old_l = h->lags_per_cta, old_lc = h->lc, old_nc = h->nchunks;
-  const int old_alc = h->ahead_lc, old_anc = h->ahead_chunks;
-  const bool old_ahead = h->use_ahead;
   h->variant = variant;
   h->lags_per_cta = lags_per_cta;
   if (variant >= 1) {
@@ -1221,7 +1288,6 @@ int sbim_set_conv_config(sbim_handle h, int variant, int lags_per_cta) {
   const int rc = configure_conv(*h);
   if (rc != SBIM_OK) {
     h->variant = old_v; h->lags_per_cta = old_l; h->lc = old_lc; h->nchunks = old_nc;
-    h->ahead_lc = old_alc; h->ahead_chunks = old_anc; h->use_ahead = old_ahead;
     return rc;
   }
   return SBIM_OK;
@@ -1236,8 +1302,6 @@ int sbim_set_conv_tile(sbim_handle h, int orbits_per_cta) {
                 h->n_orb_pad, orbits_per_cta);
   h->can_repeat = false;
   const int old_t = h->tile, old_lc = h->lc, old_nc = h->nchunks;
-  const int old_alc = h->ahead_lc, old_anc = h->ahead_chunks;
-  const bool old_ahead = h->use_ahead;
   h->tile = orbits_per_cta;
   if (h->variant >= 1) {
     const cudaError_t e = sbim::prepare_conv_tma(h->prec, h->kahan, h->variant, h->tile, h->halves);
@@ -1249,9 +1313,27 @@ int sbim_set_conv_tile(sbim_handle h, int orbits_per_cta) {
   const int rc = configure_conv(*h);
   if (rc != SBIM_OK) {
     h->tile = old_t; h->lc = old_lc; h->nchunks = old_nc;
-    h->ahead_lc = old_alc; h->ahead_chunks = old_anc; h->use_ahead = old_ahead;
     return rc;
   }
+  return SBIM_OK;
+}
+
+int sbim_set_time_blocks(sbim_handle h, int enable) {
+  if (!h) return fail(SBIM_ERR_ARG, "NULL handle");
+  h->can_repeat = false;
+  h->blocks_off = !enable;
+  if (enable) {
+    if (h->blocks == 0) h->blocks = -1;
+    return SBIM_OK;
+  }
+  h->blocks = 0;
+  return drop_blocks(h);
+}
+
+int sbim_get_time_blocks(sbim_handle h, int* enabled) {
+  if (!h || !enabled) return fail(SBIM_ERR_ARG, "NULL argument");
+  if (const int rc = ready(h, h->stream)) return rc;
+  *enabled = h->blocks == 1;
   return SBIM_OK;
 }
 
@@ -1264,7 +1346,7 @@ int sbim_set_far_field(sbim_handle h, const double tau_inf[3]) {
 int sbim_reset(sbim_handle h) {
   if (!h) return fail(SBIM_ERR_ARG, "NULL handle");
   CU(cudaMemsetAsync(h->d_step, 0, sizeof(long long), h->stream));
-  if (const int rc = forget_ahead(h)) return rc;
+  if (const int rc = forget_ahead(h, h->stream)) return rc;
   h->n = 0;
   h->can_repeat = false;
   return SBIM_OK;
@@ -1352,7 +1434,7 @@ int sbim_load(sbim_handle h, const void* buf, size_t bytes) {
   CU(cudaMemcpyAsync(h->d_hist, (const char*)buf + sizeof(hd), h->hist_bytes,
                      cudaMemcpyHostToDevice, h->stream));
   CU(cudaMemcpyAsync(h->d_step, &hd.n, sizeof(long long), cudaMemcpyHostToDevice, h->stream));
-  if (const int rc = forget_ahead(h)) return rc;
+  if (const int rc = forget_ahead(h, h->stream)) return rc;
   CU(cudaStreamSynchronize(h->stream));
   h->n = hd.n;
   h->can_repeat = false;

@@ -120,7 +120,12 @@ int configure(sbim_batch_ctx* b, int shape, int lags) {
     (sbim::handle_step_args(b->h[i]).halves ? b->halves : b->whole) = true;
   // time-blocked where every member has room for its block sums
   b->ahead = true;
-  for (sbim_handle x : b->h) b->ahead = b->ahead && sbim::handle_uses_ahead(x);
+  for (sbim_handle x : b->h) {
+    bool blocks = false;
+    const int rc = sbim::handle_uses_ahead(x, &blocks);
+    if (rc != SBIM_OK) return rc;
+    b->ahead = b->ahead && blocks;
+  }
   if (b->ahead) {
     if (b->whole) BCU(sbim::launch_ahead(sbim::StepArgs{}, b->prec, 0, false, nullptr));
     if (b->halves) BCU(sbim::launch_ahead(sbim::StepArgs{}, b->prec, 0, true, nullptr));

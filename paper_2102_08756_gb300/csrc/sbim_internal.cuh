@@ -183,7 +183,7 @@ cudaError_t pair_end(PairStreams& p, cudaStream_t st);     // st follows the sid
 void pair_release(PairStreams& p);
 int handle_epilogue(sbim_handle h, const void* v, void* tau, cudaStream_t st);
 void handle_advance(sbim_handle h);
-bool handle_uses_ahead(sbim_handle h);
+int handle_uses_ahead(sbim_handle h, bool* blocks);   // decides if need be
 void handle_hold(sbim_handle h);   // a batch keeps its arguments: no buffer of it moves away from now on
 int handle_step_by_step(sbim_handle h);   // leave the time-blocked convolution
 int handle_shape(sbim_handle h, int* precision, int* kahan, int* variant, void** stream);

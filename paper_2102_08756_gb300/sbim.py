@@ -58,6 +58,8 @@ def lib():
     L.sbim_stage_times.argtypes = [vp, ctypes.POINTER(d), ctypes.POINTER(ll)]
     L.sbim_set_conv_config.argtypes = [vp, i, i]
     L.sbim_set_window.argtypes = [vp, d]
+    L.sbim_set_time_blocks.argtypes = [vp, i]
+    L.sbim_get_time_blocks.argtypes = [vp, ctypes.POINTER(i)]
     L.sbim_check_device.argtypes = [vp]
     L.sbim_selftest_wait_timeout.argtypes = [vp]
     L.sbim_spectral_response_noalloc.argtypes = [i, i, d, d, d, d, d, d, i, i, vp, vp, vp]
@@ -101,7 +103,7 @@ def lib():
                  "sbim_reset", "sbim_get_step", "sbim_get_info", "sbim_plan", "sbim_set_profiling",
                  "sbim_set_check_finite", "sbim_set_conv_tile", "sbim_batch_set_conv_tile",
                  "sbim_hybrid_batch_set_conv_tile",
-                 "sbim_stage_times", "sbim_set_conv_config", "sbim_check_device", "sbim_set_window",
+                 "sbim_stage_times", "sbim_set_conv_config", "sbim_set_time_blocks", "sbim_get_time_blocks", "sbim_check_device", "sbim_set_window",
                  "sbim_spectral_response_noalloc", "sbim_destroy", "sbim_hybrid_create",
                  "sbim_hybrid_set_fault", "sbim_hybrid_set_state", "sbim_hybrid_get_state",
                  "sbim_hybrid_step", "sbim_hybrid_fault_fields", "sbim_hybrid_info",
@@ -226,6 +228,16 @@ def sbim_stage_times(h):
 
 def sbim_set_conv_config(h, variant, lags_per_cta=0):
     _check(lib().sbim_set_conv_config(h, int(variant), int(lags_per_cta)))
+
+
+def sbim_set_time_blocks(h, enable):
+    _check(lib().sbim_set_time_blocks(h, int(bool(enable))))
+
+
+def sbim_get_time_blocks(h):
+    on = ctypes.c_int()
+    _check(lib().sbim_get_time_blocks(h, ctypes.byref(on)))
+    return bool(on.value)
 
 
 def sbim_set_window(h, window):
@@ -524,6 +536,14 @@ class SBIM:
 
     def set_conv_config(self, variant, lags_per_cta=0):
         sbim_set_conv_config(self.h, variant, lags_per_cta)
+
+    def set_time_blocks(self, enable=True):
+        """Convolve blocked in time where memory allows it, or step by step (see include/sbim.h)."""
+        sbim_set_time_blocks(self.h, enable)
+
+    def time_blocks(self):
+        """Whether the next step takes block sums."""
+        return sbim_get_time_blocks(self.h)
 
     def set_window(self, window):
         """Mode-dependent truncation window in T = |k| c_s t (0: uniform cutoff)."""
