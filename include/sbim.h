@@ -177,7 +177,11 @@ int sbim_get_step(sbim_handle h, long long* n);
  * counter n, the far-field traction and the whole history ring (the spectra of
  * every displacement the truncated convolution of Eq. (SBI) can still reach;
  * Section 2.3).  A run restored from a checkpoint continues bit-for-bit as the
- * original run did from the step it was taken at.
+ * original run did from the step it was taken at, given the same launch settings
+ * (sbim_set_conv_config, sbim_set_conv_tile, sbim_set_window, which a checkpoint does
+ * not hold).  A checkpoint tells whether the convolution took block sums
+ * (sbim_set_time_blocks), and the restored handle goes on in that form; one that has
+ * no room for block sums, or was told to do without, differs by rounding.
  *
  *   sbim_save(h, buf, &bytes)
  *     buf == NULL: writes the size a checkpoint needs to *bytes and returns OK.

@@ -1372,13 +1372,15 @@ namespace {
 // Checkpoint header: the parameters a restored handle must match, then the state.
 struct SaveHeader {
   char magic[8];
-  int version, n1, n3, n_cut, side, prec, n_orb_pad, pad0;
+  int version, n1, n3, n_cut, side, prec, n_orb_pad;
+  int form;   // of the convolution: kFormBlocks, kFormSteps, or 0 (undecided, FP64, variant 0)
   double L1, L3, cs, cp, rho, dt;
   long long n, hist_bytes;
   double tau_inf[3];
 };
 constexpr char kSaveMagic[8] = {'S', 'B', 'I', 'M', 'H', 'S', 'T', '1'};
 constexpr int kSaveVersion = 1;
+constexpr int kFormBlocks = 1, kFormSteps = 2;
 
 SaveHeader make_header(const sbim_ctx& c) {
   SaveHeader hd;
@@ -1388,6 +1390,8 @@ SaveHeader make_header(const sbim_ctx& c) {
   hd.n1 = c.n1; hd.n3 = c.n3; hd.n_cut = c.n_cut; hd.side = c.side; hd.prec = c.prec;
   hd.n_orb_pad = c.n_orb_pad;
   hd.L1 = c.L1; hd.L3 = c.L3; hd.cs = c.cs; hd.cp = c.cp; hd.rho = c.rho; hd.dt = c.dt;
+  if (c.prec != SBIM_FP64 && c.variant >= 1 && c.blocks >= 0)
+    hd.form = c.blocks ? kFormBlocks : kFormSteps;
   hd.n = c.n;
   hd.hist_bytes = (long long)c.hist_bytes;
   for (int i = 0; i < 3; ++i) hd.tau_inf[i] = c.tau_inf[i];
@@ -1438,6 +1442,9 @@ int sbim_load(sbim_handle h, const void* buf, size_t bytes) {
   CU(cudaStreamSynchronize(h->stream));
   h->n = hd.n;
   h->can_repeat = false;
+  // the run goes on in the form it had (block sums only if there is room for them)
+  if (hd.form == kFormSteps) h->blocks = 0;
+  if (hd.form == kFormBlocks && h->blocks == 0 && !h->blocks_off) h->blocks = -1;
   for (int i = 0; i < 3; ++i) h->tau_inf[i] = hd.tau_inf[i];
   return SBIM_OK;
 }

@@ -160,3 +160,35 @@ def test_first_steps_under_capture():
             stream.synchronize()
             err.update(rel_l2(tau.double().cpu().numpy(), r))
     assert err.value < TOL["fp32"], err
+
+
+def test_a_restored_run_goes_on_in_its_form():
+    n, n_cut = 48, 40
+    f = [(1e-3 * torch.randn((3, n, n), device="cuda"), torch.randn((3, n, n), device="cuda")) for _ in range(70)]
+
+    def run(h, a, b):
+        return [h.step(u, v) for u, v in f[a:b]]
+
+    def same(x, y):
+        return all(torch.equal(p, q) for p, q in zip(x, y))
+
+    by_step, by_block = _make(n, n_cut), _make(n, n_cut)
+    by_step.set_time_blocks(False)
+    run(by_step, 0, 37)
+    run(by_block, 0, 37)
+    saved = by_step.save(), by_block.save()
+    after = run(by_step, 37, 70), run(by_block, 37, 70)
+    assert not same(*after)                       # the forms round differently
+    h = _make(n, n_cut)
+    for k in (0, 1, 0, 1):
+        h.load(saved[k])
+        assert same(run(h, 37, 70), after[k]) and h.time_blocks() == bool(k)
+    # told to do without block sums, a handle does, and differs by rounding only
+    h.set_time_blocks(False)
+    h.load(saved[1])
+    got = run(h, 37, 70)
+    assert not h.time_blocks()
+    err = Worst()
+    for p, q in zip(got, after[1]):
+        err.update(rel_l2(p.double().cpu().numpy(), q.double().cpu().numpy()))
+    assert err.value < TOL["fp32"], err
