@@ -300,8 +300,8 @@ int sbim_set_conv_config(sbim_handle h, int variant, int lags_per_cta);
  *     captured from this handle's steps must be captured again.
  *   get tells whether the next step takes block sums (deciding it if no step has yet).
  * A first step under stream capture allocates nothing and goes step by step.  FP64
- * handles, variant 0 and very short hi-only BF16 histories (n_cut < 28) on planes of
- * 16,384 whole records and more always do.  Library utility: the paper has no counterpart.
+ * handles, variant 0 and very short hi-only BF16 histories (n_cut < 36) on large planes
+ * (16,384 records and more) always do.  Library utility: the paper has no counterpart.
  */
 int sbim_set_time_blocks(sbim_handle h, int enable);
 int sbim_get_time_blocks(sbim_handle h, int* enabled);

@@ -495,16 +495,23 @@ int have_room(const sbim_ctx& c, size_t bytes, bool* room) {
   return SBIM_OK;
 }
 
+// On large planes a very short hi-only BF16 history is read faster than the lags inside
+// a block are added.  us a step, step by step / blocked: 1024^2, 16 lags 124 / 135, 32
+// lags 144 / 148, 40 lags 158 / 156; 720^2 24 lags 95 / 100, 32 lags 101 / 97; half
+// records, uncompensated: 1024 x 768, 4 lags 90 / 98, 16 lags 111 / 120, 32 lags 131 / 126;
+// 1024 x 500, 16 lags 84 / 92, 24 lags 97 / 96; compensated, 16 lags 98 / 92.  Hi/lo and
+// FP32: 1024^2, 16 lags 153 / 152 and 149 / 130.
+bool reads_faster(const sbim_ctx& c) {
+  if (c.prec != SBIM_BF16) return false;
+  if (!c.halves) return c.n_cut < (c.n_orb_pad >= 98304 ? 36 : c.n_orb_pad >= 16384 ? 28 : 0);
+  return !c.kahan && c.n_orb_pad >= 49152 && c.n_cut >= 4 && c.n_cut < 24;
+}
+
 // Room for the sums of the current chunking, and everything that goes with them if this
 // is the first time; *ok is false where there is none.
 int start_blocks(sbim_ctx* c, cudaStream_t st, bool* ok) {
   *ok = false;
-  // On large planes of whole records a very short BF16 history is read faster than the lags
-  // inside a block are added (1024^2, hi-only, us a step: 16 lags 129 step by step against
-  // 143, 24 lags 141 / 150, 39 lags 162 / 151; hi/lo, 16 lags: 163 / 152; half records,
-  // 1024 x 500, 20 lags: 96 / 90).
-  const int least = c->prec == SBIM_BF16 && !c->halves && c->n_orb_pad >= 16384 ? 28 : 0;
-  if (c->prec == SBIM_FP64 || c->variant < 1 || c->blocks_off || c->n_cut < least) return SBIM_OK;
+  if (c->prec == SBIM_FP64 || c->variant < 1 || c->blocks_off || reads_faster(*c)) return SBIM_OK;
   const size_t sums = ahead_need(*c);
   if (!c->d_extra) {
     const size_t w32 = sbim::ahead_weight_bytes(c->n_orb_pad, c->n_cut, c->halves);

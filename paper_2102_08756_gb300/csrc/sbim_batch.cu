@@ -28,7 +28,7 @@ struct sbim_batch_ctx {
   int* d_item_prefix = nullptr;
   int* d_tile_prefix = nullptr;
   int* d_counter = nullptr;
-  int total_items = 0, total_tiles = 0, ctas = 0;
+  int total_items = 0, total_tiles = 0, ctas = 0, chunks = 1;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   // side streams for the members' small stages (FFTs, epilogues): they run
@@ -147,6 +147,8 @@ int configure(sbim_batch_ctx* b, int shape, int lags) {
     items[i + 1] = items[i] + (b->ahead ? sbim::ahead_ctas(args[i].n_orb_pad) * args[i].ahead_chunks
                                         : args[i].n_orb_pad / b->tile * args[i].nchunks);
   }
+  b->chunks = 1;
+  for (const sbim::StepArgs& x : args) b->chunks = x.nchunks > b->chunks ? x.nchunks : b->chunks;
   b->total_items = items[b->nb];
   b->total_tiles = tiles[b->nb];
   if (!b->d_args) BCU(cudaMalloc(&b->d_args, b->nb * sizeof(sbim::StepArgs)));
@@ -208,6 +210,7 @@ int enqueue(sbim_batch_ctx* b, const void* const* u, const void* const* v, void*
   bl.counter = b->d_counter;
   bl.ctas = b->ctas;
   bl.items = b->per_item || b->ahead ? b->total_items : 0;
+  bl.chunks = b->chunks;
   bl.whole = b->whole;
   int rc = fork(b);
   // the block sums need only the stored histories: they run beside the transforms

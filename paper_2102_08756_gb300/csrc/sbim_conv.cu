@@ -124,13 +124,46 @@ conv_kernel(const StepArgs a) {
           KAHAN ? acc[g][k] - cmp[g][k] : acc[g][k];
 }
 
+// A member's output spectrum from its five sums v, current spectra d_xi and d_2 and
+// direction e, scaled by wsc.
+template <class R, class C>
+__device__ __forceinline__ void modal_operator(const R (&v)[kFields], const C dxi, const C d2, const C e,
+                                               R muq, R wsc, R sd, R inst, R (&F)[6]) {
+  // F_xi = -side mu q C11 + i mu q [(2 - eta) D_2 + C12a]
+  const R bxr = inst * d2.x + v[6], bxi = inst * d2.y + v[7];
+  C fxi, fp, f2;
+  fxi.x = muq * (-sd * v[0] - bxi);
+  fxi.y = muq * (-sd * v[1] + bxr);
+  // F_perp = -side mu q C33
+  fp.x = -sd * muq * v[2];
+  fp.y = -sd * muq * v[3];
+  // F_2 = -i mu q [(2 - eta) D_xi + C12b] - side mu q C22
+  const R b2r = inst * dxi.x + v[8], b2i = inst * dxi.y + v[9];
+  f2.x = muq * (b2i - sd * v[4]);
+  f2.y = muq * (-b2r - sd * v[5]);
+  F[0] = wsc * (e.x * fxi.x - e.y * fp.x);
+  F[1] = wsc * (e.x * fxi.y - e.y * fp.y);
+  F[2] = f2.x * wsc;
+  F[3] = f2.y * wsc;
+  F[4] = wsc * (e.y * fxi.x + e.x * fp.x);
+  F[5] = wsc * (e.y * fxi.y + e.x * fp.y);
+}
+// Sums of two members' spectra are rounded by themselves (not fused with the scaling), so
+// that both forms of the assembly give the same bits.
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+template <class C> __device__ __forceinline__ C add_cplx(C a, C b) {
+  return make_cplx(add_rn(a.x, b.x), add_rn(a.y, b.y));
+}
+
 // The chunk reduction and the modal operator for 32 records, one thread per member
 // (warp g holds member g of each record, so the partial sums are read coalesced).  The
 // chunk loop keeps four chunks' 10 sums in flight; each sum's order over the chunks,
 // and its compensation, are those of a loop over single chunks.  A thread per record
-// with all 40 sums left a 64^2 plane 5 blocks of 4 warps: 105 us of its 163 us step in
-// FP64 (16 chunks); with one per member the step takes 106 us.
+// with all 40 sums leaves a 64^2 plane 5 blocks of 4 warps: 105 us of its 163 us step in
+// FP64 (16 chunks); with one per member the step takes 106 us (by_record chooses).
 constexpr int kAsmRec = 32, kAsmThreads = kAsmRec * kMembers;
+static_assert(kAsmThreads == kOrbitTile, "both forms of the assembly run the same blocks");
 
 template <class S, int KAHAN>
 __device__ __forceinline__ void assemble_records(const StepArgs& a, int o0) {
@@ -182,23 +215,9 @@ __device__ __forceinline__ void assemble_records(const StepArgs& a, int o0) {
   }
 
   const int b = a.bin[o * kMembers + g];
-  const C dxi = D[0], d2 = D[1];
-  // F_xi = -side mu q C11 + i mu q [(2 - eta) D_2 + C12a]
-  const R bxr = inst * d2.x + v[6], bxi = inst * d2.y + v[7];
-  C fxi, fp, f2;
-  fxi.x = muq * (-sd * v[0] - bxi);
-  fxi.y = muq * (-sd * v[1] + bxr);
-  // F_perp = -side mu q C33
-  fp.x = -sd * muq * v[2];
-  fp.y = -sd * muq * v[3];
-  // F_2 = -i mu q [(2 - eta) D_xi + C12b] - side mu q C22
-  const R b2r = inst * dxi.x + v[8], b2i = inst * dxi.y + v[9];
-  f2.x = muq * (b2i - sd * v[4]);
-  f2.y = muq * (-b2r - sd * v[5]);
-  const C e = reinterpret_cast<const C*>(a.dir)[o * kMembers + g];
-  const R wsc = (R)a.wout[o * kMembers + g] * (R)a.inv_n;
-  const R F[6] = {wsc * (e.x * fxi.x - e.y * fp.x), wsc * (e.x * fxi.y - e.y * fp.y), f2.x * wsc,
-                  f2.y * wsc, wsc * (e.y * fxi.x + e.x * fp.x), wsc * (e.y * fxi.y + e.x * fp.y)};
+  R F[6];
+  modal_operator(v, D[0], D[1], reinterpret_cast<const C*>(a.dir)[o * kMembers + g], muq,
+                 (R)a.wout[o * kMembers + g] * (R)a.inv_n, sd, inst, F);
   shB[g][r] = b;
 #pragma unroll
   for (int k = 0; k < 6; ++k) shF[g][k][r] = F[k];
@@ -210,28 +229,137 @@ __device__ __forceinline__ void assemble_records(const StepArgs& a, int o0) {
   for (int k = 0; k < 6; ++k) G[k] = F[k];
   for (int h = g + 1; h < kMembers && shB[h][r] == b; ++h)
 #pragma unroll
-    for (int k = 0; k < 6; ++k) G[k] += shF[h][k][r];
+    for (int k = 0; k < 6; ++k) G[k] = add_rn(G[k], shF[h][k][r]);
   C* fh = reinterpret_cast<C*>(a.fhat);
   fh[b] = make_cplx(G[0], G[1]);
   fh[a.nbins + b] = make_cplx(G[2], G[3]);
   fh[2 * (long long)a.nbins + b] = make_cplx(G[4], G[5]);
 }
 
+// The same with one thread per record.
 template <class S, int KAHAN>
+__device__ __forceinline__ void assemble_orbit(const StepArgs& a, int o) {
+  using R = typename S::real;
+  using C = typename S::cplx;
+  const long long n = *a.step;
+  const int n_valid = (n + 1 < (long long)a.n_cut) ? (int)(n + 1) : a.n_cut;
+  const int m_end = a.tile_lmax ? min(n_valid, a.tile_lmax[o / kOrbitTile]) : n_valid;
+  const int nch = (m_end + a.lc - 1) / a.lc;
+  const long long orb = a.n_orb_pad;
+  const R muq0 = reinterpret_cast<const R*>(a.muq)[2 * o];
+  const R muq1 = reinterpret_cast<const R*>(a.muq)[2 * o + 1];
+  const R sd = (R)a.side;
+  const R inst = (R)(2.0 - a.eta);
+  const R* part = reinterpret_cast<const R*>(a.part);
+  C* fh = reinterpret_cast<C*>(a.fhat);
+
+  C D[3][4];
+  rotate_current(a, o, D);
+
+  // Chunk reduction of the 4 x kFields sums: the chunk loop is outermost so that
+  // each iteration issues 40 independent loads (each sum's own order over the
+  // chunks, and its compensation, are those of a per-sum loop).
+  R sum[4][kFields], cmp[4][kFields];
+#pragma unroll
+  for (int g = 0; g < 4; ++g)
+#pragma unroll
+    for (int k = 0; k < kFields; ++k) { sum[g][k] = (R)0; cmp[g][k] = (R)0; }
+  auto load_chunk = [&](int ch, R (&x)[4][kFields]) {
+#pragma unroll
+    for (int g = 0; g < 4; ++g)
+#pragma unroll
+      for (int k = 0; k < kFields; ++k)
+        x[g][k] = part[((long long)ch * (4 * kFields) + g * kFields + k) * orb + o];
+  };
+  if constexpr (KAHAN) {
+    for (int ch = 0; ch < nch; ++ch) {
+      R x[4][kFields];
+      load_chunk(ch, x);
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+#pragma unroll
+        for (int k = 0; k < kFields; ++k) {
+          const R y = x[g][k] - cmp[g][k];
+          const R t = sum[g][k] + y;
+          cmp[g][k] = (t - sum[g][k]) - y;
+          sum[g][k] = t;
+        }
+    }
+  } else if constexpr (sizeof(R) == 8) {
+    // FP64 sums (their step is bound by the FP64 pipe): one chunk at a time
+    for (int ch = 0; ch < nch; ++ch) {
+      R x[4][kFields];
+      load_chunk(ch, x);
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+#pragma unroll
+        for (int k = 0; k < kFields; ++k) sum[g][k] += x[g][k];
+    }
+  } else if (nch > 0) {
+    // Plain float sums: the next chunk's 40 loads are issued before this chunk's
+    // adds (left to the compiler, the uncompensated loop kept few loads in flight
+    // and ran at a third of the compensated one's rate on GB300).
+    R x[4][kFields], xn[4][kFields];
+    load_chunk(0, x);
+    for (int ch = 0; ch < nch; ++ch) {
+      const bool more = ch + 1 < nch;
+      if (more) load_chunk(ch + 1, xn);
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+#pragma unroll
+        for (int k = 0; k < kFields; ++k) sum[g][k] += x[g][k];
+      if (more)
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+#pragma unroll
+          for (int k = 0; k < kFields; ++k) x[g][k] = xn[g][k];
+    }
+  }
+
+  int pend = -1;
+  C P1, P2, P3;
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    const int b = a.bin[o * 4 + g];
+    if (b < 0) continue;
+    const R muq = g < 2 ? muq0 : muq1;
+    R F[6];
+    modal_operator(sum[g], D[0][g], D[1][g], reinterpret_cast<const C*>(a.dir)[o * 4 + g], muq,
+                   (R)a.wout[o * 4 + g] * (R)a.inv_n, sd, inst, F);
+    const C f1 = make_cplx(F[0], F[1]), f2 = make_cplx(F[2], F[3]), f3 = make_cplx(F[4], F[5]);
+    if (b == pend) {
+      P1 = add_cplx(P1, f1); P2 = add_cplx(P2, f2); P3 = add_cplx(P3, f3);
+    } else {
+      if (pend >= 0) {
+        fh[pend] = P1; fh[a.nbins + pend] = P2; fh[2 * (long long)a.nbins + pend] = P3;
+      }
+      pend = b; P1 = f1; P2 = f2; P3 = f3;
+    }
+  }
+  if (pend >= 0) {
+    fh[pend] = P1; fh[a.nbins + pend] = P2; fh[2 * (long long)a.nbins + pend] = P3;
+  }
+}
+
+// RECORDS: one thread per record, else one per member.
+template <class S, int KAHAN, bool RECORDS>
 __global__ void __launch_bounds__(kAsmThreads) assemble_kernel(const StepArgs a) {
-  assemble_records<S, KAHAN>(a, blockIdx.x * kAsmRec);
+  if constexpr (RECORDS) assemble_orbit<S, KAHAN>(a, blockIdx.x * kOrbitTile + threadIdx.x);
+  else assemble_records<S, KAHAN>(a, blockIdx.x * kAsmRec);
 }
 
 // The same over the orbit tiles of every member of a batch.
-template <class S, int KAHAN>
+template <class S, int KAHAN, bool RECORDS>
 __global__ void __launch_bounds__(kAsmThreads)
 assemble_batch_kernel(const StepArgs* __restrict__ args, const int* __restrict__ tile_prefix, int nb) {
-  constexpr int SUB = kOrbitTile / kAsmRec;
+  constexpr int SUB = RECORDS ? 1 : kOrbitTile / kAsmRec;
   const int t = blockIdx.x / SUB;
   int s = 0;
   while (s + 1 < nb && tile_prefix[s + 1] <= t) ++s;
   const StepArgs a = args[s];
-  assemble_records<S, KAHAN>(a, (t - tile_prefix[s]) * kOrbitTile + (blockIdx.x % SUB) * kAsmRec);
+  const int o0 = (t - tile_prefix[s]) * kOrbitTile;
+  if constexpr (RECORDS) assemble_orbit<S, KAHAN>(a, o0 + threadIdx.x);
+  else assemble_records<S, KAHAN>(a, o0 + (blockIdx.x % SUB) * kAsmRec);
 }
 
 template <class R>
@@ -363,9 +491,23 @@ cudaError_t conv_dispatch(const StepArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// A thread per record has four members' loads in flight and needs a quarter of the
+// threads, so it is the faster form once there are records enough to fill the chip, the
+// more so the fewer chunks each of its threads adds up; one per member is where there
+// are not.  Measured, us of the assembly, record / member form: FP32 256^2 1 chunk 8.1 /
+// 8.1, 4 chunks 10.2 / 8.3; 512^2 1 chunk 10.2 / 12.4, 4 13.3 / 16.0, 16 29 / 29; 720^2
+// 16 chunks 52 / 47; 1024^2 1 chunk 24 / 35, 8 53 / 57.  FP64 384^2 1 chunk 16.4 / 16.5;
+// 512^2 1 chunk 22 / 27, 4 41 / 39; 1024^2 1 chunk 61 / 88, 4 117 / 120, 8 135 / 126.
+bool by_record(int precision, long long records, int chunks) {
+  return records >= (precision == SBIM_FP64 ? 30000ll : 6000ll) * chunks;
+}
+
 template <class S, int KAHAN>
 cudaError_t assemble_dispatch(const StepArgs& a, cudaStream_t st) {
-  assemble_kernel<S, KAHAN><<<a.n_orb_pad / kAsmRec, kAsmThreads, 0, st>>>(a);
+  if (by_record(sizeof(typename S::real) == 8 ? SBIM_FP64 : SBIM_FP32, a.n_orb_pad, a.nchunks))
+    assemble_kernel<S, KAHAN, true><<<a.n_orb_pad / kOrbitTile, kAsmThreads, 0, st>>>(a);
+  else
+    assemble_kernel<S, KAHAN, false><<<a.n_orb_pad / kAsmRec, kAsmThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -403,8 +545,11 @@ cudaError_t launch_assemble(const StepArgs& a, int precision, int kahan, cudaStr
 
 template <class S, int KAHAN>
 cudaError_t assemble_batch_dispatch(const BatchLaunch& b, int tiles, cudaStream_t st) {
-  assemble_batch_kernel<S, KAHAN><<<tiles * (kOrbitTile / kAsmRec), kAsmThreads, 0, st>>>(
-      b.args, b.tile_prefix, b.nb);
+  if (by_record(SBIM_FP32, (long long)tiles * kOrbitTile, b.chunks))
+    assemble_batch_kernel<S, KAHAN, true><<<tiles, kAsmThreads, 0, st>>>(b.args, b.tile_prefix, b.nb);
+  else
+    assemble_batch_kernel<S, KAHAN, false><<<tiles * (kOrbitTile / kAsmRec), kAsmThreads, 0, st>>>(
+        b.args, b.tile_prefix, b.nb);
   return cudaGetLastError();
 }
 

@@ -86,6 +86,7 @@ struct BatchLaunch {
   int* counter;             // work counter, zero before each launch
   int ctas;                 // persistent CTAs
   int items;                // > 0: one CTA per item (this many), no persistent CTAs
+  int chunks;               // most lag chunks of a member (step by step)
   bool whole;               // some member has whole records (others may have half records)
 };
 

@@ -113,3 +113,52 @@ def test_batches(precision, kahan, members, shape, lags, tile):
             B.sbim_check_device(B.sbim_batch_member(b, i))
         B.sbim_batch_destroy(b)
     assert err.value < TOL[precision], err
+
+
+# the assembly by record (few chunks for the records) and by member (the same plane in more chunks),
+# whole and half records; FP64 against itself
+@pytest.mark.parametrize("precision,grid", [("fp32", (256, 256)), ("bf16x2", (256, 256)), ("bf16", (256, 256)),
+                                            ("fp32", (384, 160)), ("fp64", (512, 512)), ("fp64", (1024, 250))])
+@pytest.mark.parametrize("kahan", [0, 1])
+def test_assembly_by_record_and_by_member(precision, grid, kahan):
+    n1, n3 = grid
+    n_cut = 14
+    ref = _make(n1, n3, n_cut, "fp64", 0)
+    ref.set_conv_config(1, 4)
+    hs = []
+    for lags in (0, 4):
+        h = _make(n1, n3, n_cut, precision, kahan)
+        h.set_time_blocks(False)
+        h.set_conv_config(2, lags)
+        hs.append(h)
+    tol = TOL.get(precision, 1e-12)
+    err = Worst()
+    for u, v in _fields(n1, n3, 19, seed=5):
+        r = ref.step(u.double(), v.double()).cpu().numpy()
+        x = (u.double(), v.double()) if precision == "fp64" else (u, v)
+        for h in hs:
+            err.update(rel_l2(h.step(*x).double().cpu().numpy(), r))
+    assert err.value < tol, err
+
+
+def test_batched_assembly_by_record():
+    from paper_2102_08756_gb300 import sbim as B
+    n, n_cut = 256, 12
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        b = B.sbim_batch_create([n, 32], [n, 32], [100.0 * n, 3200.0], [100.0 * n, 3200.0], [CS] * 2, [CP] * 2,
+                                [RHO] * 2, [DT] * 2, [n_cut, 7], [1, -1], 1, 1, stream.cuda_stream)
+        B.sbim_set_time_blocks(B.sbim_batch_member(b, 0), False)
+        B.sbim_batch_set_conv_config(b, 5, 1024)
+        alone = [_make(n, n, n_cut, "fp32", 1, stream=stream), _make(32, 32, 7, "fp32", 1, side=-1, stream=stream)]
+        for h in alone:
+            h.set_time_blocks(False)
+            h.set_conv_config(2, 1024)
+        f = [_fields(n, n, 20, seed=1), _fields(32, 32, 20, seed=2)]
+        for m in range(20):
+            tau = [torch.empty_like(x[m][0]) for x in f]
+            B.sbim_batch_step(b, [x[m][0].data_ptr() for x in f], [x[m][1].data_ptr() for x in f],
+                              [t.data_ptr() for t in tau])
+            for i in range(2):
+                assert torch.equal(tau[i], alone[i].step(*f[i][m])), (m, i)
+        B.sbim_batch_destroy(b)
