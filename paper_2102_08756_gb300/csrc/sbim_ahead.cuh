@@ -376,6 +376,7 @@ __device__ __forceinline__ void ahead_tiles(const StepArgs& a, int i, int q, int
           a.stamp[((long long)chunk * tiles + Tt) * kSub + q] != block_mark(a, base);
   }
   unsigned todo = __ballot_sync(0xffffffffu, due);
+  if (gridDim.z > 1) todo &= 1u << blockIdx.z;   // spread: one CTA per tile of the group
   __syncthreads();   // barriers ready; every warp has read the stamps
   unsigned g = 0;    // stages of the items before this one
   for (; todo; todo &= todo - 1) {
@@ -624,10 +625,10 @@ template <class S, bool HALVES>
 cudaError_t launch_sums(const StepArgs& a, cudaStream_t st, const BatchLaunch* batch) {
   constexpr int bytes = smem_bytes<S, HALVES>();
   if (batch) {
-    ahead_batch_kernel<S, HALVES><<<batch->items, kThreads, bytes, st>>>(batch->args, batch->item_prefix,
-                                                                        batch->nb);
+    ahead_batch_kernel<S, HALVES><<<dim3(batch->items, 1, a.spread ? kAhead : 1), kThreads, bytes, st>>>(
+        batch->args, batch->item_prefix, batch->nb);
   } else {
-    const dim3 grid(ahead_ctas(a.n_orb_pad), a.ahead_chunks);
+    const dim3 grid(ahead_ctas(a.n_orb_pad), a.ahead_chunks, a.spread ? kAhead : 1);
     ahead_kernel<S, HALVES><<<grid, kThreads, bytes, st>>>(a);
   }
   return cudaGetLastError();

@@ -133,6 +133,7 @@ struct sbim_ctx {
   float* d_ahead = nullptr;   // the sums: in d_extra, or d_ahead_own once a finer chunking outgrew that
   float* d_ahead_own = nullptr;
   size_t ahead_bytes = 0;
+  bool cold = false;          // more than one tile of a group may have its sums to form
   size_t need = 0;            // device memory of a handle without block sums
   int config_id = 0;          // counts changes of chunking and window (part of the stamps)
   double tab_h = 0;
@@ -462,6 +463,22 @@ size_t ahead_need(const sbim_ctx& c) {
 // Marks every block sum as not formed.
 int forget_ahead(sbim_ctx* c, cudaStream_t st) {
   if (c->d_stamp) CU(cudaMemsetAsync(c->d_stamp, 0xff, c->stamp_bytes, st));
+  c->cold = true;
+  return SBIM_OK;
+}
+
+// The block sums that are due, on `on`.  The first step after sums were marked invalid
+// has up to 16 tiles per group to form, which one CTA would take in turn: that launch has
+// a CTA for each, most of which would find nothing to do in a running loop.  Step in turn /
+// spread / a later step, us, FP32: 128^2 x 48 164 / 50 / 36; 256^2 x 1024 486 / 391 / 66;
+// 512^2 x 1024 1366 / 1266 / 138; 1024^2 x 1024 5174 / 4795 / 441.  Captured graphs keep
+// the running loop's launch.
+int launch_sums(sbim_ctx* c, sbim::StepArgs a, cudaStream_t on) {
+  if (c->cold && !sbim::capturing(on)) {
+    a.spread = 1;
+    c->cold = false;
+  }
+  CU(sbim::launch_ahead(a, c->prec, 1, c->halves, on));
   return SBIM_OK;
 }
 
@@ -564,12 +581,7 @@ int start_blocks(sbim_ctx* c, cudaStream_t st, bool* ok) {
 // handle that is first stepped there goes step by step and stays undecided.
 int ready(sbim_ctx* c, cudaStream_t st) {
   if (c->blocks >= 0) return SBIM_OK;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
-    cudaGetLastError();
-    return SBIM_OK;
-  }
-  if (cap != cudaStreamCaptureStatusNone) return SBIM_OK;
+  if (sbim::capturing(st)) return SBIM_OK;
   // (allocations would break a capture that another thread has under way)
   cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
   CU(cudaThreadExchangeStreamCaptureMode(&mode));
@@ -601,7 +613,10 @@ int configure_conv(sbim_ctx& c) {
   int dev = 0, sms = 148;
   CU(cudaGetDevice(&dev));
   CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int old_lc = c.ahead_lc;
   choose_ahead(c, sms);
+  // (block sums of the same chunking stay as they are)
+  if (c.blocks == 1 && c.variant >= 1 && c.ahead_lc == old_lc) return SBIM_OK;
   ++c.config_id;
   c.blocks = -1;
   return SBIM_OK;
@@ -791,6 +806,7 @@ sbim::StepArgs step_args(const sbim_ctx* c) {
   a.stamp = c->d_stamp;
   a.ahead_lc = c->ahead_lc;
   a.ahead_chunks = c->ahead_chunks;
+  a.spread = 0;
   a.config_id = c->config_id & 0xffff;
   a.uhat = c->d_uhat;
   a.fhat = c->d_fhat;
@@ -811,6 +827,13 @@ sbim::StepArgs step_args(const sbim_ctx* c) {
 
 namespace sbim {
 void set_last_error(const char* msg) { g_err = msg; }
+
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  cudaGetLastError();   // the legacy stream beside another stream's capture
+  return true;
+}
 
 StepArgs handle_step_args(sbim_handle h) { return step_args(h); }
 
@@ -861,6 +884,12 @@ int handle_uses_ahead(sbim_handle c, bool* blocks) {
 }
 
 void handle_hold(sbim_handle c) { c->held = true; }
+
+bool handle_take_cold(sbim_handle c) {
+  const bool cold = c->cold;
+  c->cold = false;
+  return cold;
+}
 
 int handle_step_by_step(sbim_handle c) {
   c->blocks = 0;
@@ -966,7 +995,7 @@ int check_inputs(sbim_ctx* c, const void* a, const void* b, cudaStream_t st) {
 // the sums in it against 37.5).
 int fork_sums(sbim_ctx* c, const sbim::StepArgs& a, cudaStream_t st) {
   CU(sbim::pair_begin(c->sums, st));
-  CU(sbim::launch_ahead(a, c->prec, 1, c->halves, c->sums.side));
+  if (const int rc = launch_sums(c, a, c->sums.side)) return rc;
   CU(cudaEventRecord(c->sums.join, c->sums.side));
   return SBIM_OK;
 }
@@ -1006,7 +1035,7 @@ int run_step(sbim_ctx* c, const void* in, const void* aux, void* out, bool adjoi
   if (beside)
     CU(cudaStreamWaitEvent(st, c->sums.join, 0));
   else if (sums)
-    CU(sbim::launch_ahead(a, c->prec, 1, c->halves, st));
+    if (const int rc = launch_sums(c, a, st)) return rc;
   if (blocks) {
   } else if (repeat)
     CU(sbim::launch_repeat_lag0(a, c->prec, st));
@@ -1190,9 +1219,9 @@ int sbim_step_host(sbim_handle h, const void* u, const void* v, void* tau) {
     CU(cudaEventRecord(c->io_join, c->io_stream));
     sbim::StepArgs a = step_args(c);
     a.uhat = zero_hat;
-    if (blocks)
-      CU(sbim::launch_ahead(a, c->prec, 1, c->halves, st));
-    else if (c->variant >= 1)
+    if (blocks) {
+      if ((rc = launch_sums(c, a, st))) return rc;
+    } else if (c->variant >= 1)
       CU(sbim::launch_conv_tma(a, c->prec, c->kahan, c->variant, st, nullptr, c->tile, c->halves));
     else
       CU(sbim::launch_conv(a, c->prec, c->kahan, st));
@@ -1222,6 +1251,7 @@ int sbim_set_window(sbim_handle h, double window) {
   if (!h) return fail(SBIM_ERR_ARG, "NULL handle");
   if (!(window >= 0)) return fail(SBIM_ERR_ARG, "window must be >= 0");
   h->can_repeat = false;
+  if (window == h->window) return SBIM_OK;
   ++h->config_id;
   if (const int rc = forget_ahead(h, h->stream)) return rc;
   if (window == 0) {
@@ -1364,6 +1394,7 @@ int sbim_rewind(sbim_handle h) {
   if (h->n == 0) return fail(SBIM_ERR_STATE, "no step to rewind");
   CU(sbim::launch_rewind(h->d_step, h->stream, h->d_stamp,
                          (long long)(h->stamp_bytes / sizeof(long long))));
+  h->cold = true;
   --h->n;
   h->can_repeat = false;
   return SBIM_OK;

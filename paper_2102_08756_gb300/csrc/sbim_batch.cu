@@ -201,7 +201,10 @@ int setup(sbim_batch_ctx* b) {
 
 // Enqueue one step of every member (pointer arrays are host arrays of device pointers).
 int enqueue(sbim_batch_ctx* b, const void* const* u, const void* const* v, void* const* tau) {
-  const sbim::StepArgs a0 = sbim::handle_step_args(b->h[0]);
+  sbim::StepArgs a0 = sbim::handle_step_args(b->h[0]);
+  a0.spread = 0;
+  if (b->ahead && !sbim::capturing(b->stream))
+    for (sbim_handle x : b->h) a0.spread |= sbim::handle_take_cold(x);
   sbim::BatchLaunch bl;
   bl.args = b->d_args;
   bl.item_prefix = b->d_item_prefix;

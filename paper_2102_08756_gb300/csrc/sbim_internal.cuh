@@ -70,6 +70,7 @@ struct StepArgs {
   int nchunks;
   int ahead_lc;                    // lags per chunk of the time-blocked sums, a multiple of 16
   int ahead_chunks;
+  int spread;                      // host: a CTA of its own for each tile whose block sums may be due
   int config_id;                   // 16 bits: chunking and window of these arguments
   int side;
   double eta;
@@ -157,6 +158,7 @@ cudaError_t launch_table_build(double* out64, float* out32, long long n, double 
                                double eta, const double* gl_x, const double* gl_w,
                                cudaStream_t s);
 
+bool capturing(cudaStream_t st);   // or cannot be told apart from it
 // Set the calling thread's message returned by sbim_last_error().
 void set_last_error(const char* msg);
 
@@ -185,6 +187,7 @@ void pair_release(PairStreams& p);
 int handle_epilogue(sbim_handle h, const void* v, void* tau, cudaStream_t st);
 void handle_advance(sbim_handle h);
 int handle_uses_ahead(sbim_handle h, bool* blocks);   // decides if need be
+bool handle_take_cold(sbim_handle h);   // whether block sums were marked invalid since the last call
 void handle_hold(sbim_handle h);   // a batch keeps its arguments: no buffer of it moves away from now on
 int handle_step_by_step(sbim_handle h);   // leave the time-blocked convolution
 int handle_shape(sbim_handle h, int* precision, int* kahan, int* variant, void** stream);

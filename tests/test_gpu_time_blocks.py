@@ -151,6 +151,42 @@ def test_batches_of_mixed_layouts(members):
         B.sbim_batch_destroy(b)
 
 
+def test_batch_members_restored_in_the_middle_of_a_run():
+    """Every tile's sums are formed again in one step: both record layouts, 18 tiles in one member,
+    members restored from the checkpoints of handles that went on alone; then a new window."""
+    from paper_2102_08756_gb300.sbim import SBIM
+    members, n_cut, dt = [(176, 96), (64, 6)], 45, 0.3 * 100.0 / CP
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        B, b = _batch(members, n_cut, dt, stream)
+        alone = [SBIM(n1, n3, n1 * 100.0, n3 * 100.0, CS, CP, RHO, dt, n_cut, 1, "fp32", True,
+                      stream=stream) for n1, n3 in members]
+        f = [_fields(n1, n3, dt, 75, seed=k) for k, (n1, n3) in enumerate(members)]
+        for k, h in enumerate(alone):
+            h.set_conv_config(2, 1024)
+            for m in range(53):
+                h.step(*f[k][m])
+            B.sbim_load(B.sbim_batch_member(b, k), h.save())
+        for m in range(53, 75):
+            tau = _batch_step(B, b, [x[m] for x in f])
+            for k, h in enumerate(alone):
+                assert torch.equal(tau[k], h.step(*f[k][m])), (m, k)
+        B.sbim_batch_destroy(b)
+
+
+def test_settings_that_change_nothing_keep_the_sums():
+    """The same window, another pipeline shape or tile: no sums are formed again, the bits are those of
+    a handle left alone."""
+    n1, n3, n_cut = 48, 32, 40
+    g, same, dt = _pair(n1, n3, n_cut, "fp32")[0], _pair(n1, n3, n_cut, "fp32")[0], 0.3 * 100.0 / CP
+    for m, (u, v) in enumerate(_fields(n1, n3, dt, 60, seed=3)):
+        if m % 7 == 3:
+            g.set_window(0.0)
+            g.set_conv_config(1 + m % 3, 0)
+            g.set_conv_tile(64 if m % 2 else 128)
+        assert torch.equal(g.step(u, v), same.step(u, v)), m
+
+
 def test_member_with_its_own_chunking_between_batch_steps():
     """A batch keeps its copy of a member's chunking; the member, given a coarser one and
     stepped by itself, and the batch then alternate on the same sums buffer."""
