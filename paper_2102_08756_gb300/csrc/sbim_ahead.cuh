@@ -11,19 +11,21 @@
 // (near_kernel).  The history is read once per 16 steps and the work per step is
 // the same multiply-adds, now bound by the FP32 pipe (39-40 T multiply-adds/s
 // measured on GB300: 0.54 ms for 1024^2 x 4096 against 7.1 ms for the bytes).  The kernel
-// takes 1.11 ms there, 155 ns per lag of a CTA against 77 on the pipe alone: 17 of a
-// warp's 41 instructions per lag are the two-lane multiply-adds (ncu, 512^2 x 1024), and
-// the pipe is busy 59 % of the time.  A warp set aside for the requests (spills: 21 warps
-// leave 80 registers), the requests in turns behind an mbarrier (+3 %), a skew of at most
-// one (+15 %) or two stages (+1 %) between the warps, and weights loaded into both halves
-// of a register pair (same) were measured and not kept.
+// takes 1.17 ms there, ~160 ns per lag of a CTA against 77 on the pipe alone: 16 of a
+// warp's 35 instructions per lag are the two-lane multiply-adds and 4 the folds (ncu,
+// 512^2 x 1024), and the pipe is busy 61 % of the time.  A warp set aside for the
+// requests (spills: 21 warps leave 80 registers), the requests in turns behind an
+// mbarrier (+3 %), a skew of at most one (+15 %) or two stages (+1 %) between the warps,
+// weights loaded into both halves of a register pair (same) and a stage released before
+// its fold (+3 to 5 %) were measured and not kept.
 //
 // Blocks are aligned and staggered: tile T (128 records) starts its blocks at the
-// steps with (n + T) mod 16 = 0, so every step renews 1/16 of the tiles and costs
-// the same.  A tile's block is a function of n and T only, and every sum has a
-// fixed order, so a step's result does not depend on when its sums were formed: a
-// restored checkpoint, a rewound or repeated step and a replayed graph give the
-// same bits as the run they continue.  Each (chunk, tile, 32 records) carries a stamp
+// steps with (n + T) mod 16 = 0, so every step of a plane of 16 and more tiles renews
+// about 1/16 of them and costs the same (smaller planes have steps that renew none).
+// A tile's block is a function of n and T only, and every sum has a fixed order, so a
+// step's result does not depend on when its sums were formed: a restored checkpoint, a
+// rewound or repeated step and a replayed graph give the same bits as the run they
+// continue.  Each (chunk, tile, 32 records) carries a stamp
 // of the block its sums belong to and of the arguments' chunking and window; sums
 // whose stamp is not the current one are formed again, all on the device, so that a
 // captured graph renews them as a direct step does.  sbim_reset and sbim_load, which
