@@ -372,14 +372,14 @@ def cpu_workers():
     return max(1, os.cpu_count() or 1)
 
 
-def conv_roofline(pairs, alg_bytes, ms, kernel, traffic=None):
+def conv_roofline(pairs, alg_bytes, ms, kernel, blocked, traffic=None):
     """Roofline of a float-class convolution that took `ms` a step.  Step by step it is bound by the
     history's bytes; blocked in time (one pass over the history forms the sums of 16 steps) by the FP32
-    pipe: 10 real multiply-adds (20 flops) per (mode, lag) pair.  A step that beats the copy bandwidth
-    by 15 % on the step-by-step bytes has not read them all, so it ran blocked."""
+    pipe: 10 real multiply-adds (20 flops) per (mode, lag) pair.  `blocked` is the form the handles
+    report (sbim_get_time_blocks)."""
     peak, kind = peaks()
     hbm = alg_bytes / (ms * 1e-3) / 1e9
-    if hbm <= 1.15 * peak:
+    if not blocked:
         return {"bound": "hbm", "achieved": hbm, "peak": peak, "unit": "GB/s", "frac": hbm / peak,
                 "traffic": traffic, "kernel": kernel, "peak_kind": kind,
                 "algorithmic_bytes_per_launch": alg_bytes, "launch_ms": ms}
@@ -564,6 +564,7 @@ def run_native(args):
 
     # roofline of the convolution kernel (algorithmic bytes per launch)
     conv_ms = stage["convolution"] / nprof
+    blocked = g.time_blocks()
     bpp = BYTES_PER_PAIR[prec]
     alg_bytes = (pairs + modes) * bpp
     achieved = alg_bytes / (conv_ms * 1e-3) / 1e9
@@ -628,12 +629,13 @@ def run_native(args):
         "config": {"workload": workload_name(c, prec, args.kahan, adjoint), "n1": n1, "n3": n3,
                    "n_cut": n_cut, "precision": prec, "kahan": int(bool(args.kahan)),
                    "conv_variant": args.variant if args.variant >= 0 else DEFAULT_VARIANT[prec],
-                   "window": args.window, "mode_lag_pairs": pairs,
+                   "time_blocks": blocked, "window": args.window, "mode_lag_pairs": pairs,
                    "modes": modes, "history_bytes": hist_bytes,
                    "l2": "inputs larger than L2 (history ring buffer >> 129 MB)",
                    "parallelism": f"replicas x{world}"},
         "roofline": alu or conv_roofline(pairs, alg_bytes, conv_ms,
-                                         "conv_tma_kernel" if args.variant != 0 else "conv_kernel", traffic),
+                                         "conv_tma_kernel" if args.variant != 0 else "conv_kernel", blocked,
+                                         traffic),
         "stage_ms_per_step": {k: v / nprof for k, v in stage.items()},
         "hbm_gbs_step": alg_bytes / (ms_step * 1e-3) / 1e9,
         "cpu_baseline": cpu,
@@ -739,7 +741,8 @@ def run_coupled(args):
                    "elements": n1 * n2 * n3, "l2": "history (12.6 GB) >> L2"},
         "sbim_macs_per_s": macs / (ms * 1e-3),
         # the two half-spaces run side by side: the whole step, a lower bound
-        "roofline": conv_roofline(2 * modes * n_cut, alg, ms, "whole coupled step (FE stages included)"),
+        "roofline": conv_roofline(2 * modes * n_cut, alg, ms, "whole coupled step (FE stages included)",
+                                  B.sbim_get_time_blocks(top)),
         "stage_ms_per_step_top": {k: v / nprof for k, v in stage.items()},
         "fault": {"max_slip_m": float(slip.abs().max()), "max_slip_rate_m_s": float(rate.abs().max()),
                   "simulated_s": (n_cut + W + K) * dt},
@@ -808,7 +811,7 @@ def run_tpv3(args):
         if up is not None:
             stage, _ = B.sbim_stage_times(up)
             B.sbim_set_profiling(up, False)
-            conv = stage["convolution"] / K
+            conv = stage["convolution"] / K, B.sbim_get_time_blocks(up)
         out = (arrival.cpu().numpy(), mag.cpu().numpy(), e0.elapsed_time(e1) / K, clk.summary(), conv)
         g.close()
         return out
@@ -833,7 +836,8 @@ def run_tpv3(args):
                                f"(symmetry plane) vs hybrid with a 4-element slab",
                    "l2": "history >> L2"},
         "hybrid_ms_per_step": ms_h,
-        "roofline": conv_roofline(modes * steps, alg, conv_p, "conv_tma_kernel (the step's one history pass)"),
+        "roofline": conv_roofline(modes * steps, alg, conv_p[0], "conv_tma_kernel (the step's one history pass)",
+                                  conv_p[1]),
         "layout": {"modes": modes, "slots": slots, "padding": slots / modes},
         "agreement": {
             "ruptured_nodes": int(both.sum()), "ruptured_either": int(either.sum()),
@@ -902,7 +906,8 @@ def run_ensemble(args):
         tuned = None
         if args.tune:
             from paper_2102_08756_gb300.tune import autotune_hybrid_batch
-            tuned = autotune_hybrid_batch(b, stream)
+            tuned = autotune_hybrid_batch(b, stream, handles=[x for m in members
+                                                              for x in B.sbim_hybrid_info(m.h)[2:]])
         e0 = torch.cuda.Event(enable_timing=True)
         e1 = torch.cuda.Event(enable_timing=True)
         with ClockSampler(0) as clk:
@@ -915,6 +920,7 @@ def run_ensemble(args):
         ms = e0.elapsed_time(e1) / K
         macs = sum(2 * sc["n"] * (sc["n"] // 2 + 1) * sc["n_cut"] * MACS_PER_PAIR for sc in scen)
         peak_rate = max(float(x.fault_fields()[1].abs().max()) for x in members)
+        blocked = all(B.sbim_get_time_blocks(x) for m in members for x in B.sbim_hybrid_info(m.h)[2:])
         B.sbim_hybrid_batch_destroy(b)
         for x in members:
             x.close()
@@ -930,7 +936,7 @@ def run_ensemble(args):
         # the batched convolution runs inside the replayed graph, so only the
         # whole step is timed: a lower bound on the convolution's own rate
         "roofline": conv_roofline(macs // MACS_PER_PAIR, hist_bytes, ms,
-                                  "whole ensemble step (graph replay, FE stages included)"),
+                                  "whole ensemble step (graph replay, FE stages included)", blocked),
         "max_slip_rate_m_s": peak_rate, "clocks": clk.summary(),
     }
     if tuned is not None:
