@@ -72,7 +72,8 @@ typedef enum {
  *              -1: half-space x2 < boundary (S-)
  *   precision  an sbim_precision value
  *   kahan      non-zero: compensated (Kahan) float accumulation over the lags
- *              (ignored for SBIM_FP64)
+ *              (ignored for SBIM_FP64; block sums, see sbim_set_time_blocks, are
+ *              compensated either way)
  *   stream     cudaStream_t every call of this handle is ordered on; NULL = the
  *              legacy default stream
  * The kernel tables are built on the device in double precision.  Returns
@@ -153,8 +154,8 @@ int sbim_reset(sbim_handle h);
  * the two plane FFTs are recomputed: a predictor-corrector time stepper pays for
  * one history pass per step instead of two.  Needs a preceding sbim_step (or
  * sbim_step_repeat) on this handle with no sbim_step_adjoint, sbim_rewind,
- * sbim_reset, sbim_load, sbim_set_conv_config, sbim_set_window or batched step in
- * between (SBIM_ERR_STATE otherwise).  Arguments as sbim_step; stream-ordered.
+ * sbim_reset, sbim_load, sbim_set_conv_config, sbim_set_conv_tile, sbim_set_window,
+ * sbim_set_time_blocks or batched step in between (SBIM_ERR_STATE otherwise).  Arguments as sbim_step; stream-ordered.
  */
 int sbim_step_repeat(sbim_handle h, const void* u, const void* v, void* tau);
 
@@ -254,8 +255,9 @@ int sbim_set_check_finite(sbim_handle h, int enable);
  * sbim_set_profiling / sbim_stage_times -- per-stage device time.  While
  * profiling is on, every sbim_step records CUDA events on the handle's stream
  * around its stages; sbim_stage_times waits for them and returns the summed
- * milliseconds of (0) forward FFT, (1) history convolution, (2) reduction and
- * assembly, (3) inverse FFT, (4) traction epilogue, and the number of steps
+ * milliseconds of (0) forward FFT, (1) history convolution (with block sums, those
+ * that are due), (2) reduction and assembly (with block sums, the lags inside the block
+ * too), (3) inverse FFT, (4) traction epilogue, and the number of steps
  * summed (the stages of the spectral evaluation of Eq. (SBI), Section 2.3).
  * Enabling clears the sums.
  */
@@ -274,10 +276,16 @@ int sbim_stage_times(sbim_handle h, double ms[5], long long* steps);
  *                 prefetch, per-term compensated sums.  Default: 2 for float,
  *                 bf16 hi/lo and bf16 hi-only history, 1 for double (the
  *                 fastest shapes measured on GB300 at 1024^2 x 4096).
- *   lags_per_cta  lags one CTA convolves (0 = automatic: ~16 waves of resident CTAs)
- * Both variants compute the same sums to within float rounding.  May reallocate
- * the lag-chunk partial buffer (synchronising the stream); on failure the
- * previous configuration is kept.
+ *   lags_per_cta  lags one CTA convolves (0 = automatic: ~16 waves of resident CTAs
+ *                 step by step; whole waves of CTAs against the chunks' traffic for
+ *                 block sums, whose chunks are multiples of 16 lags)
+ * Variants 1 to 3 of a float-class handle with block sums (sbim_set_time_blocks) run one
+ * kernel, and only lags_per_cta changes its launch; the pipeline shapes are those of the
+ * step-by-step convolution.  All variants compute the same sums to within float rounding.
+ * May reallocate the lag-chunk partial buffer (synchronising the stream); on failure the
+ * previous configuration is kept.  A new chunking has the next step form all block sums
+ * again (as sbim_load and a new sbim_set_window do): that one step takes up to 2.7 times a
+ * step-by-step one.
  */
 int sbim_set_conv_config(sbim_handle h, int variant, int lags_per_cta);
 
@@ -310,7 +318,8 @@ int sbim_get_time_blocks(sbim_handle h, int* enabled);
  * sbim_set_conv_tile -- orbit records per CTA of the TMA-staged convolution
  * (variants 1-3; Section 2.3's per-mode convolution, one thread per record of 4
  * Fourier-bin members): 64, 128 (the default) or 256, i.e. 256, 512 or 1024
- * member slots ("modes") per CTA.  A shape's shared memory and threads per SM
+ * member slots ("modes") per CTA.  Block sums (sbim_set_time_blocks) do not depend on it.
+ * A shape's shared memory and threads per SM
  * stay the same (twice the resident CTAs at 64, half at 256).  SBIM_ERR_ARG
  * unless the handle's record count (n_slots / 4) is a multiple of it.  The
  * results equal the 128-record launch's to within float rounding.  May
@@ -401,10 +410,11 @@ typedef struct sbim_batch_ctx* sbim_batch;
  * compensation flag and one stream.  The members are handles the batch owns
  * (reachable through sbim_batch_member).  A batch step runs the FFTs and the
  * epilogue per member and the history convolution of ALL members in one launch
- * over their (member, orbit tile, lag chunk) work items; each item writes its
- * own partial sums, so results do not depend on the schedule.  The batch sets
- * its members' convolution launch (sbim_set_conv_config) to its own pipeline
- * shape and 1024 lags per item (the default of sbim_batch_set_conv_config).
+ * over their (member, orbit tile, lag chunk) work items (two, with block sums, where
+ * members of both record layouts meet); each item writes its own partial sums, so
+ * results do not depend on the schedule.  The batch sets its members' convolution
+ * launch (sbim_set_conv_config) to its own pipeline shape and 1024 lags per item (the
+ * default of sbim_batch_set_conv_config).
  */
 int sbim_batch_create(sbim_batch* out, int nb, const int* n1, const int* n3, const double* L1,
                       const double* L3, const double* cs, const double* cp, const double* rho,
@@ -434,7 +444,9 @@ int sbim_batch_replay(sbim_batch b);
  * lags per work item (0: 1024).  Default: one CTA per 1024-lag item with shape
  * 2 for float history, persistent shape 1 for bf16.  The results are the same
  * for every launch with the same lags per item (each item writes its own
- * partial sums).  Drops a captured graph: capture again before replaying.
+ * partial sums).  A batch whose members all take block sums (sbim_set_time_blocks) has
+ * one launch for them, and only lags_per_item, rounded up to a multiple of 16, changes it.
+ * Drops a captured graph: capture again before replaying.
  * Library utility (the launch of the Section 2.3 convolution): the paper has no
  * counterpart.
  */

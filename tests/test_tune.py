@@ -123,3 +123,35 @@ def test_chunkings_stop_below_the_history_length():
     u = torch.zeros(3, 32, 64)
     _, table = autotune(h, u, u, steps=1)
     assert sorted({r["lags_per_cta"] for r in table}) == [0, 256, 512]
+
+
+class BlockedHandle(FakeHandle):
+    """Takes block sums: one kernel, whose sums are partly added in the assembly."""
+
+    def __init__(self, times):
+        super().__init__(times)
+        self.timed = []
+
+    def time_blocks(self):
+        return True
+
+    def stage_times(self):
+        self.timed.append(self.prof_steps)
+        return ({"convolution": self.times[self.config] * self.prof_steps,
+                 "assemble": self.config[1] / 100.0 * self.prof_steps}, self.prof_steps)
+
+
+def test_block_sums_are_tuned_over_their_chunking_alone(tmp_path):
+    from paper_2102_08756_gb300.tune import autotune
+    cache = tmp_path / "c.json"
+    h = BlockedHandle({(2, 0): 9.0, (2, 256): 5.0, (2, 512): 4.0, (2, 1024): 3.0})
+    u = torch.zeros(3, 32, 64)
+    best, table = autotune(h, u, u, cache=str(cache))
+    # convolution + assembly: 9.0, 7.56, 9.12, 13.24
+    assert best["variant"] == 2 and best["lags_per_cta"] == 256 and abs(best["conv_ms"] - 7.56) < 1e-12
+    assert [(r["variant"], r["tile"]) for r in table] == [(2, 128)] * 4
+    assert set(h.timed) == {16}                     # whole blocks of steps
+    # the step-by-step handle of the same size has a result of its own
+    assert set(json.load(open(cache))) == {"64x32:1500:fp32:1:GB300-test:blocks"}
+    autotune(FakeHandle(_times()), u, u, cache=str(cache))
+    assert len(json.load(open(cache))) == 2
