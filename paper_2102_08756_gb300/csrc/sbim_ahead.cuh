@@ -29,9 +29,10 @@
 // of the block its sums belong to and of the arguments' chunking and window; sums
 // whose stamp is not the current one are formed again, all on the device, so that a
 // captured graph renews them as a direct step does.  sbim_reset and sbim_load, which
-// change the ring itself, mark every stamp invalid, and sbim_rewind those of blocks
-// that begin after the step it goes back to: a level before them may be written again,
-// and a block whose predecessor has no history in a chunk finds its old stamp there.
+// change the ring itself, mark every stamp invalid, and the second of two sbim_rewind
+// calls in a row those of blocks that begin after the step it goes back to: a level
+// before them may be written again, and a block whose predecessor has no history in a
+// chunk finds its old stamp there.
 #pragma once
 
 #include <type_traits>

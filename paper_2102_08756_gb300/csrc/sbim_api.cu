@@ -179,6 +179,7 @@ struct sbim_ctx {
   bool have_fwd = false, have_inv = false;
 
   long long n = 0;
+  int rewound = 0;            // rewinds since the last step
   bool can_repeat = false;    // the sums hold the last forward level,
   bool level_blocks = false;  // which took block sums
   double tau_inf[3] = {0, 0, 0};
@@ -194,6 +195,11 @@ struct sbim_ctx {
 namespace {
 
 sbim::StepArgs step_args(const sbim_ctx* c);
+
+void advanced(sbim_ctx* c) {
+  ++c->n;
+  c->rewound = 0;
+}
 
 // Integer weights (a, b) with L1 / L3 = a / b exactly, a and b coprime and
 // small, so that |k|^2 (L1 L3 / 2 pi)^2 = (j1 b)^2 + (j3 a)^2 is an exact integer
@@ -874,7 +880,7 @@ int handle_epilogue(sbim_handle c, const void* v, void* tau, cudaStream_t st) {
 }
 
 void handle_advance(sbim_handle c) {
-  ++c->n;
+  advanced(c);
   c->can_repeat = false;   // the batch kept its partial sums in its own buffers
 }
 
@@ -1064,7 +1070,7 @@ int run_step(sbim_ctx* c, const void* in, const void* aux, void* out, bool adjoi
     CU(cudaEventRecord(e[5], st));
     ++c->prof_issued;
   }
-  ++c->n;
+  advanced(c);
   c->can_repeat = !adjoint;
   return SBIM_OK;
 }
@@ -1124,7 +1130,7 @@ int handle_raw_step(sbim_handle c, const void* in, void* out, bool again, cudaSt
 const double* handle_far_field(sbim_handle c) { return c->tau_inf; }
 long long* handle_counter(sbim_handle c) { return c->d_step; }
 void handle_advanced(sbim_handle c) {
-  ++c->n;
+  advanced(c);
   c->can_repeat = true;
 }
 
@@ -1238,7 +1244,7 @@ int sbim_step_host(sbim_handle h, const void* u, const void* v, void* tau) {
     if (rc != SBIM_OK) return rc;
     rc = sbim::handle_epilogue(c, dv, dtau, st);
     if (rc != SBIM_OK) return rc;
-    ++c->n;
+    advanced(c);
     c->can_repeat = true;
   }
   // tau and the device error word come back under one synchronisation
@@ -1386,6 +1392,7 @@ int sbim_reset(sbim_handle h) {
   CU(cudaMemsetAsync(h->d_step, 0, sizeof(long long), h->stream));
   if (const int rc = forget_ahead(h, h->stream)) return rc;
   h->n = 0;
+  h->rewound = 0;
   h->can_repeat = false;
   return SBIM_OK;
 }
@@ -1393,9 +1400,11 @@ int sbim_reset(sbim_handle h) {
 int sbim_rewind(sbim_handle h) {
   if (!h) return fail(SBIM_ERR_ARG, "NULL handle");
   if (h->n == 0) return fail(SBIM_ERR_STATE, "no step to rewind");
-  CU(sbim::launch_rewind(h->d_step, h->stream, h->d_stamp,
+  // (one rewind rewrites the last level, and no sums were formed from it yet)
+  const bool several = ++h->rewound > 1;
+  CU(sbim::launch_rewind(h->d_step, h->stream, several ? h->d_stamp : nullptr,
                          (long long)(h->stamp_bytes / sizeof(long long))));
-  h->cold = true;
+  if (several) h->cold = true;
   --h->n;
   h->can_repeat = false;
   return SBIM_OK;
@@ -1480,6 +1489,7 @@ int sbim_load(sbim_handle h, const void* buf, size_t bytes) {
   if (const int rc = forget_ahead(h, h->stream)) return rc;
   CU(cudaStreamSynchronize(h->stream));
   h->n = hd.n;
+  h->rewound = 0;
   h->can_repeat = false;
   // the run goes on in the form it had (block sums only if there is room for them)
   if (hd.form == kFormSteps) h->blocks = 0;
