@@ -11,13 +11,12 @@
 // (near_kernel).  The history is read once per 16 steps and the work per step is
 // the same multiply-adds, now bound by the FP32 pipe (39-40 T multiply-adds/s
 // measured on GB300: 0.54 ms for 1024^2 x 4096 against 7.1 ms for the bytes).  The kernel
-// takes 1.17 ms there, ~160 ns per lag of a CTA against 77 on the pipe alone: 16 of a
-// warp's 35 instructions per lag are the two-lane multiply-adds and 4 the folds (ncu,
-// 512^2 x 1024), and the pipe is busy 61 % of the time.  A warp set aside for the
+// takes 1.11 ms there, ~155 ns per lag of a CTA against 77 on the pipe alone: 16 of a
+// warp's 33 instructions per lag are the two-lane multiply-adds and 2 the folds (ncu,
+// 512^2 x 1024), and the pipe is busy 59 % of the time.  A warp set aside for the
 // requests (spills: 21 warps leave 80 registers), the requests in turns behind an
 // mbarrier (+3 %), a skew of at most one (+15 %) or two stages (+1 %) between the warps,
-// weights loaded into both halves of a register pair (same) and a stage released before
-// its fold (+3 to 5 %) were measured and not kept.
+// and weights loaded into both halves of a register pair (same) were measured and not kept.
 //
 // Blocks are aligned and staggered: tile T (128 records) starts its blocks at the
 // steps with (n + T) mod 16 = 0, so every step of a plane of 16 and more tiles renews
@@ -56,6 +55,7 @@ using namespace dev;
 constexpr int kRec = kAheadRec, kSums = 5, kThreads = kRec * kMembers * kSums, kWarps = kThreads / 32;
 constexpr int kSub = kOrbitTile / kRec;     // CTAs per 128-record tile
 constexpr int kLags = kAheadLags;   // lags per stage
+constexpr int kFoldAll = 97;        // first lag of the longer chains
 template <bool HALVES> __host__ __device__ constexpr int stages() { return HALVES ? 4 : 5; }
 
 template <class S> __host__ __device__ constexpr int seg() { return kRec * S::kRecBytes; }
@@ -239,15 +239,16 @@ __device__ __forceinline__ void request_stage(const StepArgs& a, int j, unsigned
 }
 
 // A warp's part of an item: one of the five sums for the 32 members of 8 records.
-// The terms of 16 lags are chained by multiply-adds, then folded into the running
-// sums (in shared memory) with one compensated addition, half of the outputs after
-// each stage.  With chains of 32 lags the error against 64 bits was up to 0.6 % above
-// that of the step-by-step convolution (compensated every 2 lags); with 16, and the
-// stored weights for the lags inside a block too, it is 0.99 of it for FP32 on average
-// and equal for BF16 hi/lo.  Folds of 8 lags gain nothing more and cost 18 % at
-// 512^2 x 2000; these cost 4 % (208 to 215 us a step), 8 % with all outputs folded at
-// once.  The warps meet only at the stages: each waits for its copies, and the last to
-// leave one requests its next filling.  Returns false if a bounded wait gave up.
+// The terms of 16 lags (32 from lag kFoldAll on) are chained by multiply-adds, then
+// folded into the running sums (in shared memory) with one compensated addition.  With
+// chains of 32 lags throughout, and float weights inside the block, the error against 64
+// bits was up to 0.6 % above that of the step-by-step convolution (compensated every 2
+// lags); with 16 for the lags that carry the largest weights, and the stored weights
+// inside the block, it is 0.99 of it for FP32 on average and equal for BF16 hi/lo (36
+// sizes, spectra and precisions).  Chains of 16 throughout gain 0.1 % more and cost 4 %
+// of a step (512^2 x 2000: 206 against 215 us), of 8 lags 18 %.  The warps meet only at
+// the stages: each waits for its copies, and the last to leave one requests its next
+// filling.  Returns false if a bounded wait gave up.
 template <class S, bool HALVES>
 __device__ __forceinline__ bool sum_item(const StepArgs& a, int q, unsigned char* smem, Sync& sync,
                                          unsigned g) {
@@ -311,14 +312,6 @@ __device__ __forceinline__ bool sum_item(const StepArgs& a, int q, unsigned char
         w[l] = pack2(make_float2(v, v));
       }
       __syncwarp();
-#pragma unroll
-      for (int s = L0; s < L0 + kLags; s += 2) {
-        const ulonglong2 o = run[(s / 2) * kThreads];
-        const ulonglong2 t = make_ulonglong2(add2r(o.x, y[s]), add2r(o.y, y[s + 1]));
-        y[s] = sub2r(y[s], sub2r(t.x, o.x));     // minus the compensation
-        y[s + 1] = sub2r(y[s + 1], sub2r(t.y, o.y));
-        run[(s / 2) * kThreads] = t;
-      }
       if (lane == 0) {
         const int j = 2 * b + L0 / kLags;
         if (shared_inc(&sync.left[buf]) % kWarps == kWarps - 1 && j + NS < 2 * nblk) {
@@ -342,6 +335,16 @@ __device__ __forceinline__ bool sum_item(const StepArgs& a, int q, unsigned char
     else
       block(std::false_type{}, std::false_type{});
     if (!ok) return false;
+    if (b % 2 || mb < kFoldAll) {
+#pragma unroll
+      for (int s = 0; s < kAhead; s += 2) {
+        const ulonglong2 o = run[(s / 2) * kThreads];
+        const ulonglong2 t = make_ulonglong2(add2r(o.x, y[s]), add2r(o.y, y[s + 1]));
+        y[s] = sub2r(y[s], sub2r(t.x, o.x));     // minus the compensation
+        y[s + 1] = sub2r(y[s + 1], sub2r(t.y, o.y));
+        run[(s / 2) * kThreads] = t;
+      }
+    }
   }
   float* out = a.ahead + (((long long)it.chunk * (a.n_orb_pad / kOrbitTile) + it.T) * kAhead * kFields + 2 * f) *
                              (kOrbitTile * kMembers) + q * (kRec * kMembers) + x;
