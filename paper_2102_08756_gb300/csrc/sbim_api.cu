@@ -124,9 +124,9 @@ struct sbim_ctx {
   int blocks = -1;
   bool blocks_off = false;    // the caller wants no block sums
   int ahead_lc = sbim::kAhead, ahead_chunks = 1;
-  // One allocation of its own, made at the first step: ring map, weights, stamps, sums.
-  void* d_extra = nullptr;
   void* d_tmap = nullptr;     // CUtensorMap of the ring
+  // One allocation of its own, made at the first step: weights, stamps, sums.
+  void* d_extra = nullptr;
   void* d_wts32 = nullptr;    // the block sums' weights
   long long* d_stamp = nullptr;
   size_t stamp_bytes = 0;
@@ -470,7 +470,7 @@ size_t ahead_need(const sbim_ctx& c) {
 // Marks every block sum as not formed.
 int forget_ahead(sbim_ctx* c, cudaStream_t st) {
   if (c->d_stamp) CU(cudaMemsetAsync(c->d_stamp, 0xff, c->stamp_bytes, st));
-  c->cold = true;
+  c->cold = c->n > 0;
   return SBIM_OK;
 }
 
@@ -543,28 +543,20 @@ int start_blocks(sbim_ctx* c, cudaStream_t st, bool* ok) {
     // the chunking changes, so that a batch's own copy of the arguments stays consistent
     const size_t stamps = (size_t)((c->n_cut + sbim::kAhead - 1) / sbim::kAhead) *
                           (c->n_orb_pad / sbim::kAheadRec) * sizeof(long long);
-    const size_t o_stamp = 256 + w32, o_sums = o_stamp + (stamps + 255) / 256 * 256;
+    const size_t o_stamp = w32, o_sums = o_stamp + (stamps + 255) / 256 * 256;
     bool room;
     if (const int rc = have_room(*c, o_sums + sums, &room)) return rc;
     if (!room) return SBIM_OK;
-    if (!c->sums.side) CU(sbim::pair_init(c->sums));
-    CU(sbim::launch_ahead(sbim::StepArgs{}, c->prec, 0, c->halves, st));
-    CUtensorMap map;
-    std::memset(&map, 0, sizeof map);
-    if (c->n_cut >= sbim::kAheadLags)   // shorter rings always wrap: copied row by row
-      if (const int rc = make_ring_map(*c, &map)) return rc;
     if (cudaMalloc(&c->d_extra, o_sums + sums) != cudaSuccess) {
       c->d_extra = nullptr;
       cudaGetLastError();
       return SBIM_OK;
     }
-    c->d_tmap = c->d_extra;
-    c->d_wts32 = (char*)c->d_extra + 256;
+    c->d_wts32 = c->d_extra;
     c->d_stamp = (long long*)((char*)c->d_extra + o_stamp);
     c->stamp_bytes = stamps;
     c->d_ahead = (float*)((char*)c->d_extra + o_sums);
     c->ahead_bytes = sums;
-    CU(cudaMemcpyAsync(c->d_tmap, &map, sizeof map, cudaMemcpyHostToDevice, st));
     CU(sbim::launch_ahead(step_args(c), c->prec, 3, c->halves, st));
   } else if (sums > c->ahead_bytes) {
     bool room;
@@ -606,7 +598,7 @@ int drop_blocks(sbim_ctx* c) {
   CU(cudaFree(c->d_ahead_own));
   c->d_ahead_own = nullptr;
   CU(cudaFree(c->d_extra));
-  c->d_extra = c->d_tmap = c->d_wts32 = nullptr;
+  c->d_extra = c->d_wts32 = nullptr;
   c->d_stamp = nullptr;
   c->d_ahead = nullptr;
   c->stamp_bytes = c->ahead_bytes = 0;
@@ -736,6 +728,7 @@ int create_impl(sbim_ctx* c) {
   const size_t o_muq = put(&c->d_muq, o2 * c->real_size);
   const size_t o_us = put((void**)&c->d_ustep, o2 * sizeof(unsigned long long));
   const size_t o_gl = put((void**)&c->d_gl, 32 * sizeof(double));
+  const size_t o_map = put(&c->d_tmap, sizeof(CUtensorMap));
   put((void**)&c->d_step, sizeof(long long));   // zero, like the error word
   put((void**)&c->d_err, sizeof(int));
   const size_t filled = at;
@@ -768,11 +761,20 @@ int create_impl(sbim_ctx* c) {
   }
   std::memcpy(&host[o_us], ustep.data(), o2 * sizeof(unsigned long long));
   gauss_legendre16((double*)&host[o_gl], (double*)&host[o_gl] + 16);
+  if (!dbl && c->n_cut >= sbim::kAheadLags) {   // shorter rings always wrap: copied row by row
+    CUtensorMap map;
+    if (const int rc = make_ring_map(*c, &map)) return rc;
+    std::memcpy(&host[o_map], &map, sizeof map);
+  }
   cudaStream_t st = c->stream;
   CU(cudaMemcpyAsync(c->d_arena, host.data(), filled, cudaMemcpyHostToDevice, st));
   CU(sbim::launch_table_build(c->d_tab64, c->d_tab32, c->tab_n, c->tab_h, c->eta, c->d_gl,
                               c->d_gl + 16, st));
   if (c->d_wts) CU(sbim::launch_weights64(step_args(c), c->d_wts, st));
+  if (!dbl) {   // what block sums need besides memory, while the table is built
+    CU(sbim::pair_init(c->sums));
+    CU(sbim::launch_ahead(step_args(c), c->prec, 0, c->halves, st));
+  }
   if (const int rc = configure_conv(*c)) return rc == SBIM_ERR_CUDA ? rc : SBIM_ERR_OOM;
   CU(cudaStreamSynchronize(st));
 
