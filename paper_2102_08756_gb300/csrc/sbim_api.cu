@@ -437,11 +437,13 @@ int alloc_partials(sbim_ctx& c) {
 
 // Lag chunks of the block sums.  One chunk is groups x 4 CTAs of 32 records (one
 // tile in 16 is due at a step), one CTA per SM; a CTA takes ~155 ns per lag (1.11 ms
-// for 7 waves of 1024 lags at 1024^2 x 4096) and ~50 lags' worth to start and end, and
+// for 7 waves of 1024 lags at 1024^2 x 4096) and ~40 lags' worth to start and end, and
 // every chunk adds partial sums that are written and read once (2 x 160 B per record
-// and step).  The count that minimises the sum of both keeps the last wave full on
-// small grids and few chunks on large ones (4 at 1024^2 x 4096, where 8 take 3 % and 2
-// take 11 % more; 4 at 1024^2 x 2048: 0.68 ms a step, 0.73 with 1).
+// and step, at ~4.2 TB/s).  The count that minimises the sum of both keeps the last wave
+// full on small grids and few chunks on large ones.  us a step, chosen chunk lags first:
+// 256^2 x 100, 16 / 32 / 48 lags 41.2 / 41.3 / 43.7; 512^2 x 32, 32 / 16 53.6 / 56.4;
+// 384^2 x 2000, 288 / 672 139 / 149; 720^2 x 4096, 512 / 4096 647 / 687; 1024^2 x 2048,
+// 512 / 2048 679 / 726 (1024^2 x 4096, 1024: 8 chunks take 3 % more, 2 take 11 %).
 void choose_ahead(sbim_ctx& c, int sms) {
   const int lags = std::max(1, c.n_cut - 1);
   auto round16 = [](int x) { return (x + sbim::kAhead - 1) / sbim::kAhead * sbim::kAhead; };
@@ -453,7 +455,7 @@ void choose_ahead(sbim_ctx& c, int sms) {
     for (int S = 1; S <= std::min(32, round16(lags) / sbim::kAhead); ++S) {
       const int lc = round16((lags + S - 1) / S);
       const double waves = std::ceil(ctas * ((lags + lc - 1) / lc) / sms);
-      const double ns = waves * (lc + 50) * 155.0 + S * (double)c.n_orb_pad * 320.0 / 6000.0;
+      const double ns = waves * (lc + 40) * 155.0 + S * (double)c.n_orb_pad * 320.0 / 4200.0;
       if (S == 1 || ns < best) {
         best = ns;
         c.ahead_lc = lc;
