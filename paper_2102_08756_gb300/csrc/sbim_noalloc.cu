@@ -78,18 +78,21 @@ struct BinGeom {
 // convolution needs these (one per bin and lag chunk), and GB300 has two FP64
 // multiply-adds per SM and clock: the library's square root and the quotients of the
 // bin's whole geometry, formed here for every chunk, took most of the kernel (188 us
-// for 256 x 256 x 500 lags, 141 without).  One Newton step from the float reciprocal
-// root (relative error 1.5 e^2, e ~ 1e-7) gives |k| to ~2e-14, and one step of Heron's
-// method with the residual s - q^2 in one rounding makes it a double's.
+// for 256 x 256 x 500 lags, 141 without).  Two steps of Heron's method, q += (s - q^2)
+// r / 2 with the float reciprocal root r and the residual in one rounding, take s r from
+// 1e-7 to 2e-14 and to a double's precision.
 __device__ __forceinline__ double bin_dT(const NAArgs& a, int b) {
   const int j1 = b % a.nh, r3 = b / a.nh;
   const int j3 = r3 <= a.n3 / 2 ? r3 : r3 - a.n3;
   const double k1 = a.d1 * j1, k3 = a.d3 * j3;
   const double s = k1 * k1 + k3 * k3;
   if (!(s > 1e-30 && s < 1e30)) return sqrt(s) * a.cs_dt;   // k = 0, and past a float's range
-  const double r = rsqrtf((float)s);
-  const double q = s * (r * (1.5 - 0.5 * s * r * r));
-  return fma(fma(-q, q, s), 0.5 * r, q) * a.cs_dt;
+  const float rf = rsqrtf((float)s);
+  const double h = 0.5f * rf;
+  double q = s * rf;
+  q = fma(fma(-q, q, s), h, q);
+  q = fma(fma(-q, q, s), h, q);
+  return q * a.cs_dt;
 }
 
 __device__ BinGeom bin_geom(const NAArgs& a, int b) {
